@@ -34,8 +34,9 @@
  *     than 2, 3 and 5; otherwise EVX_ERR_SIZE. Every such size runs the same
  *     arithmetic. Each pass picks its kernel by its own length: nx, ny in
  *     {64, ..., 1024 powers of two, 400} and nz in {128, ..., 1024 powers of
- *     two, 400} take the tuned four-step kernels; other lengths take the
- *     mixed-radix ones (same results to FP32 rounding, several times slower).
+ *     two, 400} take the tuned four-step kernels, other lengths the two-radix
+ *     kernels, and nx, ny = 972 and 1000 the mixed-radix ones (same results to
+ *     FP32 rounding, several times slower).
  */
 #ifndef EVX_H
 #define EVX_H

@@ -352,6 +352,125 @@ struct Dft<20, DIR> {
     }
 };
 
+// cos and sin of 2 pi m / n, evaluated by the compiler: range reduction to
+// [0, pi/4] by the octant symmetries, then the Taylor series to double precision
+struct Root {
+    double c, s;
+};
+__host__ __device__ constexpr Root root_of_unity(int m, int n) {
+    m %= n;
+    if (m < 0) m += n;
+    int o = 8 * m / n;  // octant: 2 pi m / n = o pi / 4 + rest
+    double num = 8.0 * m - (double)o * n;
+    if (o & 1) num = n - num;  // odd octants from the other side
+    const double x = num / n * 0.78539816339744830962, x2 = x * x;
+    double c = 0.0, s = 0.0, tc = 1.0, ts = x;
+    for (int k = 0; k < 12; ++k) {
+        c += tc;
+        s += ts;
+        tc *= -x2 / ((2 * k + 1) * (2 * k + 2));
+        ts *= -x2 / ((2 * k + 2) * (2 * k + 3));
+    }
+    switch (o) {
+        case 0: return Root{c, s};
+        case 1: return Root{s, c};
+        case 2: return Root{-s, c};
+        case 3: return Root{-c, s};
+        case 4: return Root{-c, -s};
+        case 5: return Root{-s, -c};
+        case 6: return Root{s, -c};
+        default: return Root{c, -s};
+    }
+}
+// a exp(DIR 2 pi i m / n) for fixed m, n
+template <int DIR, int m, int n>
+__device__ __forceinline__ float2 wroot(float2 a) {
+    constexpr Root r = root_of_unity(m, n);
+    constexpr float c = (float)r.c, s = (float)(DIR < 0 ? -r.s : r.s);
+    if (m % n == 0) return a;
+    return make_float2(fmaf(a.x, c, -a.y * s), fmaf(a.x, s, a.y * c));
+}
+
+// length N1 N2 with coprime factors (Good-Thomas): no twiddles. Input
+// n = (N2 n1 + N1 n2) mod N, output k = k1 mod N1, k = k2 mod N2.
+__host__ __device__ constexpr int crt_index(int k1, int N1, int k2, int N2) {
+    for (int k = 0; k < N1 * N2; ++k)
+        if (k % N1 == k1 && k % N2 == k2) return k;
+    return 0;
+}
+template <int N1, int N2, int DIR>
+struct DftCoprime {
+    template <int K1, int K2>
+    __device__ __forceinline__ static void put(float2* v, const float2 (&t)[N1][N2]) {
+        constexpr int k = crt_index(K1, N1, K2, N2);
+        v[k] = t[K1][K2];
+        if constexpr (K2 + 1 < N2)
+            put<K1, K2 + 1>(v, t);
+        else if constexpr (K1 + 1 < N1)
+            put<K1 + 1, 0>(v, t);
+    }
+    __device__ __forceinline__ static void run(float2* v) {
+        constexpr int N = N1 * N2;
+        float2 t[N1][N2];
+#pragma unroll
+        for (int n1 = 0; n1 < N1; ++n1) {
+#pragma unroll
+            for (int n2 = 0; n2 < N2; ++n2) t[n1][n2] = v[(N2 * n1 + N1 * n2) % N];
+            Dft<N2, DIR>::run(t[n1]);
+        }
+#pragma unroll
+        for (int k2 = 0; k2 < N2; ++k2) {
+            float2 u[N1];
+#pragma unroll
+            for (int n1 = 0; n1 < N1; ++n1) u[n1] = t[n1][k2];
+            Dft<N1, DIR>::run(u);
+#pragma unroll
+            for (int k1 = 0; k1 < N1; ++k1) t[k1][k2] = u[k1];
+        }
+        put<0, 0>(v, t);
+    }
+};
+// length N1 N2, decimation in time: n = N2 n1 + n2, k = k1 + N1 k2
+template <int N1, int N2, int DIR>
+struct DftTwiddled {
+    template <int n2, int k1>
+    __device__ __forceinline__ static void twiddle(float2 (&t)[N2][N1]) {
+        t[n2][k1] = wroot<DIR, n2 * k1, N1 * N2>(t[n2][k1]);
+        if constexpr (k1 + 1 < N1)
+            twiddle<n2, k1 + 1>(t);
+        else if constexpr (n2 + 1 < N2)
+            twiddle<n2 + 1, 1>(t);
+    }
+    __device__ __forceinline__ static void run(float2* v) {
+        float2 t[N2][N1];
+#pragma unroll
+        for (int n2 = 0; n2 < N2; ++n2) {
+#pragma unroll
+            for (int n1 = 0; n1 < N1; ++n1) t[n2][n1] = v[N2 * n1 + n2];
+            Dft<N1, DIR>::run(t[n2]);
+        }
+        twiddle<1, 1>(t);
+#pragma unroll
+        for (int k1 = 0; k1 < N1; ++k1) {
+            float2 u[N2];
+#pragma unroll
+            for (int n2 = 0; n2 < N2; ++n2) u[n2] = t[n2][k1];
+            Dft<N2, DIR>::run(u);
+#pragma unroll
+            for (int k2 = 0; k2 < N2; ++k2) v[k1 + N1 * k2] = u[k2];
+        }
+    }
+};
+template <int DIR> struct Dft<6, DIR> : DftCoprime<2, 3, DIR> {};
+template <int DIR> struct Dft<9, DIR> : DftTwiddled<3, 3, DIR> {};
+template <int DIR> struct Dft<12, DIR> : DftCoprime<4, 3, DIR> {};
+template <int DIR> struct Dft<15, DIR> : DftCoprime<3, 5, DIR> {};
+template <int DIR> struct Dft<18, DIR> : DftCoprime<2, 9, DIR> {};
+template <int DIR> struct Dft<24, DIR> : DftCoprime<8, 3, DIR> {};
+template <int DIR> struct Dft<25, DIR> : DftTwiddled<5, 5, DIR> {};
+template <int DIR> struct Dft<27, DIR> : DftTwiddled<3, 9, DIR> {};
+template <int DIR> struct Dft<30, DIR> : DftCoprime<2, 15, DIR> {};
+
 // Tile descriptor: pencil p, element i at buf[i*es + p*ps].
 struct Tile {
     float2* buf;

@@ -146,6 +146,7 @@ struct ZPassArgs {
     Plan plan;
     const float2* tw;       // M-entry table exp(-2 pi i m / M)
     const float2* rtw;      // (M + 1)-entry table exp(-2 pi i k / nz)
+    const float2* twA;      // M = R1 R2: w_M^{n2 k1} as [k1][n2], then as [n2][k1] (2 M entries), or null
     float scale;            // 1 / (ny nz)
     const double* cbar;     // FP64 mean (Z_STEP, Z_C2R); may be null (0)
     double* partials;       // bulk energy partial per CTA (Z_C2R) or null
@@ -231,6 +232,12 @@ bool fast_zstep(const ZPassArgs& a, cudaStream_t st, cudaError_t* err, int* grid
 bool fast_xadj(const XAdjArgs& a, cudaStream_t st, cudaError_t* err);
 bool fast_zconv(const ZPassArgs& a, int dir, cudaStream_t st, cudaError_t* err, int* grid_used);
 bool fast_paths_enabled();  // false when the environment sets EVX_GENERIC=1
+// two-radix passes for lengths R1 R2, R1, R2 <= 32 (evx_mixed.cu); false if not applicable
+bool mixed_split(int L, int* R1, int* R2);
+bool mixed_spass(const SPassArgs& a, int dir, cudaStream_t st, cudaError_t* err);
+bool mixed_xupdate(const XUpdArgs& a, cudaStream_t st, cudaError_t* err);
+bool mixed_zpass(const ZPassArgs& a, int mode, cudaStream_t st, cudaError_t* err, int* grid_used);
+int mixed_zgrid(const ZPassArgs& a);  // CTAs (partials) of a two-radix z pass, 0 if there is none
 // reads (and optionally clears) the flag a bounded TMA wait sets when it gives up
 bool fast_timeout_flag(int* flag, bool clear);
 

@@ -1,0 +1,131 @@
+// Two-radix passes for every other 2/3/5-smooth length L = R1 R2 (R1, R2 <= 32):
+// the y pass, the x pass with the k-space update, the z passes.
+//
+// Four-step FFT of a length-L pencil, n = n2 + R2 n1, k = k1 + R1 k2:
+//   pass A: item n2 (R2 of them): DFT-R1 over n1 in registers, times w_L^{n2 k1}
+//   pass B: item k1 (R1 of them): DFT-R2 over n2 in registers
+// One shared-memory exchange between the two, and none elsewhere: pass A of the
+// y and x passes reads its R1 values straight from global memory (8 adjacent
+// columns = 64-byte rows, R1 independent loads in flight per thread) and the
+// last pass writes straight back. The radices are compile-time (register DFTs),
+// which ones a launch uses is a uniform switch, so a handful of kernels serve
+// all lengths; a stage-by-stage Stockham kernel pays one exchange, two barriers
+// and the index divisions per radix (evx_kernels.cu, kept for lengths that are
+// no product of two radices up to 32: 972 and 1000).
+//
+// The exchange keeps item k1's R2 values in a row of R2p = R2 | 1 slots: pass A
+// writes neighbouring slots, pass B reads an odd distance apart, both without
+// bank conflicts. Every thread rewrites only the slots it has read, so an
+// inverse walks back through the same slots with one barrier per exchange.
+//
+// Measured on a GB300 against the stage-by-stage kernels, 300 x 240 x 200: y pass
+// 137 -> 21 us (5.5 TB/s), z pass 237 -> 61 us, x pass 620 -> 74 us; 48 x 40 x 36:
+// y 10.9 -> 3.6, z 56 -> 8, x 26 -> 8 us. The y pass is bound by memory, the z and
+// x passes by instruction issue and their barriers.
+#pragma once
+#include <algorithm>
+#include <cstdint>
+
+#include "evx_internal.h"
+
+namespace evx {
+namespace mixed {
+
+// ------------------------------------------------------------------ radices
+#define EVX_MX_SMALL(F) F(1) F(2) F(3) F(4) F(5) F(6) F(8) F(9) F(10) F(12) F(15) F(16)
+#define EVX_MX_LARGE(F) F(18) F(20) F(24) F(25) F(27) F(30) F(32)
+
+// f.template run<R>() for the radix r; BIG: radices above 16 are compiled in
+template <bool BIG, typename Fn>
+__device__ __forceinline__ void with_radix(int r, Fn&& f) {
+    switch (r) {
+#define EVX_MX_CASE(R) \
+    case R: f.template run<R>(); return;
+        EVX_MX_SMALL(EVX_MX_CASE)
+#undef EVX_MX_CASE
+        default: break;
+    }
+    if constexpr (BIG) {
+        switch (r) {
+#define EVX_MX_CASE(R) \
+    case R: f.template run<R>(); return;
+            EVX_MX_LARGE(EVX_MX_CASE)
+#undef EVX_MX_CASE
+            default: break;
+        }
+    }
+}
+
+template <int DIR>
+__device__ __forceinline__ float2 twmul(float2 v, float2 w) {
+    if (DIR > 0) w.y = -w.y;
+    return cmul(v, w);
+}
+
+// ------------------------------------------- column tiles (x and y passes)
+// A CTA holds SP = 8 adjacent columns; thread = (p, it), p = column, items it,
+// it + T, ... Slot of (k1, n2): (k1 R2p + n2) 8 + p.
+constexpr int CP = SP;
+
+// pass A from global: v[n1] = src[n1 stride], DFT-R1, twiddle, into column n2 of the exchange
+template <int DIR>
+struct ColLoad {
+    const float2* src;
+    long long stride;
+    float2* x;  // exchange, at column p and n2
+    int pitch;  // R2p * 8
+    const float2* tw;
+    int n2;
+    template <int R>
+    __device__ __forceinline__ void run() const {
+        float2 v[R];
+#pragma unroll
+        for (int i = 0; i < R; ++i) v[i] = src[i * stride];
+        Dft<R, DIR>::run(v);
+        x[0] = v[0];
+#pragma unroll
+        for (int k = 1; k < R; ++k) x[k * pitch] = twmul<DIR>(v[k], __ldg(tw + n2 * k));
+    }
+};
+// pass B to global: v[n2] from row k1 of the exchange, DFT-R2, dst[k2 stride]
+template <int DIR>
+struct ColStore {
+    float2* dst;
+    long long stride;
+    const float2* x;  // exchange, at column p and row k1
+    template <int R>
+    __device__ __forceinline__ void run() const {
+        float2 v[R];
+#pragma unroll
+        for (int i = 0; i < R; ++i) v[i] = x[i * CP];
+        Dft<R, DIR>::run(v);
+#pragma unroll
+        for (int k = 0; k < R; ++k) dst[k * stride] = v[k];
+    }
+};
+// last pass of an inverse, to global: v[k1] from column n2, DFT-R1, dst[n1 stride]
+struct ColStoreInv {
+    float2* dst;
+    long long stride;
+    const float2* x;  // exchange, at column p and n2
+    int pitch;
+    template <int R>
+    __device__ __forceinline__ void run() const {
+        float2 v[R];
+#pragma unroll
+        for (int k = 0; k < R; ++k) v[k] = x[k * pitch];
+        Dft<R, 1>::run(v);
+#pragma unroll
+        for (int i = 0; i < R; ++i) dst[i * stride] = v[i];
+    }
+};
+
+}  // namespace mixed
+
+template <typename K>
+static cudaError_t mx_smem(K kernel, size_t bytes) {
+    if (bytes <= 48 * 1024) return cudaSuccess;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+}  // namespace evx

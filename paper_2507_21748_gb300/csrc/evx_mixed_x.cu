@@ -1,0 +1,131 @@
+// Two-radix x pass with the k-space update (see evx_mixed.cuh).
+#include "evx_mixed.cuh"
+
+namespace evx {
+namespace mixed {
+
+// middle of the x pass: forward pass B of W and S, the update, inverse pass B;
+// row k1 of the exchanges (column p). MODE as in XUpdArgs.model, 0 also for 1.
+// SPILL: F_x W is put back into its own slots instead of being held in registers.
+template <int MODE, bool SPILL>
+struct ColUpdate {
+    const XUpdArgs& a;
+    float2* w;
+    float2* s;
+    const float* k2x;  // + k1
+    int R1, k1;
+    float k2yz, gpb;
+    bool zero;  // row holds the k = 0 mode at k2 = 0
+    __device__ __forceinline__ void blk(float k2, float Dinv, float& P, float& S) const {
+        // P = L^n, S = sum_{j<n} L^j by binary powers: P_{2m} = P_m^2, S_{2m} = S_m (1 + P_m)
+        const float Lk = fmaf(-a.dtM * k2, gpb, 1.f) * Dinv;
+        P = 1.f, S = 0.f;
+        for (int b = 31 - __clz(a.nblk); b >= 0; --b) {
+            S = fmaf(S, P, S);
+            P *= P;
+            if ((a.nblk >> b) & 1) {
+                S = fmaf(S, Lk, 1.f);
+                P *= Lk;
+            }
+        }
+    }
+    template <int R>
+    __device__ __forceinline__ void run() const {
+        const bool ac = a.model == 1;
+        float2 g[R];
+#pragma unroll
+        for (int i = 0; i < R; ++i) g[i] = w[i * CP];
+        Dft<R, -1>::run(g);
+        float2 v[R];
+        if (MODE == 2) {  // preconditioner: dt / (1 + dt M kappa |k|^4) F_x W / L (dtM holds dt)
+#pragma unroll
+            for (int k = 0; k < R; ++k) {
+                const float k2 = __ldg(k2x + R1 * k) + k2yz;
+                v[k] = cscale(g[k], a.dtM * (a.invL / fmaf(a.dtMk, k2 * k2, 1.f)));
+            }
+        } else {
+            if (SPILL) {
+#pragma unroll
+                for (int i = 0; i < R; ++i) w[i * CP] = g[i];
+            }
+#pragma unroll
+            for (int i = 0; i < R; ++i) v[i] = s[i * CP];
+            Dft<R, -1>::run(v);
+#pragma unroll
+            for (int k = 0; k < R; ++k) {
+                const float2 gk = SPILL ? w[k * CP] : g[k];
+                const float k2 = __ldg(k2x + R1 * k) + k2yz;
+                if (MODE == 3) {
+                    const float Dinv = 1.f / fmaf(a.dtMk, k2 * k2, 1.f);
+                    float P, S;
+                    blk(k2, Dinv, P, S);
+                    const float bs = -a.dtM * k2 * Dinv * S * a.invL, as = P * a.invL;
+                    v[k] = make_float2(fmaf(bs, gk.x, as * v[k].x), fmaf(bs, gk.y, as * v[k].y));
+                } else {  // (c_hat - dt M |k|^2 g_hat) / (1 + dt M kappa |k|^4); Allen-Cahn: 1 and |k|^2
+                    const float f = a.invL / fmaf(a.dtMk, ac ? k2 : k2 * k2, 1.f);
+                    const float b = -a.dtM * (ac ? 1.f : k2);
+                    v[k] = make_float2(f * fmaf(b, gk.x, v[k].x), f * fmaf(b, gk.y, v[k].y));
+                }
+            }
+        }
+        if (zero) v[0] = make_float2(0.f, 0.f);  // the mean is carried in FP64
+        Dft<R, 1>::run(v);
+        s[0] = v[0];
+#pragma unroll
+        for (int i = 1; i < R; ++i) s[i * CP] = twmul<1>(v[i], __ldg(a.tw + i * k1));
+    }
+};
+
+// BIG1 / BIG2: radices above 16 for R1 / R2
+template <int MODE, bool BIG1, bool BIG2>
+__global__ void __launch_bounds__(BIG1 ? 256 : 128, BIG1 ? 2 : 5) mx_x_kernel(XUpdArgs a, int R1, int R2) {
+    extern __shared__ float4 smem4[];
+    const int p = threadIdx.x & 7, it = threadIdx.x >> 3, T = blockDim.x >> 3;
+    const int R2p = R2 | 1, pitch = R2p * CP;
+    float2* xw = reinterpret_cast<float2*>(smem4);
+    float2* xs = MODE == 2 ? xw : xw + R1 * pitch;
+    const int ky = blockIdx.y, kz = (int)blockIdx.x * CP + p;
+    const bool valid = kz < a.ncols;
+    const long long base = split_off(ky, a.YB, a.os, a.os2) + kz;
+    if (valid)
+        for (int i = it; i < (MODE == 2 ? R2 : 2 * R2); i += T) {
+            const bool second = i >= R2;
+            const int n2 = second ? i - R2 : i;
+            with_radix<BIG1>(R1, ColLoad<-1>{(second ? a.S : a.W) + base + n2 * a.rs, R2 * a.rs,
+                                             (second ? xs : xw) + n2 * CP + p, pitch, a.tw, n2});
+        }
+    __syncthreads();
+    if (valid) {
+        const float k2yz = a.k2y[ky] + a.k2z[kz];
+        const float gpb = MODE == 3 ? (float)(3.0 * (*a.cbar) * (*a.cbar) - 1.0) : 0.f;
+        for (int k1 = it; k1 < R1; k1 += T)
+            with_radix<BIG2>(R2, ColUpdate<MODE, BIG2>{a, xw + k1 * pitch + p, xs + k1 * pitch + p, a.k2x + k1, R1, k1,
+                                                       k2yz, gpb, k1 == 0 && ky == 0 && kz == 0});
+    }
+    __syncthreads();
+    if (valid)
+        for (int n2 = it; n2 < R2; n2 += T)
+            with_radix<BIG1>(R1, ColStoreInv{a.S_out + base + n2 * a.rs, R2 * a.rs, xs + n2 * CP + p, pitch});
+}
+
+}  // namespace mixed
+
+template <int MODE>
+static auto mx_x_pick(int R1, int R2) {
+    return R2 > 16   ? mixed::mx_x_kernel<MODE, true, true>
+           : R1 > 16 ? mixed::mx_x_kernel<MODE, true, false>
+                     : mixed::mx_x_kernel<MODE, false, false>;
+}
+
+bool mixed_xupdate(const XUpdArgs& a, cudaStream_t st, cudaError_t* err) {
+    int R1, R2;
+    if (!a.W || !mixed_split(a.L, &R1, &R2)) return false;
+    const size_t smem = sizeof(float2) * R1 * (R2 | 1) * SP * (a.model == 2 ? 1 : 2);
+    auto kern = a.model == 3 ? mx_x_pick<3>(R1, R2) : a.model == 2 ? mx_x_pick<2>(R1, R2) : mx_x_pick<0>(R1, R2);
+    if ((*err = mx_smem(kern, smem)) != cudaSuccess) return true;
+    kern<<<dim3(a.nchunks, a.ny), R1 * SP, smem, st>>>(a, R1, R2);
+    *err = cudaGetLastError();
+    return true;
+}
+
+}  // namespace evx

@@ -1,0 +1,58 @@
+// Two-radix y pass (see evx_mixed.cuh).
+#include "evx_mixed.cuh"
+
+namespace evx {
+namespace mixed {
+
+template <int DIR, bool BIG>
+__global__ void __launch_bounds__(BIG ? 256 : 128, BIG ? 2 : 8) mx_y_kernel(SPassArgs a, int R1, int R2) {
+    extern __shared__ float4 smem4[];
+    float2* xb = reinterpret_cast<float2*>(smem4);
+    const int p = threadIdx.x & 7, it = threadIdx.x >> 3, T = blockDim.x >> 3;
+    const int R2p = R2 | 1;
+    const bool valid = (int)blockIdx.x * CP + p < a.ncols;
+    const long long base = (long long)blockIdx.y * a.os + (long long)blockIdx.x * CP + p;
+    if (valid)
+        for (int n2 = it; n2 < R2; n2 += T)
+            with_radix<BIG>(R1, ColLoad<DIR>{a.in + base + n2 * a.rs, R2 * a.rs, xb + n2 * CP + p, R2p * CP, a.tw, n2});
+    __syncthreads();
+    if (valid)
+        for (int k1 = it; k1 < R1; k1 += T)
+            with_radix<BIG>(R2, ColStore<DIR>{a.out + base + k1 * a.rs, R1 * a.rs, xb + k1 * R2p * CP + p});
+}
+
+}  // namespace mixed
+
+// The radices of a length: the smallest R1 >= R2 whose product is L (0 if none).
+bool mixed_split(int L, int* R1, int* R2) {
+    static const int radices[] = {1, 2, 3, 4, 5, 6, 8, 9, 10, 12, 15, 16, 18, 20, 24, 25, 27, 30, 32};
+    for (int r1 : radices) {
+        if (L % r1) continue;
+        const int r2 = L / r1;
+        if (r2 > r1) continue;
+        for (int r : radices)
+            if (r == r2) {
+                *R1 = r1;
+                *R2 = r2;
+                return true;
+            }
+    }
+    return false;
+}
+
+// true if the strided rows can be addressed with one stride (plain layout)
+static bool plain_rows(int YB, int ny) { return YB == ny; }
+
+bool mixed_spass(const SPassArgs& a, int dir, cudaStream_t st, cudaError_t* err) {
+    int R1, R2;
+    if (!plain_rows(a.YB, a.L) || !mixed_split(a.L, &R1, &R2)) return false;
+    const size_t smem = sizeof(float2) * R1 * (R2 | 1) * SP;
+    auto kern = R1 > 16 ? (dir < 0 ? mixed::mx_y_kernel<-1, true> : mixed::mx_y_kernel<1, true>)
+                        : (dir < 0 ? mixed::mx_y_kernel<-1, false> : mixed::mx_y_kernel<1, false>);
+    if ((*err = mx_smem(kern, smem)) != cudaSuccess) return true;
+    kern<<<dim3(a.nchunks, a.nouter), R1 * SP, smem, st>>>(a, R1, R2);
+    *err = cudaGetLastError();
+    return true;
+}
+
+}  // namespace evx

@@ -166,6 +166,7 @@ ZPassArgs z_args(const evx_grid* g) {
     a.plan = g->pz;
     a.tw = g->twz;
     a.rtw = g->rtw;
+    a.twA = g->ztab ? g->twz + g->M : nullptr;
     a.scale = (float)(1.0 / ((double)g->ny * g->nz));
     a.YB = g->YB;
     a.nxr = g->nx;
@@ -405,6 +406,8 @@ evx_status evx_grid_create(int nx, int ny, int nz, evx_params p, void* cuda_stre
         const int zg = zpass_grid(z);
         const int xg = (g->Zp / SP) * ny;
         g->npart = std::max(std::max(zg, xg), SUM_BLOCKS);
+        z.twA = reinterpret_cast<const float2*>(g);  // non-null: the grid alone is asked for
+        g->npart = std::max(g->npart, mixed_zgrid(z));
         if (fused_yzy_enabled() && fused_yzy_shape(ny, g->M, g->YB)) {
             g->fused = true;
             if (const char* lg = std::getenv("EVX_FUSE_LAG")) g->lag = std::min(16, std::max(1, std::atoi(lg)));
@@ -414,7 +417,18 @@ evx_status evx_grid_create(int nx, int ny, int nz, evx_params p, void* cuda_stre
         TRY(dmalloc(g, &g->d_part, (size_t)g->npart * sizeof(double)));
         TRY(upload(g, &g->twx, twiddles(nx)));
         TRY(upload(g, &g->twy, twiddles(ny)));
-        TRY(upload(g, &g->twz, twiddles(g->M)));
+        {   // followed by the two-radix z pass's orders of w_M^{n2 k1}
+            std::vector<float2> tz = twiddles(g->M);
+            int R1 = 0, R2 = 0;
+            g->ztab = mixed_split(g->M, &R1, &R2);
+            if (g->ztab) {
+                tz.resize(3 * (size_t)g->M);
+                for (int k1 = 0; k1 < R1; ++k1)
+                    for (int n2 = 0; n2 < R2; ++n2)
+                        tz[g->M + k1 * R2 + n2] = tz[2 * g->M + n2 * R1 + k1] = tz[n2 * k1];
+            }
+            TRY(upload(g, &g->twz, tz));
+        }
         TRY(upload(g, &g->rtw, twiddles(nz, g->M + 1)));  // exp(-2 pi i k / nz), k <= M
         TRY(dmalloc(g, &g->k2x, sizeof(float) * nx));
         TRY(dmalloc(g, &g->k2y, sizeof(float) * ny));
