@@ -59,6 +59,7 @@ struct SPassArgs {
     Plan plan;
     const float2* tw;   // L-entry table exp(-2 pi i m / L)
     int generic;        // 1: mixed-radix kernel only (no fast path, no bounded waits)
+    int small;          // grid of at most STAGED_MAX_VOXELS
 };
 
 // x pass fused with the k-space update (one step of the scheme).
@@ -86,6 +87,7 @@ struct XUpdArgs {
                         //   L = (1 - dt M |k|^2 g'(cbar)) / D, B = -dt M |k|^2 / D,
                         //   S' = F_x^-1 [L^n F_x S + B sum_{j<n} L^j F_x W] / L_x (W: F_y F_z N)
     int generic;        // 1: mixed-radix kernel only (no fast path, no bounded waits)
+    int small;          // grid of at most STAGED_MAX_VOXELS
     int nblk;           // model 3: steps per block
     const double* cbar; // model 3: FP64 mean (for g'(cbar))
 };
@@ -157,6 +159,7 @@ struct ZPassArgs {
     // row r of the y-blocked spectrum is caller row x * ny + y
     int map_rows, YB, nxr, nyr;
     int generic;            // 1: mixed-radix kernel only (no fast path)
+    int small;              // grid of at most STAGED_MAX_VOXELS
     int nl_only;            // Z_STEP: form N = d^2 (3 cbar + d) instead of g(c) - g(cbar)
 };
 __host__ __device__ inline long long user_row(long long r, int YB, int nx, int ny) {
@@ -232,6 +235,12 @@ bool fast_zstep(const ZPassArgs& a, cudaStream_t st, cudaError_t* err, int* grid
 bool fast_xadj(const XAdjArgs& a, cudaStream_t st, cudaError_t* err);
 bool fast_zconv(const ZPassArgs& a, int dir, cudaStream_t st, cudaError_t* err, int* grid_used);
 bool fast_paths_enabled();  // false when the environment sets EVX_GENERIC=1
+// grids whose mixed-radix passes run with grouped stages (evx_staged.cu), bit for bit
+constexpr long long STAGED_MAX_VOXELS = 1LL << 22;
+bool staged_spass(const SPassArgs& a, int dir, cudaStream_t st, cudaError_t* err);
+bool staged_xupdate(const XUpdArgs& a, cudaStream_t st, cudaError_t* err);
+bool staged_zpass(const ZPassArgs& a, int mode, cudaStream_t st, cudaError_t* err, int* grid_used);
+int staged_zgrid(const ZPassArgs& a);
 // two-radix passes for lengths R1 R2, R1, R2 <= 32 (evx_mixed.cu); false if not applicable
 bool mixed_split(int L, int* R1, int* R2);
 bool mixed_spass(const SPassArgs& a, int dir, cudaStream_t st, cudaError_t* err);

@@ -719,7 +719,9 @@ bool fast_paths_enabled() {
 
 cudaError_t launch_spass(const SPassArgs& a, int dir, cudaStream_t st) {
     cudaError_t fe;
-    if (!a.generic && fast_paths_enabled() && (fast_spass(a, dir, st, &fe) || mixed_spass(a, dir, st, &fe))) return fe;
+    if (!a.generic && fast_paths_enabled() &&
+        (fast_spass(a, dir, st, &fe) || staged_spass(a, dir, st, &fe) || mixed_spass(a, dir, st, &fe)))
+        return fe;
     const size_t sm = spass_smem(a.L);
     dim3 grid(a.nchunks, a.nouter);
     cudaError_t e;
@@ -735,7 +737,9 @@ cudaError_t launch_spass(const SPassArgs& a, int dir, cudaStream_t st) {
 
 cudaError_t launch_xupdate(const XUpdArgs& a, cudaStream_t st) {
     cudaError_t fe;
-    if (!a.generic && fast_paths_enabled() && (fast_xupdate(a, st, &fe) || mixed_xupdate(a, st, &fe))) return fe;
+    if (!a.generic && fast_paths_enabled() &&
+        (fast_xupdate(a, st, &fe) || staged_xupdate(a, st, &fe) || mixed_xupdate(a, st, &fe)))
+        return fe;
     const size_t sm = xupdate_smem(a.L);
     cudaError_t e;
     if ((e = set_smem(xupdate_kernel, sm)) != cudaSuccess) return e;
@@ -765,7 +769,9 @@ cudaError_t launch_zpass(const ZPassArgs& a, int mode, cudaStream_t st, int* gri
     if ((mode == Z_R2C || mode == Z_C2R) && a.fast_ok && !a.generic && fast_paths_enabled() &&
         fast_zconv(a, mode == Z_R2C ? -1 : 1, st, &fe, grid_used))
         return fe;
-    if (!a.generic && fast_paths_enabled() && mixed_zpass(a, mode, st, &fe, grid_used)) return fe;
+    if (!a.generic && fast_paths_enabled() &&
+        (staged_zpass(a, mode, st, &fe, grid_used) || mixed_zpass(a, mode, st, &fe, grid_used)))
+        return fe;
     const size_t sm = zpass_smem(a.M, a.PZ, a.rows_per_cta);
     const int grid = zpass_grid(a);
     if (grid_used) *grid_used = grid;

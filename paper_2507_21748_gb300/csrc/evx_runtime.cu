@@ -113,6 +113,8 @@ static evx_status upload_k2(evx_grid* g) {
 // ------------------------------------------------------------ pass args
 namespace evxrt {
 
+static int small_grid(const evx_grid* g) { return (long long)g->nx * g->ny * g->nz <= STAGED_MAX_VOXELS; }
+
 SPassArgs y_args(const evx_grid* g, const float2* in, float2* out) {
     SPassArgs a{};
     a.in = in;
@@ -127,6 +129,7 @@ SPassArgs y_args(const evx_grid* g, const float2* in, float2* out) {
     a.nchunks = g->Zp / SP;
     a.plan = g->py;
     a.tw = g->twy;
+    a.small = small_grid(g);
     return a;
 }
 
@@ -153,6 +156,7 @@ XUpdArgs x_args(const evx_grid* g, const float2* W, float2* S, float2* S_out, do
     a.dtMk = (float)(dt * M * kappa);
     a.invL = (float)(1.0 / g->nx);
     a.model = g->model == EVX_MODEL_AC ? 1 : 0;
+    a.small = small_grid(g);
     return a;
 }
 
@@ -171,6 +175,7 @@ ZPassArgs z_args(const evx_grid* g) {
     a.YB = g->YB;
     a.nxr = g->nx;
     a.nyr = g->ny;
+    a.small = small_grid(g);
     return a;
 }
 
@@ -407,7 +412,7 @@ evx_status evx_grid_create(int nx, int ny, int nz, evx_params p, void* cuda_stre
         const int xg = (g->Zp / SP) * ny;
         g->npart = std::max(std::max(zg, xg), SUM_BLOCKS);
         z.twA = reinterpret_cast<const float2*>(g);  // non-null: the grid alone is asked for
-        g->npart = std::max(g->npart, mixed_zgrid(z));
+        g->npart = std::max(g->npart, std::max(mixed_zgrid(z), staged_zgrid(z)));
         if (fused_yzy_enabled() && fused_yzy_shape(ny, g->M, g->YB)) {
             g->fused = true;
             if (const char* lg = std::getenv("EVX_FUSE_LAG")) g->lag = std::min(16, std::max(1, std::atoi(lg)));
