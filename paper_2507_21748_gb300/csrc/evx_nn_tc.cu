@@ -1,6 +1,6 @@
 // tcgen05 engine of the surrogate's 32 -> 32 convolutions (sm_103a).
 //
-// Both kernels compute the periodic 3x3x3 convolution as an implicit GEMM on
+// conv_ring_kernel computes the periodic 3x3x3 convolution as an implicit GEMM on
 // the 5th-generation tensor cores: D[128 voxels x N] (FP32, in tensor memory)
 // += A[128 x 16] (BF16 activations, shared memory) x B[16 x N] (BF16 weights,
 // shared memory), over the taps and 2 K-steps of 16 input channels. The
@@ -9,8 +9,7 @@
 // distance of core matrices adjacent along K (leading byte offset, 128 B) and
 // along N (stride byte offset, 512 B)).
 //
-// conv_ring_kernel (Z a multiple of 128): a persistent, warp-specialised
-// pipeline. A work unit is a run of output rows (b, x, y = ys .. ye-1,
+// It is a persistent, warp-specialised pipeline. A work unit is a run of output rows (b, x, y = ys .. ye-1,
 // z0 .. z0+127); the 128 voxels of a row are the MMA's M. The kernel walks the
 // INPUT rows y' = ys-1 .. ye: a ring slot holds input row (b, x-1 .. x+1, y')
 // as [dx][z][32 ci] with 64-byte z rows in the 64-byte swizzle layout, exactly
@@ -36,8 +35,15 @@
 //               the block, applies bias and the fused epilogue and stores BF16
 //               channels-last; the two partial rows at each end of a unit are
 //               dropped
-// conv_tc_kernel (Z a multiple of 64): an unpipelined variant per tile of
-// 2 rows x 64 z with three dz-shifted no-swizzle halo copies, N = 32.
+// Rows are walked along y when Z is a multiple of 128 and along x otherwise: an
+// output's taps are then added in the order (dy, dx, dz) and (dx, dy, dz), the
+// orders earlier versions used for these sizes (results to the bit).
+//
+// When Z is an odd multiple of 64 the last z chunk of a row holds 64 voxels: the
+// producer loads 64-row boxes, the MMAs still run with M = 128 (the upper lanes
+// accumulate stale rows, and are zeroed and not stored). Half of such a chunk's
+// tensor work is idle, but an unpipelined kernel with 2 x 64 voxel tiles took
+// 740 us where this takes 180 us (4 x 64^3, GELU epilogue).
 //
 // Every mbarrier wait is bounded (about 1 s); a wait that runs out sets the
 // device flag g_tc_timeout, makes the other roles stop, waits (bounded) for
@@ -80,15 +86,7 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-__device__ __forceinline__ void tc_mma(uint32_t dtmem, uint64_t a, uint64_t b, uint32_t idesc, int acc) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtmem),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc)
-        : "memory");
-}
-
-// the same MMA executed by the whole (converged) warp and issued by lane 0 alone
+// one MMA, executed by the whole (converged) warp and issued by lane 0 alone
 // through an instruction predicate: no divergent branch around the issue, which
 // on sm_103a took the ring's 18-MMA issue sequence from about 1,570 to 1,200 cycles
 __device__ __forceinline__ void tc_mma_lane0(uint32_t dtmem, uint64_t a, uint64_t b, uint32_t idesc) {
@@ -254,15 +252,6 @@ __device__ __forceinline__ void resid32_staged(const ConvArgs& a, long long vox0
     __syncwarp();  // staging reads done before the next row overwrites it
 }
 
-// weights [t][co][ci] -> core-matrix layout [t][co/8][ci/8][8 co][8 ci]
-__device__ __forceinline__ void stage_weights(unsigned char* swb, const __nv_bfloat16* w, int nthreads) {
-    for (int e = threadIdx.x; e < 27 * 32 * 4; e += nthreads) {  // 16-byte pieces (t, co, ci/8)
-        const int cig = e & 3, co = (e >> 2) & 31, t = e >> 7;
-        const uint4 v = *reinterpret_cast<const uint4*>(w + (t * 32 + co) * 32 + cig * 8);
-        *reinterpret_cast<uint4*>(swb + (((t * 4 + (co >> 3)) * 4 + cig) * 8 + (co & 7)) * 16) = v;
-    }
-}
-
 // ----------------------------------------------- pipelined scatter kernel
 namespace ring {
 constexpr int ZT = 128;                    // voxels per output row tile (MMA M)
@@ -278,15 +267,17 @@ constexpr int BAR = WB + NS * SLOT;        // barriers: full[NS], tfull[NBLK], t
 constexpr int STG = (BAR + 8 * (NS + 2 * NBLK) + 16 + 15) & ~15;  // after the tensor-memory slot and abort flag
 constexpr int STG_WARP = 32 * 16 * 4;      // per epilogue warp: [32 voxels][16 channels] FP32 staging
 constexpr int SMEM = STG + NEPI * STG_WARP + 1024;  // + alignment
-constexpr uint32_t SLOT_TX = SLOT;         // TMA bytes per slot
 constexpr long long WAIT_BUDGET = 1LL << 31;
 }  // namespace ring
 
 struct RingArgs {
     ConvArgs a;
-    int nzc;     // Z / 128
-    int nseg;    // y segments per (b, x, z-chunk) column
-    int nunits;  // B * X * nzc * nseg
+    int nzc;     // z chunks: ceil(Z / 128), the last of 64 voxels when Z is an odd multiple of 64
+    int zbox;    // z rows of the main TMA box: 128, or 64 when there is a 64-voxel chunk
+    int walkx;   // 0: columns (b, x, z chunk) walked along y; 1: columns (b, y, z chunk) walked along x
+    int len;     // rows of a column (Y or X)
+    int nseg;    // segments of a column
+    int nunits;  // columns * nseg
 };
 
 // non-blocking probe of a phase (no suspend, unlike try_wait)
@@ -317,13 +308,13 @@ __device__ __forceinline__ bool ring_wait(uint32_t bar, uint32_t parity, volatil
     }
 }
 
-// unit u -> column bx = b * X + x, z-chunk start z0, output rows ys .. ye-1
+// unit u -> column bx = b * X + x (b * Y + y), z-chunk start z0, output rows ys .. ye-1
 __device__ __forceinline__ void ring_unit(const RingArgs& r, int u, int& bx, int& z0, int& ys, int& ye) {
     const int seg = u % r.nseg, col = u / r.nseg;
     z0 = (col % r.nzc) * ring::ZT;
     bx = col / r.nzc;
-    ys = (int)((long long)seg * r.a.Y / r.nseg);
-    ye = (int)((long long)(seg + 1) * r.a.Y / r.nseg);
+    ys = (int)((long long)seg * r.len / r.nseg);
+    ye = (int)((long long)(seg + 1) * r.len / r.nseg);
 }
 
 // accumulator block of virtual output row v: descending, so that the rows
@@ -363,10 +354,11 @@ __global__ void __launch_bounds__(ring::NTH, 1)
     const int X = a.X, Y = a.Y, Z = a.Z;
 
     // weights [t][co][ci] -> [dx][dz][n = 32 (dy+1) + co][ci]: one input row feeds the output rows
-    // y' + 1 (dy = -1), y' (dy = 0), y' - 1 (dy = +1) through N = 96 stacked columns
+    // y' + 1 (dy = -1), y' (dy = 0), y' - 1 (dy = +1) through N = 96 stacked columns (walking x:
+    // x and y change places)
     for (int e = threadIdx.x; e < 9 * 96 * 4; e += NTH) {
         const int kg = e & 3, n = (e >> 2) % 96, dd = e / (96 * 4), dxi = dd / 3, dzi = dd % 3;
-        const int t = 9 * dxi + 3 * (n >> 5) + dzi, co = n & 31;
+        const int t = r.walkx ? 9 * (n >> 5) + 3 * dxi + dzi : 9 * dxi + 3 * (n >> 5) + dzi, co = n & 31;
         const uint4 v = *reinterpret_cast<const uint4*>(a.w + (t * 32 + co) * 32 + kg * 8);
         *reinterpret_cast<uint4*>(swb + (((dd * 12 + (n >> 3)) * 4 + kg) * 8 + (n & 7)) * 16) = v;
     }
@@ -410,9 +402,10 @@ __global__ void __launch_bounds__(ring::NTH, 1)
         for (int u = blockIdx.x; u < r.nunits && ok; u += gridDim.x) {
             int bx, z0, ys, ye;
             ring_unit(r, u, bx, z0, ys, ye);
-            const int b = bx / X, x = bx - b * X;
+            const int across = r.walkx ? Y : X, b = bx / across, x = bx - b * across;
+            const int nz = min(ZT, Z - z0);  // 128, or 64 in a last half chunk (its rows 64 .. are not loaded)
             for (int j = -1; j <= ye - ys; ++j) {
-                const int yp = (ys + j + Y) % Y;
+                const int yp = (ys + j + r.len) % r.len;
                 const uint32_t slot = k % NS;
                 uint32_t w_ok = 1;
                 if (lane == 0 && k >= NS)
@@ -424,15 +417,17 @@ __global__ void __launch_bounds__(ring::NTH, 1)
                 }
                 if (lane == 0) {
                     const uint32_t base = smem_addr(sring + slot * SLOT);
-                    const int zl = (z0 - 16 + Z) % Z, zr = (z0 + ZT) % Z;  // periodic z halo: 16-row boxes
-                    mbar_expect_tx(full + 8 * slot, SLOT_TX);
+                    const int zl = (z0 - 16 + Z) % Z, zr = (z0 + nz) % Z;  // periodic z halo: 16-row boxes
+                    mbar_expect_tx(full + 8 * slot, 3 * (nz + 32) * 64);
 #pragma unroll
                     for (int dxi = 0; dxi < 3; ++dxi) {
-                        const int bxx = b * X + (x + dxi - 1 + X) % X;
+                        const int side = (x + dxi - 1 + across) % across;
+                        const int cy = r.walkx ? side : yp, cx = b * X + (r.walkx ? yp : side);
                         const uint32_t run = base + dxi * RUN;
-                        tma_load4(run + 16 * 64, &map, 0, z0, yp, bxx, full + 8 * slot);
-                        tma_load4(run, &hmap, 0, zl, yp, bxx, full + 8 * slot);
-                        tma_load4(run + (16 + ZT) * 64, &hmap, 0, zr, yp, bxx, full + 8 * slot);
+                        tma_load4(run + 16 * 64, &map, 0, z0, cy, cx, full + 8 * slot);
+                        if (nz > r.zbox) tma_load4(run + (16 + 64) * 64, &map, 0, z0 + 64, cy, cx, full + 8 * slot);
+                        tma_load4(run, &hmap, 0, zl, cy, cx, full + 8 * slot);
+                        tma_load4(run + (16 + nz) * 64, &hmap, 0, zr, cy, cx, full + 8 * slot);
                     }
                 }
                 __syncwarp();
@@ -553,8 +548,10 @@ __global__ void __launch_bounds__(ring::NTH, 1)
                 fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(tempty + 8 * blk);
-                if (jv >= 2 && jv < L + 2) {
-                    const long long vox0 = ((long long)bx * Y + (ys + jv - 2)) * Z + z0 + q4 * 32;
+                if (jv >= 2 && jv < L + 2 && z0 + q4 * 32 < Z) {  // a half chunk's lanes 64 .. are not voxels
+                    const int o = ys + jv - 2;
+                    const long long line = r.walkx ? ((long long)(bx / Y) * X + o) * Y + bx % Y : (long long)bx * Y + o;
+                    const long long vox0 = line * Z + z0 + q4 * 32;
                     if (EPI == EVX_NN_EPI_RESID32)
                         resid32_staged(a, vox0, h * 16, acc, bias, stg, lane);
                     else
@@ -569,127 +566,6 @@ __global__ void __launch_bounds__(ring::NTH, 1)
     if (warp == 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(NBLK * 32) : "memory");
 }
-
-// ---------------------------------------------------- unpipelined tile kernel
-// Implicit GEMM on the 5th-generation tensor cores: per tile of 128 output
-// voxels (2 rows x 64 z) D[128 x 32] (FP32, tensor memory) accumulates
-// 27 taps x 2 K-steps of A[128 x 16] (BF16 activations) times B[16 x 32]
-// (BF16 weights). Operands sit in shared memory in the no-swizzle K-major
-// core-matrix layout (8 rows x 16 bytes per 128-byte core matrix): weights as
-// [t][co/8][ci/8][8][8], the halo as three copies shifted by dz = -1, 0, +1 so
-// that every tap's A operand starts on an 8-voxel boundary:
-// [dz][halo row][v/8][ci/8][8][8]. Core matrices adjacent along K are 128 B
-// apart (leading byte offset), along M/N 512 B (stride byte offset).
-// One thread issues the MMAs, the commit arrives on an mbarrier (bounded
-// wait), and each of the 4 warps reads its 32 accumulator lanes (one voxel
-// row each) with tcgen05.ld for the fused epilogue.
-template <int EPI>
-__global__ void __launch_bounds__(128, 1) conv_tc_kernel(ConvArgs a) {
-    constexpr int C = 32, HALO = HR * 8 * 4 * 128;  // bytes per dz copy
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    unsigned char* swb = smem_raw;                          // weights: 27 * 4 * 4 * 128 B
-    unsigned char* shalo = smem_raw + 27 * 4 * 4 * 128;     // 3 copies of HALO bytes
-    uint64_t* bar = reinterpret_cast<uint64_t*>(shalo + 3 * HALO);
-    uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 1);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // weights -> core-matrix layout
-    for (int e = threadIdx.x; e < 27 * C * 4; e += 128) {  // 16-byte pieces: (t, co, cig)
-        const int cig = e & 3, co = (e >> 2) % C, t = e / (4 * C);
-        const uint4 v = *reinterpret_cast<const uint4*>(a.w + ((long long)t * C + co) * C + cig * 8);
-        *reinterpret_cast<uint4*>(swb + (((t * 4 + (co >> 3)) * 4 + cig) * 8 + (co & 7)) * 16) = v;
-    }
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 32;" ::"r"(smem_addr(tslot))
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    if (threadIdx.x == 0) {
-        mbar_init(smem_addr(bar), 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = *tslot;
-    float bias[32];
-#pragma unroll
-    for (int i = 0; i < 32; ++i) bias[i] = a.bias ? a.bias[i] : 0.f;
-    constexpr uint32_t IDESC = idesc_bf16(128, 32);
-    uint32_t parity = 0;
-    bool failed = false;
-    for (int tile = blockIdx.x; tile < a.ntiles && !failed; tile += gridDim.x) {
-        int b, x, y0, z0;
-        tile_coords(tile, a.X, a.Y, a.Z, b, x, y0, z0);
-        // halo -> three dz-shifted copies in core-matrix layout
-        for (int e = threadIdx.x; e < HR * (TZ + 2) * 4; e += 128) {
-            const int cig = e & 3, rem = e >> 2, zi = rem % (TZ + 2), nb = rem / (TZ + 2);
-            const int dx = nb / (TY + 2) - 1, yi = nb % (TY + 2) - 1;
-            const int xx = (x + dx + a.X) % a.X, yy = (y0 + yi + a.Y) % a.Y, zz = (z0 + zi - 1 + a.Z) % a.Z;
-            const long long vox = (((long long)b * a.X + xx) * a.Y + yy) * a.Z + zz;
-            const uint4 v = *reinterpret_cast<const uint4*>(a.in + vox * C + cig * 8);
-#pragma unroll
-            for (int s = 0; s < 3; ++s) {  // copy s holds position p = zi - s (dz = s - 1)
-                const int p = zi - s;
-                if (p >= 0 && p < TZ)
-                    *reinterpret_cast<uint4*>(shalo + s * HALO + (((nb * 8 + (p >> 3)) * 4 + cig) * 8 + (p & 7)) * 16) =
-                        v;
-            }
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncthreads();
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        if (threadIdx.x == 0) {
-            const uint32_t hbase = smem_addr(shalo), wbase = smem_addr(swb);
-            int k = 0;
-            for (int t = 0; t < 27; ++t) {
-                const int dxi = t / 9, dyi = (t / 3) % 3, s = t % 3;
-                const int nb0 = dxi * (TY + 2) + dyi;  // halo row of the first output row (yl = 0)
-#pragma unroll
-                for (int ks = 0; ks < 2; ++ks, ++k) {
-                    const uint64_t ad = sdesc(hbase + s * HALO + ((nb0 * 8) * 4 + 2 * ks) * 128, 128, 512);
-                    const uint64_t bd = sdesc(wbase + (t * 16 + 2 * ks) * 128, 128, 512);
-                    tc_mma(tmem, ad, bd, IDESC, k > 0);
-                }
-            }
-            tc_commit(smem_addr(bar));
-        }
-        const bool ok = tc_wait(smem_addr(bar), parity);
-        if (__syncthreads_or(!ok)) {
-            failed = true;
-            break;
-        }
-        parity ^= 1;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        // epilogue: thread = accumulator lane = voxel m of the tile (m < 64: row y0, else y0 + 1)
-        uint32_t r[32];
-        const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16);
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-            "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-              "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-              "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
-              "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
-              "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-            : "r"(taddr)
-            : "memory");
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        const int m = warp * 32 + lane;
-        const long long vox = (((long long)b * a.X + x) * a.Y + y0 + (m >> 6)) * a.Z + z0 + (m & 63);
-        epilogue_store<EPI, 32>(a, vox, 0, r, bias);
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncthreads();  // accumulator read before the next tile's MMAs overwrite it
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    }
-    if (failed && threadIdx.x == 0) {
-        atomicExch(&g_tc_timeout, 1);
-        tc_wait(smem_addr(bar), parity);  // let the outstanding commit land (bounded) before freeing TMEM
-    }
-    __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 32;" ::"r"(tmem) : "memory");
-}
-
 
 }  // namespace evxnn
 
@@ -729,43 +605,34 @@ bool ring_map(CUtensorMap* m, const ConvArgs& a, int zrows) {
 }
 
 template <int EPI>
-cudaError_t launch_ring(const ConvArgs& a, cudaStream_t st, int sms, bool* launched) {
-    *launched = false;
-    CUtensorMap map, hmap;
-    if (a.Z % ring::ZT || !ring_map(&map, a, ring::ZT) || !ring_map(&hmap, a, 16)) return cudaSuccess;
+cudaError_t launch_ring(const ConvArgs& a, cudaStream_t st, int sms) {
     RingArgs r{};
     r.a = a;
-    r.nzc = a.Z / ring::ZT;
-    const long long ncol = (long long)a.B * a.X * r.nzc;
-    int nseg = 1;  // split columns along y until there are enough units for an even spread
-    while (ncol * nseg < 8LL * sms && nseg * 2 <= a.Y / 8) nseg *= 2;
-    if (ncol * nseg > (1LL << 30)) return cudaSuccess;  // unit index would overflow int: not launched, tile kernel
+    r.nzc = (a.Z + ring::ZT - 1) / ring::ZT;
+    r.zbox = a.Z % ring::ZT ? 64 : ring::ZT;
+    CUtensorMap map, hmap;
+    if (!ring_map(&map, a, r.zbox) || !ring_map(&hmap, a, 16)) return cudaErrorInvalidValue;
+    r.walkx = a.Z % ring::ZT != 0;
+    r.len = r.walkx ? a.X : a.Y;
+    const long long ncol = (long long)a.B * (r.walkx ? a.Y : a.X) * r.nzc;
+    // columns split into segments of at least 8 rows: the split with the fewest
+    // input rows on the busiest CTA (a segment of n rows walks n + 2)
+    int nseg = 1;
+    long long best = 0;
+    for (int s = 1; s == 1 || s <= r.len / 8; ++s) {
+        const long long rows = (ncol * s + sms - 1) / sms * ((r.len + s - 1) / s + 2);
+        if (s == 1 || rows < best) {
+            best = rows;
+            nseg = s;
+        }
+    }
+    if (ncol * nseg > (1LL << 30)) return cudaErrorInvalidValue;  // unit index would overflow int
     r.nseg = nseg;
     r.nunits = (int)(ncol * nseg);
     cudaError_t e = cudaFuncSetAttribute(conv_ring_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, ring::SMEM);
     if (e != cudaSuccess) return e;
     conv_ring_kernel<EPI><<<std::min(r.nunits, sms), ring::NTH, ring::SMEM, st>>>(map, hmap, r);
-    *launched = true;
     return cudaGetLastError();
-}
-
-template <int EPI>
-cudaError_t launch_tile(const ConvArgs& a0, cudaStream_t st, int sms) {
-    ConvArgs a = a0;
-    a.ntiles = a.B * a.X * (a.Y / TY) * (a.Z / TZ);
-    const size_t smem = 27 * 4 * 4 * 128 + 3 * (size_t)HR * 8 * 4 * 128 + 16;
-    cudaError_t e = cudaFuncSetAttribute(conv_tc_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    conv_tc_kernel<EPI><<<std::min(a.ntiles, sms), 128, smem, st>>>(a);
-    return cudaGetLastError();
-}
-
-template <int EPI>
-cudaError_t conv32_tc_epi(const ConvArgs& a, cudaStream_t st, int sms) {
-    bool launched = false;
-    const cudaError_t e = launch_ring<EPI>(a, st, sms, &launched);
-    if (launched || e != cudaSuccess) return e;
-    return launch_tile<EPI>(a, st, sms);
 }
 }  // namespace
 
@@ -773,11 +640,11 @@ namespace evxnn {
 
 cudaError_t conv32_tc(const ConvArgs& a, int epilogue, cudaStream_t st, int sms) {
     switch (epilogue) {
-        case EVX_NN_EPI_PLAIN: return conv32_tc_epi<EVX_NN_EPI_PLAIN>(a, st, sms);
-        case EVX_NN_EPI_GELU: return conv32_tc_epi<EVX_NN_EPI_GELU>(a, st, sms);
-        case EVX_NN_EPI_RESID: return conv32_tc_epi<EVX_NN_EPI_RESID>(a, st, sms);
-        case EVX_NN_EPI_GELU_BWD: return conv32_tc_epi<EVX_NN_EPI_GELU_BWD>(a, st, sms);
-        case EVX_NN_EPI_RESID32: return conv32_tc_epi<EVX_NN_EPI_RESID32>(a, st, sms);
+        case EVX_NN_EPI_PLAIN: return launch_ring<EVX_NN_EPI_PLAIN>(a, st, sms);
+        case EVX_NN_EPI_GELU: return launch_ring<EVX_NN_EPI_GELU>(a, st, sms);
+        case EVX_NN_EPI_RESID: return launch_ring<EVX_NN_EPI_RESID>(a, st, sms);
+        case EVX_NN_EPI_GELU_BWD: return launch_ring<EVX_NN_EPI_GELU_BWD>(a, st, sms);
+        case EVX_NN_EPI_RESID32: return launch_ring<EVX_NN_EPI_RESID32>(a, st, sms);
     }
     return cudaErrorInvalidValue;
 }
