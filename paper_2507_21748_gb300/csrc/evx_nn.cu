@@ -831,6 +831,14 @@ evx_status conv_epi(int epi, const ConvArgs& a, cudaStream_t st) {
 template <int CIN, int COUT>
 evx_status launch_wgrad(const WgradArgs& a0, float* dw, float* partials, size_t partial_floats,
                         cudaStream_t st) {
+    if (CIN == 32 && COUT == 32 && use_tcgen05()) {
+        int ctas = 0;
+        cudaError_t e = wgrad32_tc(a0.dy, a0.x, partials, (int)std::min<size_t>(partial_floats / (27 * 1024), 1 << 20), a0.B,
+                                   a0.X, a0.Y, a0.Z, st, nn_sms(), &ctas);
+        if (e != cudaSuccess) return nn_cuda(e);
+        reduce_partials_f32<<<108, 256, 0, st>>>(partials, ctas, 27 * 1024, dw);
+        return nn_cuda(cudaGetLastError());
+    }
     WgradArgs a = a0;
     a.ntiles = a.B * a.X * (a.Y / TY) * (a.Z / TZ);
     const size_t smem = sizeof(__nv_bfloat16) * (HR * (TZ + 2) * (CIN + 8) + TY * TZ * (COUT + 8));

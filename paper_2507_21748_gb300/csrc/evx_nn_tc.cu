@@ -308,6 +308,21 @@ __device__ __forceinline__ bool ring_wait(uint32_t bar, uint32_t parity, volatil
     }
 }
 
+// as ring_wait for an event at the end of the kernel: gives up when another role has,
+// or after 32 times the bound of a single pipeline wait
+__device__ __forceinline__ bool ring_wait_long(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+    const long long t0 = clock64();
+    while (true) {
+        if (mbar_try(bar, parity)) return true;
+        if (*abort_flag) return false;
+        if (clock64() - t0 > 32 * ring::WAIT_BUDGET) {
+            *abort_flag = 1;
+            atomicExch(&g_tc_timeout, 1);
+            return false;
+        }
+    }
+}
+
 // unit u -> column bx = b * X + x (b * Y + y), z-chunk start z0, output rows ys .. ye-1
 __device__ __forceinline__ void ring_unit(const RingArgs& r, int u, int& bx, int& z0, int& ys, int& ye) {
     const int seg = u % r.nseg, col = u / r.nseg;
@@ -567,6 +582,219 @@ __global__ void __launch_bounds__(ring::NTH, 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(NBLK * 32) : "memory");
 }
 
+// ------------------------------------------------------- weight gradient
+// dW[t][co][ci] = sum_v dY(v, co) X(v + off_t, ci): a GEMM whose K is the voxels.
+// Both operands lie in shared memory as TMA writes them, rows of one voxel's 32
+// channels (64 bytes, 64-byte swizzle), so the MMA reads both with the channels
+// contiguous (MN-major) and no transposition. One input row (x' = x - 1 .. x + 1,
+// y', 128 z) meets the three output rows y' - 1, y', y' + 1:
+//   A (M = 128): four groups of 32 ci, one z row (64 bytes) apart: dz = -1, 0, +1
+//                and a fourth that is not used
+//   B (N = 96):  three groups of 32 co, one dY row slot apart: dy = +1, 0, -1
+//   K = 16 voxels per MMA: 3 dx x 8 = 24 MMAs per row into 3 x 96 columns of
+//   tensor memory, accumulated over every row of the CTA (27 taps at once)
+// An input row costs about what a convolution's does (18 MMAs of N = 96); a unit's
+// rows each count in full (the halo is on the dY rows: 8 of the 38 KB a row
+// loads). The mma.sync kernel it replaces for 32 -> 32 re-read its fragments from
+// shared memory for every tap: 382 us at 64 x 96 x 128 and 3.71 ms at 4 x 128^3 with the
+// sum of the partials, this kernel 102 us and 0.62 ms (error against 64 bits unchanged).
+//   warp 0 producer, warp 1 MMA issuer, warps 2..5 write the CTA's partial sums.
+namespace wg {
+constexpr int NS = 4;                        // input-row slots (3 runs each, as in the ring)
+constexpr int NR = 11;                       // dY row slots (128 z x 64 bytes)
+constexpr int DYROW = 128 * 64;
+constexpr int XOFF = NR * DYROW;
+constexpr int BAR = XOFF + NS * ring::SLOT;  // full[NS], free[NS], done
+constexpr int SMEM = BAR + 8 * (2 * NS + 1) + 16 + 1024;
+constexpr int NTH = 6 * 32;
+constexpr uint32_t COLS = 512;
+}  // namespace wg
+
+struct WgArgs {
+    float* partials;  // [grid][27][32][32]
+    int B, X, Y, Z, nzc, zbox, nseg, nunits;
+};
+
+// MN-major operand in the 64-byte swizzle layout: 8 K rows of 64 bytes per 512-byte
+// group (stride byte offset), groups of 32 channels mn_stride bytes apart (leading)
+__device__ __forceinline__ uint64_t sdesc_mn64(uint32_t saddr, uint32_t mn_stride) {
+    return sdesc(saddr, mn_stride, 512) | (4ull << 61);
+}
+__host__ __device__ constexpr uint32_t idesc_bf16_mn(int M, int N) { return idesc_bf16(M, N) | (1u << 15) | (1u << 16); }
+
+__device__ __forceinline__ void tc_mma_lane0_acc(uint32_t dtmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n .reg .pred p, q;\n .reg .u32 l;\n mov.u32 l, %%laneid;\n setp.eq.u32 p, l, 0;\n"
+        " setp.ne.b32 q, %4, 0;\n @p tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, q;\n}\n" ::"r"(dtmem),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc)
+        : "memory");
+}
+
+__device__ __forceinline__ void wg_unit(const WgArgs& r, int u, int& bx, int& z0, int& ys, int& ye) {
+    const int seg = u % r.nseg, col = u / r.nseg;
+    z0 = (col % r.nzc) * ring::ZT;
+    bx = col / r.nzc;
+    ys = (int)((long long)seg * r.Y / r.nseg);
+    ye = (int)((long long)(seg + 1) * r.Y / r.nseg);
+}
+
+__global__ void __launch_bounds__(wg::NTH, 1)
+    conv_wgrad_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap xhalo,
+                         const __grid_constant__ CUtensorMap dymap, WgArgs r) {
+    using namespace wg;
+    using ring::RUN;
+    using ring::SLOT;
+    using ring::ZT;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    unsigned char* sm = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
+    const uint32_t sdy = smem_addr(sm), sx = smem_addr(sm + XOFF);
+    const uint32_t full = smem_addr(sm + BAR), freeb = full + 8 * NS, done = freeb + 8 * NS;
+    uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + BAR + 8 * (2 * NS + 1));
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int X = r.X, Y = r.Y, Z = r.Z;
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tslot)), "n"(COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < 2 * NS + 1; ++s) mbar_init(full + 8 * s, 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem = *tslot;
+    if (warp == 0) {
+        // ---------------------------------------------------------- producer
+        // Input row k takes slot k % NS once row k - NS has been consumed; dY row q takes
+        // slot q % NR once the last input row that reads q - NR has been.
+        uint32_t k = 0, q = 0;
+        uint32_t last[NR];  // input row (plus one) that last reads the dY row held by a slot
+#pragma unroll
+        for (int i = 0; i < NR; ++i) last[i] = 0;
+        if (lane == 0) {
+            uint32_t seen = 0;  // input rows known to be consumed
+            bool ok = true;
+            auto consumed = [&](uint32_t n) {  // wait until the first n input rows are
+                if (n <= seen) return true;
+                if (!ring_wait(freeb + 8 * ((n - 1) % NS), ((n - 1) / NS) & 1, abort_flag)) return false;
+                seen = n;
+                return true;
+            };
+            for (int u = blockIdx.x; u < r.nunits && ok; u += gridDim.x) {
+                int bx, z0, ys, ye;
+                wg_unit(r, u, bx, z0, ys, ye);
+                const int b = bx / X, x = bx - b * X, L = ye - ys;
+                const int nz = min(ZT, Z - z0);
+                const int zl = (z0 - 16 + Z) % Z, zr = (z0 + nz) % Z;
+                for (int i = 0; i < L; ++i, ++k) {
+                    if (k >= (uint32_t)NS && !(ok = consumed(k - NS + 1))) break;
+                    const int nd = i == 0 ? 3 : 1;  // dY rows that arrive with this input row
+                    for (int d = 0; d < nd && ok; ++d) ok = consumed(last[(q + d) % NR]);
+                    if (!ok) break;
+                    const uint32_t bar = full + 8 * (k % NS);
+                    mbar_expect_tx(bar, 3 * (nz + 32) * 64 + nd * nz * 64);
+                    for (int d = 0; d < nd; ++d, ++q) {
+                        const int j = i == 0 ? d : i + 2;  // dY row ys - 1 + j, read by input rows j - 2 .. j of the unit
+                        const int yd = (ys - 1 + j + Y) % Y;
+                        const uint32_t dst = sdy + (q % NR) * DYROW;
+                        last[q % NR] = k - i + min(j, L - 1) + 1;
+                        tma_load4(dst, &dymap, 0, z0, yd, bx, bar);
+                        if (nz > r.zbox) tma_load4(dst + 64 * 64, &dymap, 0, z0 + 64, yd, bx, bar);
+                    }
+                    const int yp = ys + i;
+                    const uint32_t base = sx + (k % NS) * SLOT;
+#pragma unroll
+                    for (int dxi = 0; dxi < 3; ++dxi) {
+                        const int cx = b * X + (x + dxi - 1 + X) % X;
+                        const uint32_t run = base + dxi * RUN;
+                        tma_load4(run + 16 * 64, &xmap, 0, z0, yp, cx, bar);
+                        if (nz > r.zbox) tma_load4(run + (16 + 64) * 64, &xmap, 0, z0 + 64, yp, cx, bar);
+                        tma_load4(run, &xhalo, 0, zl, yp, cx, bar);
+                        tma_load4(run + (16 + nz) * 64, &xhalo, 0, zr, yp, cx, bar);
+                    }
+                }
+            }
+            if (!ok)  // let the copies in flight land before the CTA exits (bounded)
+                for (uint32_t m = (k > (uint32_t)NS ? k - NS : 0); m < k; ++m) tc_wait(full + 8 * (m % NS), (m / NS) & 1);
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        // ------------------------------------------------------- MMA issuer
+        constexpr uint32_t I96 = idesc_bf16_mn(128, 96), I64 = idesc_bf16_mn(128, 64), I32 = idesc_bf16_mn(128, 32);
+        uint32_t k = 0, q = 0;
+        bool ok = true;
+        for (int u = blockIdx.x; u < r.nunits && ok; u += gridDim.x) {
+            int bx, z0, ys, ye;
+            wg_unit(r, u, bx, z0, ys, ye);
+            const int L = ye - ys, ksteps = min(ZT, Z - z0) / 16;
+            for (int i = 0; i < L; ++i, ++k, ++q) {
+                uint32_t w_ok = 1;
+                if (lane == 0) w_ok = ring_wait(full + 8 * (k % NS), (k / NS) & 1, abort_flag);
+                if (!__shfl_sync(0xffffffffu, w_ok, 0)) {
+                    ok = false;
+                    break;
+                }
+                const uint32_t s0 = q % NR;  // slots of the dY rows y' - 1, y', y' + 1: s0, s0 + 1, s0 + 2 (mod NR)
+                const uint64_t a0 = sdesc_mn64(sx + (k % NS) * SLOT + 15 * 64, 64);
+                const uint64_t b0 = sdesc_mn64(sdy + s0 * DYROW, DYROW), bw = sdesc_mn64(sdy, DYROW);
+                if (s0 <= NR - 3) {
+                    for (int ks = 0; ks < ksteps; ++ks)
+#pragma unroll
+                        for (int dx = 0; dx < 3; ++dx)
+                            tc_mma_lane0_acc(tmem + dx * 96, a0 + (dx * RUN + ks * 1024) / 16, b0 + ks * 64, I96,
+                                             k > 0 || ks > 0);
+                } else {  // the three slots wrap (never at k = 0): N = 64 + 32 or 32 + 64
+                    const uint32_t n1 = (NR - s0) * 32, i1 = n1 == 64 ? I64 : I32, i2 = n1 == 64 ? I32 : I64;
+                    for (int ks = 0; ks < ksteps; ++ks)
+#pragma unroll
+                        for (int dx = 0; dx < 3; ++dx) {
+                            const uint64_t ad = a0 + (dx * RUN + ks * 1024) / 16;
+                            tc_mma_lane0_acc(tmem + dx * 96, ad, b0 + ks * 64, i1, 1);
+                            tc_mma_lane0_acc(tmem + dx * 96 + n1, ad, bw + ks * 64, i2, 1);
+                        }
+                }
+                if (lane == 0) tc_commit(freeb + 8 * (k % NS));
+                __syncwarp();
+            }
+            q += 2;  // the unit loaded L + 2 dY rows
+        }
+        if (lane == 0) {
+            tc_commit(done);  // every MMA issued has completed
+            if (!ok) tc_wait(done, 0);
+        }
+        __syncwarp();
+    } else {
+        // --------------------------------------------------- partial sums
+        const int dzi = warp & 3;  // accumulator lanes 32 dzi .. : (dz, ci = lane); the fourth group is not used
+        uint32_t w_ok = 1;
+        if (lane == 0) w_ok = ring_wait_long(done, 0, abort_flag);
+        w_ok = __shfl_sync(0xffffffffu, w_ok, 0);
+        fence_after();
+        if (w_ok && dzi < 3) {
+            float* P = r.partials + (long long)blockIdx.x * 27 * 32 * 32;
+#pragma unroll 1
+            for (int g = 0; g < 18; ++g) {  // 16 output channels of one (dx, dy)
+                const int dxi = g / 6, j = (g / 2) % 3, co = (g & 1) * 16;
+                uint32_t acc[16];
+                tmem_ld16(tmem + ((uint32_t)(dzi * 32) << 16) + dxi * 96 + j * 32 + co, acc);
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                const int t = 9 * dxi + 3 * (2 - j) + dzi;
+#pragma unroll
+                for (int c = 0; c < 16; ++c) P[(t * 32 + co + c) * 32 + lane] = __uint_as_float(acc[c]);
+            }
+        }
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    if (warp == 1)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(COLS) : "memory");
+}
+
 }  // namespace evxnn
 
 // =================================================================== host
@@ -592,16 +820,31 @@ PFN_cuTensorMapEncodeTiled_v12000 nn_encode_fn() {
 
 // activations [B X][Y][Z][32] as a 4D BF16 tensor (32 channels, Z, Y, B X), box 32 channels x zrows z,
 // written to shared memory in the 64-byte swizzle layout
-bool ring_map(CUtensorMap* m, const ConvArgs& a, int zrows) {
+bool act_map(CUtensorMap* m, const __nv_bfloat16* act, int B, int X, int Y, int Z, int zrows) {
     auto fn = nn_encode_fn();
-    if (!fn || ((uintptr_t)a.in & 15)) return false;
-    const cuuint64_t dims[4] = {32, (cuuint64_t)a.Z, (cuuint64_t)a.Y, (cuuint64_t)a.B * a.X};
-    const cuuint64_t strides[3] = {64, (cuuint64_t)a.Z * 64, (cuuint64_t)a.Y * a.Z * 64};
+    if (!fn || ((uintptr_t)act & 15)) return false;
+    const cuuint64_t dims[4] = {32, (cuuint64_t)Z, (cuuint64_t)Y, (cuuint64_t)B * X};
+    const cuuint64_t strides[3] = {64, (cuuint64_t)Z * 64, (cuuint64_t)Y * Z * 64};
     const cuuint32_t box[4] = {32, (cuuint32_t)zrows, 1, 1};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
-    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<__nv_bfloat16*>(a.in), dims, strides, box, estr,
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<__nv_bfloat16*>(act), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// segments of at least 8 rows that columns are split into: the split with the least
+// work on the busiest CTA, a segment of n rows costing n + extra
+int segments(long long ncol, int len, int ctas, int extra) {
+    int nseg = 1;
+    long long best = 0;
+    for (int s = 1; s == 1 || s <= len / 8; ++s) {
+        const long long rows = (ncol * s + ctas - 1) / ctas * ((len + s - 1) / s + extra);
+        if (s == 1 || rows < best) {
+            best = rows;
+            nseg = s;
+        }
+    }
+    return nseg;
 }
 
 template <int EPI>
@@ -611,21 +854,12 @@ cudaError_t launch_ring(const ConvArgs& a, cudaStream_t st, int sms) {
     r.nzc = (a.Z + ring::ZT - 1) / ring::ZT;
     r.zbox = a.Z % ring::ZT ? 64 : ring::ZT;
     CUtensorMap map, hmap;
-    if (!ring_map(&map, a, r.zbox) || !ring_map(&hmap, a, 16)) return cudaErrorInvalidValue;
+    if (!act_map(&map, a.in, a.B, a.X, a.Y, a.Z, r.zbox) || !act_map(&hmap, a.in, a.B, a.X, a.Y, a.Z, 16))
+        return cudaErrorInvalidValue;
     r.walkx = a.Z % ring::ZT != 0;
     r.len = r.walkx ? a.X : a.Y;
     const long long ncol = (long long)a.B * (r.walkx ? a.Y : a.X) * r.nzc;
-    // columns split into segments of at least 8 rows: the split with the fewest
-    // input rows on the busiest CTA (a segment of n rows walks n + 2)
-    int nseg = 1;
-    long long best = 0;
-    for (int s = 1; s == 1 || s <= r.len / 8; ++s) {
-        const long long rows = (ncol * s + sms - 1) / sms * ((r.len + s - 1) / s + 2);
-        if (s == 1 || rows < best) {
-            best = rows;
-            nseg = s;
-        }
-    }
+    const int nseg = segments(ncol, r.len, sms, 2);
     if (ncol * nseg > (1LL << 30)) return cudaErrorInvalidValue;  // unit index would overflow int
     r.nseg = nseg;
     r.nunits = (int)(ncol * nseg);
@@ -647,6 +881,28 @@ cudaError_t conv32_tc(const ConvArgs& a, int epilogue, cudaStream_t st, int sms)
         case EVX_NN_EPI_RESID32: return launch_ring<EVX_NN_EPI_RESID32>(a, st, sms);
     }
     return cudaErrorInvalidValue;
+}
+
+cudaError_t wgrad32_tc(const __nv_bfloat16* dy, const __nv_bfloat16* x, float* partials, int max_ctas, int B, int X, int Y,
+                       int Z, cudaStream_t st, int sms, int* ctas) {
+    WgArgs r{};
+    r.partials = partials;
+    r.B = B, r.X = X, r.Y = Y, r.Z = Z;
+    r.nzc = (Z + ring::ZT - 1) / ring::ZT;
+    r.zbox = Z % ring::ZT ? 64 : ring::ZT;
+    CUtensorMap xm, xh, dm;
+    if (!act_map(&xm, x, B, X, Y, Z, r.zbox) || !act_map(&xh, x, B, X, Y, Z, 16) || !act_map(&dm, dy, B, X, Y, Z, r.zbox))
+        return cudaErrorInvalidValue;
+    const int most = std::min(sms, max_ctas);
+    const long long ncol = (long long)B * X * r.nzc;
+    r.nseg = segments(ncol, Y, most, 1);
+    if (ncol * r.nseg > (1LL << 30)) return cudaErrorInvalidValue;  // unit index would overflow int
+    r.nunits = (int)(ncol * r.nseg);
+    *ctas = std::min(r.nunits, most);
+    cudaError_t e = cudaFuncSetAttribute(conv_wgrad_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, wg::SMEM);
+    if (e != cudaSuccess) return e;
+    conv_wgrad_tc_kernel<<<*ctas, wg::NTH, wg::SMEM, st>>>(xm, xh, dm, r);
+    return cudaGetLastError();
 }
 
 cudaError_t tc_take_timeout(int* flag) {
