@@ -273,9 +273,7 @@ constexpr long long WAIT_BUDGET = 1LL << 31;
 struct RingArgs {
     ConvArgs a;
     int nzc;     // z chunks: ceil(Z / 128), the last of 64 voxels when Z is an odd multiple of 64
-    int zbox;    // z rows of the main TMA box: 128, or 64 when there is a 64-voxel chunk
-    int walkx;   // 0: columns (b, x, z chunk) walked along y; 1: columns (b, y, z chunk) walked along x
-    int len;     // rows of a column (Y or X)
+    int len;     // rows of a column: Y (columns (b, x, z chunk) walked along y) or X (columns (b, y, z chunk))
     int nseg;    // segments of a column
     int nunits;  // columns * nseg
 };
@@ -353,7 +351,9 @@ __device__ __forceinline__ void tmem_st16_zero(uint32_t taddr) {
         : "memory");
 }
 
-template <int EPI>
+// WX: columns are walked along x and may end in a 64-voxel chunk (a template parameter: as
+// run-time values the two forms cost the Z % 128 = 0 convolutions 4 to 9%)
+template <int EPI, bool WX>
 __global__ void __launch_bounds__(ring::NTH, 1)
     conv_ring_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap hmap, RingArgs r) {
     using namespace ring;
@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(ring::NTH, 1)
     // x and y change places)
     for (int e = threadIdx.x; e < 9 * 96 * 4; e += NTH) {
         const int kg = e & 3, n = (e >> 2) % 96, dd = e / (96 * 4), dxi = dd / 3, dzi = dd % 3;
-        const int t = r.walkx ? 9 * (n >> 5) + 3 * dxi + dzi : 9 * dxi + 3 * (n >> 5) + dzi, co = n & 31;
+        const int t = WX ? 9 * (n >> 5) + 3 * dxi + dzi : 9 * dxi + 3 * (n >> 5) + dzi, co = n & 31;
         const uint4 v = *reinterpret_cast<const uint4*>(a.w + (t * 32 + co) * 32 + kg * 8);
         *reinterpret_cast<uint4*>(swb + (((dd * 12 + (n >> 3)) * 4 + kg) * 8 + (n & 7)) * 16) = v;
     }
@@ -417,8 +417,8 @@ __global__ void __launch_bounds__(ring::NTH, 1)
         for (int u = blockIdx.x; u < r.nunits && ok; u += gridDim.x) {
             int bx, z0, ys, ye;
             ring_unit(r, u, bx, z0, ys, ye);
-            const int across = r.walkx ? Y : X, b = bx / across, x = bx - b * across;
-            const int nz = min(ZT, Z - z0);  // 128, or 64 in a last half chunk (its rows 64 .. are not loaded)
+            const int across = WX ? Y : X, b = bx / across, x = bx - b * across;
+            const int nz = WX ? min(ZT, Z - z0) : ZT;  // 128, or 64 in a last half chunk (its rows 64 .. are not loaded)
             for (int j = -1; j <= ye - ys; ++j) {
                 const int yp = (ys + j + r.len) % r.len;
                 const uint32_t slot = k % NS;
@@ -437,10 +437,10 @@ __global__ void __launch_bounds__(ring::NTH, 1)
 #pragma unroll
                     for (int dxi = 0; dxi < 3; ++dxi) {
                         const int side = (x + dxi - 1 + across) % across;
-                        const int cy = r.walkx ? side : yp, cx = b * X + (r.walkx ? yp : side);
+                        const int cy = WX ? side : yp, cx = b * X + (WX ? yp : side);
                         const uint32_t run = base + dxi * RUN;
                         tma_load4(run + 16 * 64, &map, 0, z0, cy, cx, full + 8 * slot);
-                        if (nz > r.zbox) tma_load4(run + (16 + 64) * 64, &map, 0, z0 + 64, cy, cx, full + 8 * slot);
+                        if (WX && nz == ZT) tma_load4(run + (16 + 64) * 64, &map, 0, z0 + 64, cy, cx, full + 8 * slot);
                         tma_load4(run, &hmap, 0, zl, cy, cx, full + 8 * slot);
                         tma_load4(run + (16 + nz) * 64, &hmap, 0, zr, cy, cx, full + 8 * slot);
                     }
@@ -545,7 +545,11 @@ __global__ void __launch_bounds__(ring::NTH, 1)
             int bx, z0, ys, ye;
             ring_unit(r, u, bx, z0, ys, ye);
             const int L = ye - ys;
-            for (int jv = 0; jv < L + 4; ++jv, ++v) {
+            // voxel of the row's lane 0 and the distance to the next row's
+            const long long row0 = WX ? ((long long)(bx / Y) * X + ys) * Y + bx % Y : (long long)bx * Y + ys;
+            const long long step = WX ? (long long)Y * Z : Z;
+            long long vox0 = row0 * Z + z0 + q4 * 32 - 2 * step;  // of virtual row jv = 0
+            for (int jv = 0; jv < L + 4; ++jv, ++v, vox0 += step) {
                 const uint32_t blk = ring_blk(v);
                 uint32_t w_ok = 1;
                 if (lane == 0) w_ok = ring_wait(tfull + 8 * blk, (v / NBLK) & 1, abort_flag);
@@ -563,10 +567,7 @@ __global__ void __launch_bounds__(ring::NTH, 1)
                 fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(tempty + 8 * blk);
-                if (jv >= 2 && jv < L + 2 && z0 + q4 * 32 < Z) {  // a half chunk's lanes 64 .. are not voxels
-                    const int o = ys + jv - 2;
-                    const long long line = r.walkx ? ((long long)(bx / Y) * X + o) * Y + bx % Y : (long long)bx * Y + o;
-                    const long long vox0 = line * Z + z0 + q4 * 32;
+                if (jv >= 2 && jv < L + 2 && (!WX || z0 + q4 * 32 < Z)) {  // a half chunk's lanes 64 .. are not voxels
                     if (EPI == EVX_NN_EPI_RESID32)
                         resid32_staged(a, vox0, h * 16, acc, bias, stg, lane);
                     else
@@ -847,26 +848,30 @@ int segments(long long ncol, int len, int ctas, int extra) {
     return nseg;
 }
 
-template <int EPI>
-cudaError_t launch_ring(const ConvArgs& a, cudaStream_t st, int sms) {
+template <int EPI, bool WX>
+cudaError_t launch_walk(const ConvArgs& a, cudaStream_t st, int sms) {
     RingArgs r{};
     r.a = a;
     r.nzc = (a.Z + ring::ZT - 1) / ring::ZT;
-    r.zbox = a.Z % ring::ZT ? 64 : ring::ZT;
-    CUtensorMap map, hmap;
-    if (!act_map(&map, a.in, a.B, a.X, a.Y, a.Z, r.zbox) || !act_map(&hmap, a.in, a.B, a.X, a.Y, a.Z, 16))
+    CUtensorMap map, hmap;  // with a half chunk the main box has 64 rows
+    if (!act_map(&map, a.in, a.B, a.X, a.Y, a.Z, WX ? 64 : ring::ZT) || !act_map(&hmap, a.in, a.B, a.X, a.Y, a.Z, 16))
         return cudaErrorInvalidValue;
-    r.walkx = a.Z % ring::ZT != 0;
-    r.len = r.walkx ? a.X : a.Y;
-    const long long ncol = (long long)a.B * (r.walkx ? a.Y : a.X) * r.nzc;
+    r.len = WX ? a.X : a.Y;
+    const long long ncol = (long long)a.B * (WX ? a.Y : a.X) * r.nzc;
     const int nseg = segments(ncol, r.len, sms, 2);
     if (ncol * nseg > (1LL << 30)) return cudaErrorInvalidValue;  // unit index would overflow int
     r.nseg = nseg;
     r.nunits = (int)(ncol * nseg);
-    cudaError_t e = cudaFuncSetAttribute(conv_ring_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, ring::SMEM);
+    cudaError_t e =
+        cudaFuncSetAttribute(conv_ring_kernel<EPI, WX>, cudaFuncAttributeMaxDynamicSharedMemorySize, ring::SMEM);
     if (e != cudaSuccess) return e;
-    conv_ring_kernel<EPI><<<std::min(r.nunits, sms), ring::NTH, ring::SMEM, st>>>(map, hmap, r);
+    conv_ring_kernel<EPI, WX><<<std::min(r.nunits, sms), ring::NTH, ring::SMEM, st>>>(map, hmap, r);
     return cudaGetLastError();
+}
+
+template <int EPI>
+cudaError_t launch_ring(const ConvArgs& a, cudaStream_t st, int sms) {
+    return a.Z % ring::ZT ? launch_walk<EPI, true>(a, st, sms) : launch_walk<EPI, false>(a, st, sms);
 }
 }  // namespace
 
