@@ -226,12 +226,80 @@ __global__ void __launch_bounds__(NTHR) conv_wgrad_kernel(WgradArgs a) {
     }
 }
 
-// out[i] = sum_b partials[b * n + i] in order b = 0, 1, ... (deterministic)
-__global__ void reduce_partials_f32(const float* partials, int nparts, int n, float* out) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        double s = 0.0;
-        for (int b = 0; b < nparts; ++b) s += partials[(long long)b * n + i];
-        out[i] = (float)s;
+// ------------------------------------------------------- sums in fixed order
+// GB300's FP64 pipe does two operations per SM and clock, so long sums run as
+// FP32 pairs: TwoSum keeps the rounded sum s and the sum e of its exact rounding
+// errors (Knuth), which together hold the FP64 sum to about 2^-44 over the few
+// dozen values between two additions to an FP64 accumulator.
+// Values whose sums or products leave FP32's range (HUGE_VALUE and the limits at each
+// use; infinities among them) are added in FP64 as they come; NaN passes through s.
+constexpr float HUGE_VALUE = 0x1p100f;
+constexpr int SUM_NT = 256;  // threads of the CTAs that stream a field (512 were slower below 2^24 values)
+struct Sum2 {
+    float s = 0.f, e = 0.f;
+    __device__ __forceinline__ void add(float x) {
+        const float t = s + x, bp = t - s;
+        e += (s - (t - bp)) + (x - bp);
+        s = t;
+    }
+    __device__ __forceinline__ void add2(float hi, float lo) {
+        add(hi);
+        e += lo;
+    }
+    __device__ __forceinline__ double take() {
+        const double v = (double)s + (double)e;
+        s = e = 0.f;
+        return v;
+    }
+};
+// sum over the CTA (a multiple of 32 threads, at most 1024) in a fixed order; every thread gets it
+__device__ __forceinline__ double cta_sum(double v) {
+    __shared__ double ws[32], total;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    __syncthreads();  // an earlier call's ws and total have been read
+    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        v = threadIdx.x < (blockDim.x >> 5) ? ws[threadIdx.x] : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (threadIdx.x == 0) total = v;
+    }
+    __syncthreads();
+    return total;
+}
+__device__ __forceinline__ double cta_sum_partials(const double* p, int n) {
+    double v = 0.0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) v += p[i];
+    return cta_sum(v);
+}
+
+// out[i] = sum_b partials[b * n + i]: 8 threads per output, each every 8th partial, in a
+// fixed order (one thread per output walked 152 to 304 dependent loads: 30 us for
+// 27 x 1024 outputs of 152 partials, 11 us this way)
+__global__ void __launch_bounds__(256) reduce_partials_f32(const float* partials, int nparts, int n, float* out) {
+    __shared__ double ws[8][33];
+    const int i = blockIdx.x * 32 + (threadIdx.x & 31), slice = threadIdx.x >> 5;
+    double acc = 0.0;
+    if (i < n) {
+        for (int b = slice; b < nparts; b += 8 * 16) {  // 16 loads in flight
+            float v[16];
+#pragma unroll
+            for (int u = 0; u < 16; ++u) v[u] = b + 8 * u < nparts ? partials[(long long)(b + 8 * u) * n + i] : 0.f;
+            Sum2 t;
+#pragma unroll
+            for (int u = 0; u < 16; ++u) t.add(v[u]);
+            acc += t.take();
+        }
+    }
+    ws[slice][threadIdx.x & 31] = acc;
+    __syncthreads();
+    if (slice == 0 && i < n) {
+        double v = 0.0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v += ws[q][threadIdx.x & 31];
+        out[i] = (float)v;
     }
 }
 
@@ -255,7 +323,7 @@ __global__ void bias_grad_kernel(const __nv_bfloat16* dy, long long nvox, int C,
     }
 }
 // One pass for all channels (C = 16 or 32): C / 8 threads per voxel, each summing
-// 8 channels from 16-byte loads (four voxels in flight), FP32 over 32 voxels at a
+// 8 channels from 16-byte loads (eight voxels in flight), FP32 over 32 voxels at a
 // time and FP64 beyond;
 // the CTA then adds its threads' sums per channel in a fixed order.
 template <int C>
@@ -269,17 +337,17 @@ __global__ void __launch_bounds__(256) bias_grad_vec_kernel(const __nv_bfloat16*
     float part[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) acc[k] = 0.0, part[k] = 0.f;
-    // four voxels in flight per thread per round; FP32 over 8 rounds, then FP64
+    // eight voxels in flight per thread per round; FP32 over 4 rounds, then FP64
     int cnt = 0;
-    for (long long v = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / TPV; v < nvox; v += 4 * stride) {
-        uint4 q[4];
+    for (long long v = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / TPV; v < nvox; v += 8 * stride) {
+        uint4 q[8];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < 8; ++u) {
             const long long vu = v + u * stride;
             q[u] = vu < nvox ? *reinterpret_cast<const uint4*>(dy + vu * C + 8 * piece) : make_uint4(0, 0, 0, 0);
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < 8; ++u) {
             const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&q[u]);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -288,7 +356,7 @@ __global__ void __launch_bounds__(256) bias_grad_vec_kernel(const __nv_bfloat16*
                 part[2 * j + 1] += f.y;
             }
         }
-        if (++cnt == 8) {
+        if (++cnt == 4) {
 #pragma unroll
             for (int k = 0; k < 8; ++k) acc[k] += part[k], part[k] = 0.f;
             cnt = 0;
@@ -297,20 +365,24 @@ __global__ void __launch_bounds__(256) bias_grad_vec_kernel(const __nv_bfloat16*
 #pragma unroll
     for (int k = 0; k < 8; ++k) red[threadIdx.x][k] = acc[k] + part[k];
     __syncthreads();
-    if (threadIdx.x < C) {
-        const int pc = threadIdx.x / 8, j = threadIdx.x % 8;
-        double s = 0.0;
-        for (int t = pc; t < (int)blockDim.x; t += TPV) s += red[t][j];
-        partials[(long long)blockIdx.x * C + threadIdx.x] = s;
-    }
+    // channel ch = (piece pc, j): 256 / C threads add every (256 / C)-th of its values, then shuffles
+    constexpr int TPC = 256 / C;
+    const int ch = threadIdx.x / TPC, q = threadIdx.x % TPC;
+    double s = 0.0;
+    for (int t = ch / 8 + TPV * q; t < 256; t += TPV * TPC) s += red[t][ch % 8];
+#pragma unroll
+    for (int o = TPC / 2; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o, TPC);
+    if (q == 0) partials[(long long)blockIdx.x * C + ch] = s;
 }
 
-__global__ void bias_grad_finish(const double* partials, int nparts, int C, float* db) {
-    const int co = threadIdx.x;
-    if (co < C) {
+// a warp per channel (one thread per channel: 28 us for 304 partials)
+__global__ void __launch_bounds__(1024) bias_grad_finish(const double* partials, int nparts, int C, float* db) {
+    for (int co = threadIdx.x >> 5; co < C; co += 32) {
         double s = 0.0;
-        for (int b = 0; b < nparts; ++b) s += partials[b * C + co];
-        db[co] = (float)s;
+        for (int b = threadIdx.x & 31; b < nparts; b += 32) s += partials[(long long)b * C + co];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if ((threadIdx.x & 31) == 0) db[co] = (float)s;
     }
 }
 
@@ -322,119 +394,225 @@ __global__ void field_to_act_kernel(const float* f, long long nvox, int C, float
     }
 }
 
-// per-sample FP64 sums of a field: partials[s * nb + blk]
-__global__ void sample_sum_kernel(const float* f, long long V, double* partials, int nb) {
-    __shared__ double ws[256];
-    const int s = blockIdx.y;
-    double acc = 0.0;
-    for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < V;
-         v += (long long)gridDim.x * blockDim.x)
-        acc += (double)f[s * V + v];
-    ws[threadIdx.x] = acc;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) ws[threadIdx.x] += ws[threadIdx.x + o];
-        __syncthreads();
+// the same with 16-byte stores, C a multiple of 8 and act 16-byte aligned: a thread per
+// piece of 8 channels (2-byte stores took 104 us for 4 x 64^3 voxels of 16 channels, 9 us now)
+__global__ void __launch_bounds__(256) field_to_act_vec_kernel(const float* __restrict__ f, long long nvox, int pieces,
+                                                               float scale, uint4* __restrict__ act) {
+    const long long n = nvox * pieces;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        const long long v = i / pieces;
+        uint4 q = make_uint4(0, 0, 0, 0);
+        if (v * pieces == i) q.x = __bfloat16_as_ushort(__float2bfloat16_rn(f[v] * scale));
+        act[i] = q;
     }
-    if (threadIdx.x == 0) partials[s * nb + blockIdx.x] = ws[0];
 }
 
-// out = base + (d - mean_s(d)) per sample (base may be null: out = d - mean)
-__global__ void zero_mean_add_kernel(const float* base, const float* d, const double* partials, int nb, long long V,
-                                     float* out, const double* scale) {
-    const int s = blockIdx.y;
-    double m = 0.0;
-    for (int b = 0; b < nb; ++b) m += partials[s * nb + b];
-    const float mean = (float)(m / (double)V);
-    const float f = scale ? (float)scale[s] : 1.f;
-    for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < V;
-         v += (long long)gridDim.x * blockDim.x) {
-        const float x = f * (d[s * V + v] - mean);
-        out[s * V + v] = base ? base[s * V + v] + x : x;
+// f(v, i) for the V values of x that a thread of a grid-stride loop visits: arrays v of 4
+// values i .. i + 3 where x is 16-byte aligned (eight loads in flight), of one value in the
+// rest; flush() after at most 32 values
+template <typename F, typename Flush>
+__device__ __forceinline__ void for_values(const float* __restrict__ x, long long V, F&& f, Flush&& flush) {
+    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x, nt = (long long)gridDim.x * blockDim.x;
+    const bool vec = ((uintptr_t)x & 15) == 0;
+    const long long nv = vec ? V / 4 : 0;
+    const float4* x4 = reinterpret_cast<const float4*>(x);
+    for (long long i = t; i < nv; i += 8 * nt) {
+        float4 q[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (i + u * nt < nv) q[u] = x4[i + u * nt];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (i + u * nt < nv) {
+                const float v[4] = {q[u].x, q[u].y, q[u].z, q[u].w};
+                f(v, 4 * (i + u * nt));
+            }
+        flush();
     }
+    for (long long i = 4 * nv + t; i < V; i += nt) {
+        const float v[1] = {x[i]};
+        f(v, i);
+        flush();
+    }
+}
+// the values' magnitudes: none above `most`, none but zero below `least` (NaN counts as inside)
+template <int N>
+__device__ __forceinline__ bool in_range(const float (&v)[N], float least, float most) {
+    bool out = false;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const float m = fabsf(v[i]);
+        out |= m > most || (m < least && m != 0.f);
+    }
+    return !out;
+}
+
+// per-sample FP64 sums of a field: partials[s * nb + blk]
+__global__ void __launch_bounds__(SUM_NT) sample_sum_kernel(const float* f, long long V, double* partials, int nb) {
+    const int s = blockIdx.y;
+    double acc = 0.0;
+    Sum2 t;
+    for_values(
+        f + s * V, V,
+        [&](const auto& v, long long) {
+            if (in_range(v, 0.f, HUGE_VALUE))
+                for (float x : v) t.add(x);
+            else
+                for (float x : v) acc += (double)x;
+        },
+        [&] { acc += t.take(); });
+    acc = cta_sum(acc);
+    if (threadIdx.x == 0) partials[s * nb + blockIdx.x] = acc;
+}
+
+// out = base + (d - mean_s(d)) per sample (base may be null: out = d - mean); the mean is
+// summed once per CTA (every thread summing the partials itself made the pass 190 us at
+// 4 x 64^3, bound by the FP64 pipe; 14 us now)
+__global__ void __launch_bounds__(SUM_NT) zero_mean_add_kernel(const float* base, const float* d, const double* partials,
+                                                            int nb, long long V, float* out, const double* scale) {
+    const int s = blockIdx.y;
+    const float mean = (float)(cta_sum_partials(partials + s * nb, nb) / (double)V);
+    const float f = scale ? (float)scale[s] : 1.f;
+    const float *ds = d + s * V, *bs = base ? base + s * V : nullptr;
+    float* os = out + s * V;
+    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x, nt = (long long)gridDim.x * blockDim.x;
+    const bool vec = (((uintptr_t)ds | (uintptr_t)bs | (uintptr_t)os) & 15) == 0;
+    const long long nv = vec ? V / 4 : 0;
+    for (long long i = t; i < nv; i += nt) {
+        const float4 q = reinterpret_cast<const float4*>(ds)[i];
+        float4 x = make_float4(f * (q.x - mean), f * (q.y - mean), f * (q.z - mean), f * (q.w - mean));
+        if (bs) {
+            const float4 c = reinterpret_cast<const float4*>(bs)[i];
+            x = make_float4(fmaf(f, q.x - mean, c.x), fmaf(f, q.y - mean, c.y), fmaf(f, q.z - mean, c.z),
+                            fmaf(f, q.w - mean, c.w));
+        }
+        reinterpret_cast<float4*>(os)[i] = x;
+    }
+    for (long long v = 4 * nv + t; v < V; v += nt) os[v] = bs ? fmaf(f, ds[v] - mean, bs[v]) : f * (ds[v] - mean);
+}
+
+// product of two FP32 pairs (hi + lo, |lo| <= ulp(hi) / 2), relative error about 2^-46
+__device__ __forceinline__ float2 mul22(float2 a, float2 b) {
+    const float p = a.x * b.x;
+    return make_float2(p, fmaf(a.x, b.x, -p) + fmaf(a.x, b.y, a.y * b.x));
+}
+__device__ __forceinline__ float2 two_sum(float a, float b) {
+    const float t = a + b, bp = t - a;
+    return make_float2(t, (a - (t - bp)) + (b - bp));
 }
 
 // Per sample s and block b: with the sample's FP64 mean m (from the partial sums
 // pm), partial FP64 sums of d^2 and N^2, d = x - m, N = d^2 (3 m + d) (the
 // nonlinear remainder of c^3 - c about the mean): out[(s * 2 + 0|1) * nb + b].
-__global__ void nl_moments_kernel(const float* x, long long V, const double* pm, int nb, double* out) {
-    __shared__ double ws[2][256];
+// In FP32 pairs: seven FP64 operations per value and the mean summed by every
+// thread made it 205 us at 4 x 64^3 and 2.1 ms at 8 x 256^3 (31 us and 0.30 ms now).
+// A quad of values any of which leaves the range of the pairs is added in FP64.
+__global__ void __launch_bounds__(SUM_NT) nl_moments_kernel(const float* x, long long V, const double* pm, int nb,
+                                                         double* out) {
     const int s = blockIdx.y;
-    double m = 0.0;
-    for (int b = 0; b < nb; ++b) m += pm[s * nb + b];
-    m /= (double)V;
+    const double m = cta_sum_partials(pm + s * nb, nb) / (double)V, m3 = 3.0 * m;
+    const float mh = (float)m, ml = (float)(m - (double)mh), th = (float)m3, tl = (float)(m3 - (double)th);
+    constexpr float UP = 0x1p14f;  // N^2 is formed as (2^42 N)^2: its low part stays a normal number
+    constexpr double DOWN = 0x1p-84;
     double a2 = 0.0, n2 = 0.0;
-    for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < V; v += (long long)gridDim.x * blockDim.x) {
-        const double d = (double)x[s * V + v] - m;
-        const double N = d * d * (3.0 * m + d);
-        a2 += d * d;
-        n2 += N * N;
-    }
-    ws[0][threadIdx.x] = a2;
-    ws[1][threadIdx.x] = n2;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) {
-            ws[0][threadIdx.x] += ws[0][threadIdx.x + o];
-            ws[1][threadIdx.x] += ws[1][threadIdx.x + o];
-        }
-        __syncthreads();
-    }
+    Sum2 sa, sn;
+    for_values(
+        x + s * V, V,
+        [&](const auto& v, long long) {
+            constexpr int N = sizeof(v) / sizeof(float);
+            float2 d[N];
+            float mag[N];
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                d[i] = two_sum(v[i], -mh);
+                d[i] = two_sum(d[i].x, d[i].y - ml);
+                mag[i] = d[i].x;
+            }
+            if (!in_range(mag, 0x1p-30f, 8.f)) {
+                for (float x : v) {
+                    const double dd = (double)x - m, R = dd * dd * (m3 + dd);
+                    a2 += dd * dd;
+                    n2 += R * R * 0x1p84;
+                }
+                return;
+            }
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                const float2 q = mul22(d[i], d[i]);
+                float2 c = two_sum(th, d[i].x);  // 3 m + d
+                c = two_sum(c.x, c.y + (tl + d[i].y));
+                const float2 qs = make_float2(q.x * (UP * UP), q.y * (UP * UP)), cs = make_float2(c.x * UP, c.y * UP);
+                const float2 R = mul22(qs, cs), w = mul22(R, R);
+                sa.add2(q.x, q.y);
+                sn.add2(w.x, w.y);
+            }
+        },
+        [&] {
+            a2 += sa.take();
+            n2 += sn.take();
+        });
+    a2 = cta_sum(a2);
+    n2 = cta_sum(n2) * DOWN;
     if (threadIdx.x == 0) {
-        out[(s * 2 + 0) * nb + blockIdx.x] = ws[0][0];
-        out[(s * 2 + 1) * nb + blockIdx.x] = ws[1][0];
+        out[(s * 2 + 0) * nb + blockIdx.x] = a2;
+        out[(s * 2 + 1) * nb + blockIdx.x] = n2;
     }
 }
-// scale[s] = min(1, sqrt(sum N^2 / sum d^2)) (0 for a uniform sample), fixed order
-__global__ void nl_scale_kernel(const double* mom, int nb, int nsamples, double* scale) {
-    const int s = threadIdx.x;
-    if (s >= nsamples || blockIdx.x != 0) return;
-    double a2 = 0.0, n2 = 0.0;
-    for (int b = 0; b < nb; ++b) {
-        a2 += mom[(s * 2 + 0) * nb + b];
-        n2 += mom[(s * 2 + 1) * nb + b];
-    }
-    scale[s] = a2 > 0.0 ? fmin(1.0, sqrt(n2 / a2)) : 0.0;
+// scale[s] = min(1, sqrt(sum N^2 / sum d^2)) (0 for a uniform sample), fixed order; a CTA per sample
+__global__ void __launch_bounds__(256) nl_scale_kernel(const double* mom, int nb, double* scale) {
+    const int s = blockIdx.x;
+    const double a2 = cta_sum_partials(mom + (s * 2 + 0) * nb, nb), n2 = cta_sum_partials(mom + (s * 2 + 1) * nb, nb);
+    if (threadIdx.x == 0) scale[s] = a2 > 0.0 ? fmin(1.0, sqrt(n2 / a2)) : 0.0;
 }
 
-// squared error: partials of sum (p - t)^2 (FP64); grad = scale (p - t)
-__global__ void mse_kernel(const float* p, const float* t, long long n, float scale, float* grad, double* partials) {
-    __shared__ double ws[256];
+// squared error: partials of sum (p - t)^2 (the product exact as an FP32 pair); grad = scale (p - t)
+__global__ void __launch_bounds__(SUM_NT) mse_kernel(const float* p, const float* t, long long n, float scale, float* grad,
+                                                  double* partials) {
     double acc = 0.0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        const float d = p[i] - t[i];
-        acc += (double)d * d;
-        if (grad) grad[i] = scale * d;
-    }
-    ws[threadIdx.x] = acc;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) ws[threadIdx.x] += ws[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) partials[blockIdx.x] = ws[0];
+    Sum2 sq;
+    for_values(
+        p, n,
+        [&](const auto& v, long long i) {
+            constexpr int N = sizeof(v) / sizeof(float);
+            float d[N];
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                d[j] = v[j] - t[i + j];
+                if (grad) grad[i + j] = scale * d[j];
+            }
+            if (in_range(d, 0x1p-40f, 0x1p50f)) {
+#pragma unroll
+                for (int j = 0; j < N; ++j) {
+                    const float q = d[j] * d[j];
+                    sq.add2(q, fmaf(d[j], d[j], -q));
+                }
+            } else {
+                for (float x : d) acc += (double)x * x;
+            }
+        },
+        [&] { acc += sq.take(); });
+    acc = cta_sum(acc);
+    if (threadIdx.x == 0) partials[blockIdx.x] = acc;
 }
 // partials[b] = FP64 sum of |x| over a grid-stride share of the n values
-__global__ void abs_sum_kernel(const float* x, long long n, double* partials) {
-    __shared__ double ws[256];
+__global__ void __launch_bounds__(SUM_NT) abs_sum_kernel(const float* x, long long n, double* partials) {
     double acc = 0.0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        acc += fabs((double)x[i]);
-    ws[threadIdx.x] = acc;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) ws[threadIdx.x] += ws[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) partials[blockIdx.x] = ws[0];
+    Sum2 t;
+    for_values(
+        x, n,
+        [&](const auto& v, long long) {
+            if (in_range(v, 0.f, HUGE_VALUE))
+                for (float y : v) t.add(fabsf(y));
+            else
+                for (float y : v) acc += fabs((double)y);
+        },
+        [&] { acc += t.take(); });
+    acc = cta_sum(acc);
+    if (threadIdx.x == 0) partials[blockIdx.x] = acc;
 }
-__global__ void sum_partials_kernel(const double* partials, int n, double* out) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double s = 0.0;
-        for (int i = 0; i < n; ++i) s += partials[i];
-        *out = s;
-    }
+__global__ void __launch_bounds__(256) sum_partials_kernel(const double* partials, int n, double* out) {
+    const double s = cta_sum_partials(partials, n);
+    if (threadIdx.x == 0) *out = s;
 }
 
 // dgrad weights: Wt[26 - t][ci][co] = W[t][co][ci] (BF16)
@@ -836,7 +1014,7 @@ evx_status launch_wgrad(const WgradArgs& a0, float* dw, float* partials, size_t 
         cudaError_t e = wgrad32_tc(a0.dy, a0.x, partials, (int)std::min<size_t>(partial_floats / (27 * 1024), 1 << 20), a0.B,
                                    a0.X, a0.Y, a0.Z, st, nn_sms(), &ctas);
         if (e != cudaSuccess) return nn_cuda(e);
-        reduce_partials_f32<<<108, 256, 0, st>>>(partials, ctas, 27 * 1024, dw);
+        reduce_partials_f32<<<27 * 32, 256, 0, st>>>(partials, ctas, 27 * 1024, dw);
         return nn_cuda(cudaGetLastError());
     }
     WgradArgs a = a0;
@@ -853,7 +1031,7 @@ evx_status launch_wgrad(const WgradArgs& a0, float* dw, float* partials, size_t 
     a.partials = partials;
     conv_wgrad_kernel<CIN, COUT><<<grid, NTHR, smem, st>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return nn_cuda(e);
-    reduce_partials_f32<<<(int)((per_cta + 255) / 256), 256, 0, st>>>(partials, grid, (int)per_cta, dw);
+    reduce_partials_f32<<<(int)((per_cta + 31) / 32), 256, 0, st>>>(partials, grid, (int)per_cta, dw);
     return nn_cuda(cudaGetLastError());
 }
 
@@ -1006,7 +1184,7 @@ evx_status evx_nn_bias_grad(const void* dy, long long nvox, int c, double* parti
         bias_grad_vec_kernel<16><<<nparts, 256, 0, st>>>((const __nv_bfloat16*)dy, nvox, partials);
     else
         bias_grad_kernel<<<nparts, 256, 0, st>>>((const __nv_bfloat16*)dy, nvox, c, partials);
-    bias_grad_finish<<<1, 256, 0, st>>>(partials, nparts, c, db);
+    bias_grad_finish<<<1, 1024, 0, st>>>(partials, nparts, c, db);
     return nn_cuda(cudaGetLastError());
 }
 
@@ -1019,7 +1197,10 @@ evx_status evx_nn_flip_weights(const void* w, int cout, int cin, void* wt, void*
 
 evx_status evx_nn_field_to_act(const float* f, long long nvox, int c, float scale, void* act, void* stream) {
     if (!f || !act || c <= 0) return nn_fail(EVX_ERR_ARG, "bad argument");
-    field_to_act_kernel<<<4 * nn_sms(), 256, 0, (cudaStream_t)stream>>>(f, nvox, c, scale, (__nv_bfloat16*)act);
+    if (c % 8 == 0 && ((uintptr_t)act & 15) == 0)
+        field_to_act_vec_kernel<<<8 * nn_sms(), 256, 0, (cudaStream_t)stream>>>(f, nvox, c / 8, scale, (uint4*)act);
+    else
+        field_to_act_kernel<<<4 * nn_sms(), 256, 0, (cudaStream_t)stream>>>(f, nvox, c, scale, (__nv_bfloat16*)act);
     return nn_cuda(cudaGetLastError());
 }
 
@@ -1028,8 +1209,8 @@ evx_status evx_nn_zero_mean_add(const float* base, const float* d, int nsamples,
     if (!d || !out || !partials || nsamples <= 0 || nparts <= 0 || nparts > 4096)
         return nn_fail(EVX_ERR_ARG, "bad argument");
     cudaStream_t st = (cudaStream_t)stream;
-    sample_sum_kernel<<<dim3(nparts, nsamples), 256, 0, st>>>(d, V, partials, nparts);
-    zero_mean_add_kernel<<<dim3(nparts, nsamples), 256, 0, st>>>(base, d, partials, nparts, V, out, nullptr);
+    sample_sum_kernel<<<dim3(nparts, nsamples), SUM_NT, 0, st>>>(d, V, partials, nparts);
+    zero_mean_add_kernel<<<dim3(nparts, nsamples), SUM_NT, 0, st>>>(base, d, partials, nparts, V, out, nullptr);
     return nn_cuda(cudaGetLastError());
 }
 
@@ -1038,8 +1219,8 @@ evx_status evx_nn_zero_mean_add_scaled(const float* base, const float* d, const 
     if (!d || !out || !partials || !scale || nsamples <= 0 || nparts <= 0 || nparts > 4096)
         return nn_fail(EVX_ERR_ARG, "bad argument");
     cudaStream_t st = (cudaStream_t)stream;
-    sample_sum_kernel<<<dim3(nparts, nsamples), 256, 0, st>>>(d, V, partials, nparts);
-    zero_mean_add_kernel<<<dim3(nparts, nsamples), 256, 0, st>>>(base, d, partials, nparts, V, out, scale);
+    sample_sum_kernel<<<dim3(nparts, nsamples), SUM_NT, 0, st>>>(d, V, partials, nparts);
+    zero_mean_add_kernel<<<dim3(nparts, nsamples), SUM_NT, 0, st>>>(base, d, partials, nparts, V, out, scale);
     return nn_cuda(cudaGetLastError());
 }
 
@@ -1048,9 +1229,9 @@ evx_status evx_nn_nl_scale(const float* c, int nsamples, long long V, double* pa
     if (!c || !partials || !scale || nsamples <= 0 || nsamples > 32 || V <= 0 || nparts <= 0 || nparts > 4096)
         return nn_fail(EVX_ERR_ARG, "bad argument");
     cudaStream_t st = (cudaStream_t)stream;
-    sample_sum_kernel<<<dim3(nparts, nsamples), 256, 0, st>>>(c, V, partials, nparts);
-    nl_moments_kernel<<<dim3(nparts, nsamples), 256, 0, st>>>(c, V, partials, nparts, partials + (long long)nsamples * nparts);
-    nl_scale_kernel<<<1, 32, 0, st>>>(partials + (long long)nsamples * nparts, nparts, nsamples, scale);
+    sample_sum_kernel<<<dim3(nparts, nsamples), SUM_NT, 0, st>>>(c, V, partials, nparts);
+    nl_moments_kernel<<<dim3(nparts, nsamples), SUM_NT, 0, st>>>(c, V, partials, nparts, partials + (long long)nsamples * nparts);
+    nl_scale_kernel<<<nsamples, 256, 0, st>>>(partials + (long long)nsamples * nparts, nparts, scale);
     return nn_cuda(cudaGetLastError());
 }
 
@@ -1058,16 +1239,16 @@ evx_status evx_nn_mse(const float* p, const float* t, long long n, float grad_sc
                       int nparts, double* d_sum, void* stream) {
     if (!p || !t || !partials || !d_sum || nparts <= 0) return nn_fail(EVX_ERR_ARG, "bad argument");
     cudaStream_t st = (cudaStream_t)stream;
-    mse_kernel<<<nparts, 256, 0, st>>>(p, t, n, grad_scale, grad, partials);
-    sum_partials_kernel<<<1, 32, 0, st>>>(partials, nparts, d_sum);
+    mse_kernel<<<nparts, SUM_NT, 0, st>>>(p, t, n, grad_scale, grad, partials);
+    sum_partials_kernel<<<1, 256, 0, st>>>(partials, nparts, d_sum);
     return nn_cuda(cudaGetLastError());
 }
 
 evx_status evx_nn_abs_sum(const float* x, long long n, double* partials, int nparts, double* d_sum, void* stream) {
     if (!x || n <= 0 || !partials || !d_sum || nparts <= 0) return nn_fail(EVX_ERR_ARG, "bad argument");
     cudaStream_t st = (cudaStream_t)stream;
-    abs_sum_kernel<<<nparts, 256, 0, st>>>(x, n, partials);
-    sum_partials_kernel<<<1, 32, 0, st>>>(partials, nparts, d_sum);
+    abs_sum_kernel<<<nparts, SUM_NT, 0, st>>>(x, n, partials);
+    sum_partials_kernel<<<1, 256, 0, st>>>(partials, nparts, d_sum);
     return nn_cuda(cudaGetLastError());
 }
 
