@@ -471,6 +471,44 @@ template <int DIR> struct Dft<25, DIR> : DftTwiddled<5, 5, DIR> {};
 template <int DIR> struct Dft<27, DIR> : DftTwiddled<3, 9, DIR> {};
 template <int DIR> struct Dft<30, DIR> : DftCoprime<2, 15, DIR> {};
 
+// ------------------------------------------------- FP64 sums on the FP32 pipe
+// GB300's FP64 pipe does two operations per SM and clock. Energy sums therefore
+// run on unevaluated FP32 pairs (hi + lo, about 2^-46 relative): products by FMA,
+// sums by TwoSum (Knuth), handed to an FP64 accumulator every few dozen values.
+__device__ __forceinline__ float2 two_sum(float a, float b) {
+    const float t = a + b, bp = t - a;
+    return make_float2(t, (a - (t - bp)) + (b - bp));
+}
+__device__ __forceinline__ float2 mul22(float2 a, float2 b) {
+    const float p = a.x * b.x;
+    return make_float2(p, fmaf(a.x, b.x, -p) + fmaf(a.x, b.y, a.y * b.x));
+}
+struct PairSum {
+    float s = 0.f, e = 0.f;
+    __device__ __forceinline__ void add(float2 v) {
+        const float2 t = two_sum(s, v.x);
+        s = t.x;
+        e += t.y + v.y;
+    }
+    __device__ __forceinline__ double take() {
+        const double v = (double)s + (double)e;
+        s = e = 0.f;
+        return v;
+    }
+};
+// (c^2 - 1)^2 added to a sum: pairs while the result stays in FP32's range, FP64 beyond
+__device__ __forceinline__ void add_well(PairSum& ps, double& acc, float c) {
+    if (fabsf(c) > 0x1p28f) {
+        const double q = (double)c * c - 1.0;
+        acc += q * q;
+        return;
+    }
+    const float p = c * c;
+    float2 q = two_sum(p, -1.f);
+    q.y += fmaf(c, c, -p);
+    ps.add(mul22(q, q));
+}
+
 // Tile descriptor: pencil p, element i at buf[i*es + p*ps].
 struct Tile {
     float2* buf;

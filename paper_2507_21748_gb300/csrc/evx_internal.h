@@ -151,7 +151,7 @@ struct ZPassArgs {
     const float2* twA;      // M = R1 R2: w_M^{n2 k1} as [k1][n2], then as [n2][k1] (2 M entries), or null
     float scale;            // 1 / (ny nz)
     const double* cbar;     // FP64 mean (Z_STEP, Z_C2R); may be null (0)
-    double* partials;       // bulk energy partial per CTA (Z_C2R) or null
+    double* partials;       // Z_C2R: bulk energy partial per CTA instead of real rows, or null
     double* gsum;           // Z_STEP, Allen-Cahn: per-CTA FP64 sums of g(c) - g(cbar), or null
     int accumulate;         // Z_C2R: rout += value instead of rout = value
     int fast_ok;            // Z_R2C / Z_C2R: the fast power-of-two kernels may run (grid then reported)
@@ -245,6 +245,7 @@ int staged_zgrid(const ZPassArgs& a);
 bool mixed_split(int L, int* R1, int* R2);
 bool mixed_spass(const SPassArgs& a, int dir, cudaStream_t st, cudaError_t* err);
 bool mixed_xupdate(const XUpdArgs& a, cudaStream_t st, cudaError_t* err);
+bool mixed_xenergy(const XEnergyArgs& a, cudaStream_t st, cudaError_t* err);
 bool mixed_zpass(const ZPassArgs& a, int mode, cudaStream_t st, cudaError_t* err, int* grid_used);
 int mixed_zgrid(const ZPassArgs& a);  // CTAs (partials) of a two-radix z pass, 0 if there is none
 // reads (and optionally clears) the flag a bounded TMA wait sets when it gives up

@@ -750,6 +750,8 @@ cudaError_t launch_xupdate(const XUpdArgs& a, cudaStream_t st) {
 int xenergy_grid(const XEnergyArgs& a) { return a.nchunks * a.ny; }
 
 cudaError_t launch_xenergy(const XEnergyArgs& a, cudaStream_t st) {
+    cudaError_t fe;
+    if (fast_paths_enabled() && mixed_xenergy(a, st, &fe)) return fe;
     const size_t sm = xupdate_smem(a.L);
     cudaError_t e;
     if ((e = set_smem(xenergy_kernel, sm)) != cudaSuccess) return e;

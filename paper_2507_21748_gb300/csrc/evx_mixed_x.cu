@@ -108,6 +108,76 @@ __global__ void __launch_bounds__(BIG1 ? 256 : 128, BIG1 ? 2 : 5) mx_x_kernel(XU
             with_radix<BIG1>(R1, ColStoreInv{a.S_out + base + n2 * a.rs, R2 * a.rs, xs + n2 * CP + p, pitch});
 }
 
+// gradient energy: forward passes A and B of S, sum of w(kz) |k|^2 |c_hat|^2 on FP32 pairs
+struct ColEnergy {
+    const float2* s;  // row k1
+    const float* k2x;  // + k1
+    int R1;
+    double k2yz;
+    bool edge;        // kz = 0 or M: weight 1, otherwise 2 (Hermitian half spectrum)
+    double& acc;
+    template <int R>
+    __device__ __forceinline__ void run() const {
+        float2 v[R];
+#pragma unroll
+        for (int i = 0; i < R; ++i) v[i] = s[i * CP];
+        Dft<R, -1>::run(v);
+        PairSum ps;
+        const float yh = (float)k2yz, yl = (float)(k2yz - (double)yh);
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            const float kx = __ldg(k2x + R1 * k);
+            if (fabsf(v[k].x) > 0x1p50f || fabsf(v[k].y) > 0x1p50f) {
+                acc += (edge ? 1.0 : 2.0) * ((double)kx + k2yz) * ((double)v[k].x * v[k].x + (double)v[k].y * v[k].y);
+                continue;
+            }
+            float2 k2 = two_sum(yh, kx);
+            k2.y += yl;
+            const float px = v[k].x * v[k].x, py = v[k].y * v[k].y;
+            float2 m = two_sum(px, py);
+            m.y += fmaf(v[k].x, v[k].x, -px) + fmaf(v[k].y, v[k].y, -py);
+            ps.add(mul22(k2, m));
+        }
+        acc += (edge ? 1.0 : 2.0) * ps.take();
+    }
+};
+template <bool BIG>
+__global__ void __launch_bounds__(BIG ? 256 : 128, BIG ? 2 : 5) mx_energy_kernel(XEnergyArgs a, int R1, int R2) {
+    extern __shared__ float4 smem4[];
+    __shared__ double red[8];
+    float2* xs = reinterpret_cast<float2*>(smem4);
+    const int p = threadIdx.x & 7, it = threadIdx.x >> 3, T = blockDim.x >> 3;
+    const int R2p = R2 | 1, pitch = R2p * CP;
+    const int ky = blockIdx.y, kz = (int)blockIdx.x * CP + p;
+    const bool valid = kz < a.ncols;
+    const long long base = split_off(ky, a.YB, a.os, a.os2) + kz;
+    if (valid)
+        for (int n2 = it; n2 < R2; n2 += T)
+            with_radix<BIG>(R1, ColLoad<-1>{a.S + base + n2 * a.rs, R2 * a.rs, xs + n2 * CP + p, pitch, a.tw, n2});
+    __syncthreads();
+    double acc = 0.0;
+    if (valid) {
+        const double k2yz = (double)a.k2y[ky] + (double)a.k2z[kz];
+        for (int k1 = it; k1 < R1; k1 += T)
+            with_radix<BIG>(R2, ColEnergy{xs + k1 * pitch + p, a.k2x + k1, R1, k2yz, kz == 0 || kz == a.M, acc});
+    }
+    // fixed-order sum of the CTA (its last warp may be partial)
+    const int lane = threadIdx.x & 31, live = min(32, (int)blockDim.x - (int)(threadIdx.x & ~31));
+    const unsigned here = live == 32 ? 0xffffffffu : (1u << live) - 1;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const double t = __shfl_down_sync(here, acc, o);
+        if (lane + o < live) acc += t;
+    }
+    if (lane == 0) red[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int w = 0; w < ((int)blockDim.x + 31) / 32; ++w) t += red[w];
+        a.partials[(long long)blockIdx.y * gridDim.x + blockIdx.x] = t;
+    }
+}
+
 }  // namespace mixed
 
 template <int MODE>
@@ -122,6 +192,19 @@ bool mixed_xupdate(const XUpdArgs& a, cudaStream_t st, cudaError_t* err) {
     if (!a.W || !mixed_split(a.L, &R1, &R2)) return false;
     const size_t smem = sizeof(float2) * R1 * (R2 | 1) * SP * (a.model == 2 ? 1 : 2);
     auto kern = a.model == 3 ? mx_x_pick<3>(R1, R2) : a.model == 2 ? mx_x_pick<2>(R1, R2) : mx_x_pick<0>(R1, R2);
+    if ((*err = mx_smem(kern, smem)) != cudaSuccess) return true;
+    kern<<<dim3(a.nchunks, a.ny), R1 * SP, smem, st>>>(a, R1, R2);
+    *err = cudaGetLastError();
+    return true;
+}
+
+// The energy's x pass, of every length with two radices (the tuned kernels' among them:
+// 313 us at 256^3 stage by stage with FP64 sums, 54 us now)
+bool mixed_xenergy(const XEnergyArgs& a, cudaStream_t st, cudaError_t* err) {
+    int R1, R2;
+    if (!mixed_split(a.L, &R1, &R2)) return false;
+    const size_t smem = sizeof(float2) * R1 * (R2 | 1) * SP;
+    auto kern = R1 > 16 ? mixed::mx_energy_kernel<true> : mixed::mx_energy_kernel<false>;
     if ((*err = mx_smem(kern, smem)) != cudaSuccess) return true;
     kern<<<dim3(a.nchunks, a.ny), R1 * SP, smem, st>>>(a, R1, R2);
     *err = cudaGetLastError();

@@ -209,30 +209,30 @@ __global__ void __launch_bounds__(BIG ? 256 : 192, BIG ? 2 : 3) mx_z_kernel(ZPas
         if (MODE == Z_C2R) {
             with_radix<BIG>(R2, ZInvB{z, a.scale, cb, cbl, tx, actB});
             __syncthreads();
-            double acc = 0.0;
-            for (int r = tid / T; r < nr; r += RPC) {
-                const long long rr = row0 + r;
-                const long long ur = a.map_rows ? user_row(rr, a.YB, a.nxr, a.nyr) : rr;
-                float2* dst = reinterpret_cast<float2*>(a.rout + ur * a.rpitch);
-                for (int q = tx; q < M; q += T) {
-                    float2 c = buf[r * RS + q];
-                    if (a.accumulate) c = cadd(dst[q], c);
-                    dst[q] = c;
-                    if (a.partials) {
-                        const double q0 = (double)c.x * c.x - 1.0, q1 = (double)c.y * c.y - 1.0;
-                        acc += q0 * q0 + q1 * q1;
+            if (a.partials) {  // energy: nothing is written
+                double acc = 0.0;
+                PairSum ps;
+                if (rowok)
+                    for (int q = tx; q < M; q += T) {
+                        add_well(ps, acc, z.row[q].x);
+                        add_well(ps, acc, z.row[q].y);
                     }
-                }
-            }
-            if (a.partials) {
                 __shared__ double red[256];
-                red[tid] = acc;
+                red[tid] = acc + ps.take();
                 __syncthreads();
-                if (tid == 0) {
+                if (tid < 32) {
                     double t = 0.0;
-                    for (int i = 0; i < nthr; ++i) t += red[i];
-                    a.partials[blockIdx.x] = t;
+                    for (int i = tid; i < nthr; i += 32) t += red[i];
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+                    if (tid == 0) a.partials[blockIdx.x] = t;
                 }
+                return;
+            }
+            if (rowok) {
+                const long long ur = a.map_rows ? user_row(row, a.YB, a.nxr, a.nyr) : row;
+                float2* dst = reinterpret_cast<float2*>(a.rout + ur * a.rpitch);
+                for (int q = tx; q < M; q += T) dst[q] = a.accumulate ? cadd(dst[q], z.row[q]) : z.row[q];
             }
             return;
         }
@@ -302,7 +302,7 @@ bool mixed_zpass(const ZPassArgs& a, int mode, cudaStream_t st, cudaError_t* err
     const float* real = mode == Z_R2C ? a.rin : mode == Z_ADJ ? a.cn : a.rout;
     const long long pitch = mode == Z_ADJ ? a.cnpitch : a.rpitch;
     if (real && (((uintptr_t)real & 7) || (pitch & 1))) return false;
-    if (mode == Z_C2R && !a.rout) return false;
+    if (mode == Z_C2R && !a.rout && !a.partials) return false;
     const int RS = mixed_zstride(a, R1, R2), rpc = mixed_zrows(a, R1, RS);
     const int grid = (int)((a.nrows + rpc - 1) / rpc);
     const size_t smem = sizeof(float2) * RS * rpc;

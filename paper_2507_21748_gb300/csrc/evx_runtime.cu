@@ -763,9 +763,9 @@ evx_status evx_energy(evx_grid* g, double* E, double* mass) {
         if (mass) *mass = h3 * V * host[0];
         return check_timeouts(g);
     }
-    // bulk: h^3/4 sum (c^2-1)^2 over the real field (written into W's row slots, discarded)
+    // bulk: h^3/4 sum (c^2-1)^2 over the real field, which is not written
     int zg = 0;
-    evx_status s = store_real(g, (float*)g->W, 2LL * g->Zp, g->d_part, 0, &zg);
+    evx_status s = store_real(g, nullptr, g->nz, g->d_part, 0, &zg);
     if (s != EVX_OK) return s;
     CK(launch_reduce_partials(g->d_part, zg, g->d_scal + 1, 0.25 * h3, g->st));
     // gradient: h^3 (kappa/2)(1/V) sum_k |k|^2 |c_hat|^2

@@ -426,25 +426,25 @@ __global__ void __launch_bounds__(256, 2) stg_z_kernel(ZPassArgs a, Cut c, int R
         __syncthreads();
         if (MODE == Z_C2R) {
             double acc = 0.0;
+            PairSum ps;
             if (rowok) {
-                float2* o = reinterpret_cast<float2*>(a.rout + ur * a.rpitch);
+                float2* o = a.partials ? nullptr : reinterpret_cast<float2*>(a.rout + ur * a.rpitch);
                 for (int n = tx; n < M; n += T) {
                     const int q = n / c.R1, m = n - q * c.R1;
                     float2 v = z[m * c.R2p + q];
-                    if (a.accumulate) {
+                    if (a.partials) {  // energy: nothing is written
+                        add_well(ps, acc, v.x);
+                        add_well(ps, acc, v.y);
+                    } else if (a.accumulate) {
                         const float2 prev = o[n];
                         o[n] = make_float2(prev.x + v.x, prev.y + v.y);
                     } else {
                         o[n] = v;
                     }
-                    if (a.partials) {
-                        const double q0 = (double)v.x * v.x - 1.0, q1 = (double)v.y * v.y - 1.0;
-                        acc += q0 * q0 + q1 * q1;
-                    }
                 }
             }
             if (a.partials) {
-                red[tid] = acc;
+                red[tid] = acc + ps.take();
                 __syncthreads();
                 if (tid < 32) {
                     double t = 0.0;
@@ -556,7 +556,7 @@ bool staged_zpass(const ZPassArgs& a, int mode, cudaStream_t st, cudaError_t* er
     const float* real = mode == Z_R2C ? a.rin : mode == Z_ADJ ? a.cn : a.rout;
     const long long pitch = mode == Z_ADJ ? a.cnpitch : a.rpitch;
     if (real && (((uintptr_t)real & 7) || (pitch & 1))) return false;
-    if (mode == Z_C2R && !a.rout) return false;
+    if (mode == Z_C2R && !a.rout && !a.partials) return false;
     const int RS = staged_zstride(a, c), rpc = staged_zrows(a, c, RS), T = std::max(c.R1, c.R2);
     const int grid = (int)((a.nrows + rpc - 1) / rpc);
     auto kern = mode == Z_STEP  ? staged::stg_z_kernel<Z_STEP>
