@@ -521,119 +521,185 @@ __global__ void __launch_bounds__(256) vm_rhs_kernel(const float* __restrict__ c
     }
 }
 
-// Both stencils in one pass (rhs straight from c, mu never stored): a CTA owns
-// TY x TZ columns (y, z) and marches along x through XC planes, with c in a ring
-// of 8 planes (2-halo in y and z), and mu and the mobility M(c) in rings of 4
-// planes (1-halo) in shared memory. Plane x + 3 is copied in with cp.async while
-// plane x is computed; each thread's shared and global offsets are the same on
-// every plane and are computed once. Each c value is read from HBM once (its
-// halo copies mostly from L2) and rhs written once: 8 B per voxel against 20 B
-// for the two separate kernels. The arithmetic and its grouping are those of
-// vm_mu_kernel and vm_rhs_kernel (same results to the bit).
-constexpr int VM_TY = 8, VM_TZ = 64, VM_XC = 64, VM_CS = 8, VM_NT = 256;
-constexpr int VM_CY = VM_TY + 4, VM_CZ = VM_TZ + 4, VM_MY = VM_TY + 2, VM_MZ = VM_TZ + 2;
-constexpr int VM_CP = VM_CY * VM_CZ, VM_MP = VM_MY * VM_MZ;  // floats per c / mu plane
-constexpr int VM_NL = (VM_CP + VM_NT - 1) / VM_NT, VM_NM = (VM_MP + VM_NT - 1) / VM_NT, VM_NR = VM_TY * VM_TZ / VM_NT;
-__device__ __forceinline__ int vm_wrap(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
-__device__ __forceinline__ void cp_async4(float* dst, const float* src, bool ok) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(ok ? 4 : 0) : "memory");
+// Both stencils in one pass (rhs straight from c, mu never stored). A CTA owns
+// VM_TY rows (y) x VM_TZ columns (z) and marches along x; a thread owns four
+// adjacent z of one row, the rows just outside the tile included (they compute mu
+// for the y neighbours), and one more warp the mu points at the two z edges. A
+// thread keeps its own column in registers - c of three planes, mu and M(c) of
+// three - so shared memory serves the y neighbours (16-byte reads) and the two z
+// ends of each four: 3 reads per point instead of the 21 of one thread per point,
+// which bound the earlier kernel (180 us at 320 x 384 x 320, 127 now; the field
+// read once and rhs written once take 46 us; instruction issue still bounds it). c planes sit in a ring of four
+// (2-halo in y and z, plane x + 3 copied in with cp.async while plane x is worked
+// on), mu and M planes in a ring of two; one barrier per plane. The arithmetic and
+// its grouping are those of vm_mu_kernel and vm_rhs_kernel (same results to the bit).
+constexpr int VM_TY = 16, VM_TZ = 64, VM_Q = VM_TZ / 4;
+constexpr int VM_MAIN = (VM_TY + 2) * VM_Q, VM_NT = VM_MAIN + 32;  // 288 + a warp for the z edges
+constexpr int VM_CZ = VM_TZ + 8, VM_CY = VM_TY + 4;  // c rows: z0 - 2 at 2, z0 at 4
+constexpr int VM_MZ = VM_TZ + 8, VM_MY = VM_TY + 2;  // mu, M rows: z0 - 1 at 3, z0 at 4
+constexpr int VM_CP = VM_CY * VM_CZ, VM_MP = VM_MY * VM_MZ;
+constexpr size_t VM_SMEM = sizeof(float) * (4 * VM_CP + 4 * VM_MP);  // 43,776 bytes
+static_assert(VM_MAIN % 32 == 0 && 2 * VM_TY <= 32, "vm_fd_kernel thread map");
+__device__ __forceinline__ int vm_mod(int i, int n) {
+    i %= n;
+    return i < 0 ? i + n : i;
 }
-__global__ void __launch_bounds__(VM_NT) vm_fd_kernel(const float* __restrict__ c, float* __restrict__ rhs, int nx,
-                                                       int ny, int nz, float kh2, float M0, float ih2) {
-    static_assert(VM_TY * VM_TZ % VM_NT == 0, "rhs points per thread");
-    extern __shared__ float vm_smem[];
-    float* cs = vm_smem;                  // [VM_CS][VM_CY][VM_CZ]
-    float* ms = cs + VM_CS * VM_CP;       // [4][VM_MY][VM_MZ] mu
-    float* mbs = ms + 4 * VM_MP;          // [4][VM_MY][VM_MZ] M(c)
-    const int y0 = blockIdx.x * VM_TY, z0 = blockIdx.y * VM_TZ, x0 = blockIdx.z * VM_XC;
-    const int xe = min(x0 + VM_XC, nx);
-    const long long V = (long long)nx * ny * nz;
+template <int BYTES>
+__device__ __forceinline__ void vm_cp_async(float* dst, const float* src) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    if (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+}
+__global__ void __launch_bounds__(VM_NT, 2) vm_fd_kernel(const float* __restrict__ c, float* __restrict__ rhs, int nx,
+                                                         int ny, int nz, int xc, float kh2, float M0, float ih2) {
+    extern __shared__ __align__(16) float vm_smem[];
+    float* cs = vm_smem;               // [4][VM_CY][VM_CZ]
+    float* ms = cs + 4 * VM_CP;        // [2][VM_MY][VM_MZ] mu
+    float* bs = ms + 2 * VM_MP;        // [2][VM_MY][VM_MZ] M(c)
+    const int y0 = blockIdx.x * VM_TY, z0 = blockIdx.y * VM_TZ, x0 = blockIdx.z * xc;
+    const int xe = min(x0 + xc, nx), nzv = min(VM_TZ, nz - z0);  // a multiple of 4
+    const long long V = (long long)nx * ny * nz, plane = (long long)ny * nz;
     const int tid = threadIdx.x;
-    // this thread's points: c loads (plane offset in c, index in a c plane), mu / M
-    // points (index in a mu plane, centre index in a c plane), rhs points (likewise)
-    int lg[VM_NL], ls[VM_NL], mi_[VM_NM], mc[VM_NM], rm[VM_NR], ro[VM_NR];
+    auto mob = [&](float v) { return M0 * fmaxf(1.f - v * v, 0.f); };
+    // this thread's copies of a c plane, the same on every plane: pieces of 16 bytes (VM_Q per
+    // row, those beyond the last z left out) and the two 8-byte z halos of a row
+    constexpr int NL = (VM_CY * (VM_Q + 2) + VM_NT - 1) / VM_NT;
+    int ld[NL], ls[NL];  // place in the shared plane (-1: none; halos: + VM_CP), offset in the field's plane
 #pragma unroll
-    for (int k = 0; k < VM_NL; ++k) {
-        const int i = tid + k * VM_NT, r = i / VM_CZ, q = i - r * VM_CZ;
-        lg[k] = i < VM_CP ? vm_wrap(y0 + r - 2, ny) * nz + vm_wrap(z0 + q - 2, nz) : -1;
-        ls[k] = i;
+    for (int k = 0; k < NL; ++k) {
+        const int i = tid + k * VM_NT, r = i / (VM_Q + 2), q = i - r * (VM_Q + 2);
+        const int row = vm_mod(y0 + r - 2, ny) * nz;
+        if (i >= VM_CY * (VM_Q + 2) || (q < VM_Q && 4 * q >= nzv)) {
+            ld[k] = -1;
+            ls[k] = 0;
+        } else if (q < VM_Q) {
+            ld[k] = r * VM_CZ + 4 + 4 * q;
+            ls[k] = row + z0 + 4 * q;
+        } else {
+            ld[k] = VM_CP + r * VM_CZ + (q == VM_Q ? 2 : 4 + nzv);
+            ls[k] = row + (q == VM_Q ? vm_mod(z0 - 2, nz) : vm_mod(z0 + nzv, nz));
+        }
     }
+    auto load_c = [&](int xp) {
+        float* dst = cs + ((xp + 4) & 3) * VM_CP;
+        const long long pb = (long long)(xp < 0 ? xp + nx : xp >= nx ? xp - nx : xp) * plane;
 #pragma unroll
-    for (int k = 0; k < VM_NM; ++k) {
-        const int i = tid + k * VM_NT, r = i / VM_MZ, q = i - r * VM_MZ;
-        mi_[k] = i < VM_MP ? i : -1;
-        mc[k] = (r + 1) * VM_CZ + q + 1;
-    }
-#pragma unroll
-    for (int k = 0; k < VM_NR; ++k) {
-        const int i = tid + k * VM_NT, r = i / VM_TZ, q = i - r * VM_TZ;
-        rm[k] = (r + 1) * VM_MZ + q + 1;
-        ro[k] = (y0 + r) * nz + z0 + q;
-    }
-    auto load_c = [&](int xp) {  // plane xp (x0 - 2 <= xp <= xe + 1) into slot (xp + 8) % 8, one commit group
-        float* dst = cs + ((xp + VM_CS) % VM_CS) * VM_CP;
-        const long long pb = (long long)vm_wrap(xp, nx) * ny * nz;
-#pragma unroll
-        for (int k = 0; k < VM_NL; ++k)
-            if (lg[k] >= 0) {
-                const long long g = pb + lg[k];
-                cp_async4(dst + ls[k], c + (EVX_IN(g, V) ? g : 0), EVX_IN(g, V));
+        for (int k = 0; k < NL; ++k) {
+            const long long g = pb + ls[k];
+            if (ld[k] >= VM_CP) {
+                if (EVX_IN(g + 1, V)) vm_cp_async<8>(dst + ld[k] - VM_CP, c + g);
+            } else if (ld[k] >= 0) {
+                if (EVX_IN(g + 3, V)) vm_cp_async<16>(dst + ld[k], c + g);
             }
+        }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    auto mu_plane = [&](int xp) {  // mu and M of plane xp, rows y0 - 1 .., columns z0 - 1 ..
-        const float* c0 = cs + ((xp + VM_CS) % VM_CS) * VM_CP;
-        const float* cm = cs + ((xp + VM_CS - 1) % VM_CS) * VM_CP;
-        const float* cp = cs + ((xp + 1) % VM_CS) * VM_CP;
-        float* mo = ms + ((xp + 4) & 3) * VM_MP;
-        float* bo = mbs + ((xp + 4) & 3) * VM_MP;
-#pragma unroll
-        for (int k = 0; k < VM_NM; ++k)
-            if (mi_[k] >= 0) {
-                const int e = mc[k];
-                const float v = c0[e];
-                const float nb = ((cp[e] + cm[e]) + (c0[e + VM_CZ] + c0[e - VM_CZ])) + (c0[e + 1] + c0[e - 1]);
-                mo[mi_[k]] = v * (v * v - 1.f) - kh2 * fmaf(-6.f, v, nb);
-                bo[mi_[k]] = M0 * fmaxf(1.f - v * v, 0.f);
-            }
+    // this thread's points: row r of the mu plane (y0 - 1 + r), columns 4 q .. 4 q + 3; or one z edge point
+    const bool mainw = tid < VM_MAIN;
+    const int e = tid - VM_MAIN;
+    const int r = mainw ? tid / VM_Q : 1 + (e >> 1), q = tid % VM_Q;
+    const bool active = mainw ? 4 * q < nzv : (e >> 1) < VM_TY;
+    const int ce = (r + 1) * VM_CZ + (mainw ? 4 + 4 * q : (e & 1 ? 4 + nzv : 3));  // own points in a c plane
+    const int me = r * VM_MZ + (mainw ? 4 + 4 * q : (e & 1 ? 4 + nzv : 3));        // and in a mu plane
+    const bool inner = mainw && active && r >= 1 && r <= VM_TY && y0 + r - 1 < ny;  // has rhs points
+    float cm[4], c0[4], cp[4];              // c of planes x, x + 1, x + 2 while mu of x + 1 is formed
+    float um[4], u0[4], up[4], bm[4], b0[4], bp[4];  // mu and M of planes x - 1, x, x + 1
+    auto own = [&](int xp, float (&v)[4]) {
+        const float* s = cs + ((xp + 4) & 3) * VM_CP + ce;
+        if (mainw) {
+            const float4 f = *reinterpret_cast<const float4*>(s);
+            v[0] = f.x, v[1] = f.y, v[2] = f.z, v[3] = f.w;
+        } else {
+            v[0] = s[0];
+        }
     };
-    for (int xp = x0 - 2; xp <= x0 + 2; ++xp) load_c(xp);
+    // mu and M of plane xp at this thread's points into up, bp and the ring
+    auto mu_plane = [&](int xp) {
+        const float* s = cs + ((xp + 4) & 3) * VM_CP + ce;
+        if (mainw) {
+            const float4 yp = *reinterpret_cast<const float4*>(s + VM_CZ), ym = *reinterpret_cast<const float4*>(s - VM_CZ);
+            const float a[4] = {yp.x, yp.y, yp.z, yp.w}, d[4] = {ym.x, ym.y, ym.z, ym.w};
+            const float zl = s[-1], zr = s[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float v = c0[i];
+                const float nb = ((cp[i] + cm[i]) + (a[i] + d[i])) + ((i < 3 ? c0[i + 1] : zr) + (i > 0 ? c0[i - 1] : zl));
+                up[i] = v * (v * v - 1.f) - kh2 * fmaf(-6.f, v, nb);
+                bp[i] = mob(v);
+            }
+            const int o = ((xp + 4) & 1) * VM_MP + me;
+            *reinterpret_cast<float4*>(ms + o) = make_float4(up[0], up[1], up[2], up[3]);
+            *reinterpret_cast<float4*>(bs + o) = make_float4(bp[0], bp[1], bp[2], bp[3]);
+        } else {
+            const float v = c0[0];
+            const float nb = ((cp[0] + cm[0]) + (s[VM_CZ] + s[-VM_CZ])) + (s[1] + s[-1]);
+            const int o = ((xp + 4) & 1) * VM_MP + me;
+            ms[o] = v * (v * v - 1.f) - kh2 * fmaf(-6.f, v, nb);
+            bs[o] = mob(v);
+        }
+    };
+    for (int xp = x0 - 2; xp <= x0 + 1; ++xp) load_c(xp);
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
-    mu_plane(x0 - 1);
-    mu_plane(x0);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) cm[i] = c0[i] = cp[i] = um[i] = u0[i] = up[i] = bm[i] = b0[i] = bp[i] = 0.f;
+    if (active) {  // mu of planes x0 - 1 and x0
+        own(x0 - 2, cm);
+        own(x0 - 1, c0);
+        own(x0, cp);
+        mu_plane(x0 - 1);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) um[i] = up[i], bm[i] = bp[i], cm[i] = c0[i], c0[i] = cp[i];
+        own(x0 + 1, cp);
+        mu_plane(x0);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) u0[i] = up[i], b0[i] = bp[i], cm[i] = c0[i], c0[i] = cp[i];
+    }
+    __syncthreads();
+    load_c(x0 + 2);  // the slot of plane x0 - 2
     for (int x = x0; x < xe; ++x) {
-        // planes x - 1 .. x + 2 are in; plane x + 3 takes the slot of plane x - 5
         if (x + 3 <= xe + 1)
-            load_c(x + 3);
+            load_c(x + 3);  // the slot of plane x - 1, last read two barriers ago
         else
             asm volatile("cp.async.commit_group;" ::: "memory");
-        asm volatile("cp.async.wait_group 1;" ::: "memory");  // all but the newest group: plane x + 2
+        asm volatile("cp.async.wait_group 1;" ::: "memory");  // plane x + 2 has arrived
         __syncthreads();
-        mu_plane(x + 1);  // the mu and M slots of plane x - 3
-        __syncthreads();
-        const float* u0 = ms + ((x + 4) & 3) * VM_MP;
-        const float* um = ms + ((x + 3) & 3) * VM_MP;
-        const float* up = ms + ((x + 5) & 3) * VM_MP;
-        const float* b0 = mbs + ((x + 4) & 3) * VM_MP;
-        const float* bm = mbs + ((x + 3) & 3) * VM_MP;
-        const float* bp = mbs + ((x + 5) & 3) * VM_MP;
-        const long long pb = (long long)x * ny * nz;
+        if (active) {
+            own(x + 2, cp);
+            mu_plane(x + 1);
+        }
+        if (inner) {
+            // neighbours of plane x in the order x+, x-, y+, y-, z+, z-; mu and M of the row's ends and of y +- 1 from the ring
+            const int o = ((x + 4) & 1) * VM_MP + me;
+            const float4 uyp = *reinterpret_cast<const float4*>(ms + o + VM_MZ), uym = *reinterpret_cast<const float4*>(ms + o - VM_MZ);
+            const float4 byp = *reinterpret_cast<const float4*>(bs + o + VM_MZ), bym = *reinterpret_cast<const float4*>(bs + o - VM_MZ);
+            const float ua[4] = {uyp.x, uyp.y, uyp.z, uyp.w}, ub[4] = {uym.x, uym.y, uym.z, uym.w};
+            const float ba[4] = {byp.x, byp.y, byp.z, byp.w}, bb[4] = {bym.x, bym.y, bym.z, bym.w};
+            const float ul = ms[o - 1], ur = ms[o + 4], bl = bs[o - 1], br = bs[o + 4];
+            float out[4];
 #pragma unroll
-        for (int k = 0; k < VM_NR; ++k) {
-            const int e = rm[k];
-            const float mi = b0[e], ui = u0[e];
-            // neighbours in the order x+, x-, y+, y-, z+, z-
-            float acc = 0.f;
-            acc = fmaf(0.5f * (mi + bp[e]), up[e] - ui, acc);
-            acc = fmaf(0.5f * (mi + bm[e]), um[e] - ui, acc);
-            acc = fmaf(0.5f * (mi + b0[e + VM_MZ]), u0[e + VM_MZ] - ui, acc);
-            acc = fmaf(0.5f * (mi + b0[e - VM_MZ]), u0[e - VM_MZ] - ui, acc);
-            acc = fmaf(0.5f * (mi + b0[e + 1]), u0[e + 1] - ui, acc);
-            acc = fmaf(0.5f * (mi + b0[e - 1]), u0[e - 1] - ui, acc);
-            const long long o = pb + ro[k];
-            if (EVX_IN(o, V)) rhs[o] = acc * ih2;
+            for (int i = 0; i < 4; ++i) {
+                const float mi = b0[i], ui = u0[i];
+                const float uzp = i < 3 ? u0[i + 1] : ur, uzm = i > 0 ? u0[i - 1] : ul;
+                const float bzp = i < 3 ? b0[i + 1] : br, bzm = i > 0 ? b0[i - 1] : bl;
+                float acc = 0.f;
+                acc = fmaf(0.5f * (mi + bp[i]), up[i] - ui, acc);
+                acc = fmaf(0.5f * (mi + bm[i]), um[i] - ui, acc);
+                acc = fmaf(0.5f * (mi + ba[i]), ua[i] - ui, acc);
+                acc = fmaf(0.5f * (mi + bb[i]), ub[i] - ui, acc);
+                acc = fmaf(0.5f * (mi + bzp), uzp - ui, acc);
+                acc = fmaf(0.5f * (mi + bzm), uzm - ui, acc);
+                out[i] = acc * ih2;
+            }
+            const long long g = (long long)x * plane + (long long)(y0 + r - 1) * nz + z0 + 4 * q;
+            if (EVX_IN(g + 3, V)) *reinterpret_cast<float4*>(rhs + g) = make_float4(out[0], out[1], out[2], out[3]);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            um[i] = u0[i], u0[i] = up[i], bm[i] = b0[i], b0[i] = bp[i];
+            cm[i] = c0[i], c0[i] = cp[i];
         }
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -827,14 +893,17 @@ cudaError_t launch_vm_mu(const float* c, float* mu, int nx, int ny, int nz, floa
     return cudaGetLastError();
 }
 
-bool vm_fd_fused_ok(int nx, int ny, int nz) { return ny % VM_TY == 0 && nz % VM_TZ == 0 && nx >= 8; }
+// one kernel for rows of whole 16-byte pieces; other nz take the two kernels
+bool vm_fd_fused_ok(int nx, int ny, int nz) { return nz % 4 == 0 && nx >= 8; }
 
 cudaError_t launch_vm_fd(const float* c, float* rhs, int nx, int ny, int nz, float kappa_h2, float M0, float inv_h2,
                          cudaStream_t st) {
     if (!vm_fd_fused_ok(nx, ny, nz)) return cudaErrorInvalidValue;
-    constexpr size_t smem = sizeof(float) * (VM_CS * VM_CP + 8 * VM_MP);  // 47,232 bytes
-    vm_fd_kernel<<<dim3(ny / VM_TY, nz / VM_TZ, (nx + VM_XC - 1) / VM_XC), VM_NT, smem, st>>>(c, rhs, nx, ny, nz,
-                                                                                           kappa_h2, M0, inv_h2);
+    const int ty = (ny + VM_TY - 1) / VM_TY, tz = (nz + VM_TZ - 1) / VM_TZ;
+    // x chunks of 64 planes (each loads 4 more), shorter while the launch would leave SMs idle
+    int xc = 64;
+    while (xc > 8 && (long long)ty * tz * ((nx + xc - 1) / xc) < 2 * 152) xc /= 2;
+    vm_fd_kernel<<<dim3(ty, tz, (nx + xc - 1) / xc), VM_NT, VM_SMEM, st>>>(c, rhs, nx, ny, nz, xc, kappa_h2, M0, inv_h2);
     return cudaGetLastError();
 }
 

@@ -32,27 +32,21 @@ namespace evx {
 namespace mixed {
 
 // ------------------------------------------------------------------ radices
-#define EVX_MX_SMALL(F) F(1) F(2) F(3) F(4) F(5) F(6) F(8) F(9) F(10) F(12) F(15) F(16)
-#define EVX_MX_LARGE(F) F(18) F(20) F(24) F(25) F(27) F(30) F(32)
+#define EVX_MX_RADICES(F) \
+    F(1) F(2) F(3) F(4) F(5) F(6) F(8) F(9) F(10) F(12) F(15) F(16) F(18) F(20) F(24) F(25) F(27) F(30) F(32)
 
-// f.template run<R>() for the radix r; BIG: radices above 16 are compiled in
-template <bool BIG, typename Fn>
+// f.template run<R>() for the radix r <= MAX. Kernels are compiled for a few MAX: the
+// registers of a kernel are those of its largest radix.
+template <int MAX, typename Fn>
 __device__ __forceinline__ void with_radix(int r, Fn&& f) {
     switch (r) {
-#define EVX_MX_CASE(R) \
-    case R: f.template run<R>(); return;
-        EVX_MX_SMALL(EVX_MX_CASE)
+#define EVX_MX_CASE(R)                                 \
+    case R:                                            \
+        if constexpr (R <= MAX) f.template run<R>();   \
+        return;
+        EVX_MX_RADICES(EVX_MX_CASE)
 #undef EVX_MX_CASE
         default: break;
-    }
-    if constexpr (BIG) {
-        switch (r) {
-#define EVX_MX_CASE(R) \
-    case R: f.template run<R>(); return;
-            EVX_MX_LARGE(EVX_MX_CASE)
-#undef EVX_MX_CASE
-            default: break;
-        }
     }
 }
 

@@ -4,6 +4,13 @@
 namespace evx {
 namespace mixed {
 
+// 1 / D for D >= 1: the hardware's approximation and one Newton step r + r (1 - D r)
+__device__ __forceinline__ float inverse(float D) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(D));
+    return fmaf(r, fmaf(-D, r, 1.f), r);
+}
+
 // middle of the x pass: forward pass B of W and S, the update, inverse pass B;
 // row k1 of the exchanges (column p). MODE as in XUpdArgs.model, 0 also for 1.
 // SPILL: F_x W is put back into its own slots instead of being held in registers.
@@ -41,7 +48,7 @@ struct ColUpdate {
 #pragma unroll
             for (int k = 0; k < R; ++k) {
                 const float k2 = __ldg(k2x + R1 * k) + k2yz;
-                v[k] = cscale(g[k], a.dtM * (a.invL / fmaf(a.dtMk, k2 * k2, 1.f)));
+                v[k] = cscale(g[k], a.dtM * (a.invL * inverse(fmaf(a.dtMk, k2 * k2, 1.f))));
             }
         } else {
             if (SPILL) {
@@ -56,13 +63,13 @@ struct ColUpdate {
                 const float2 gk = SPILL ? w[k * CP] : g[k];
                 const float k2 = __ldg(k2x + R1 * k) + k2yz;
                 if (MODE == 3) {
-                    const float Dinv = 1.f / fmaf(a.dtMk, k2 * k2, 1.f);
+                    const float Dinv = inverse(fmaf(a.dtMk, k2 * k2, 1.f));
                     float P, S;
                     blk(k2, Dinv, P, S);
                     const float bs = -a.dtM * k2 * Dinv * S * a.invL, as = P * a.invL;
                     v[k] = make_float2(fmaf(bs, gk.x, as * v[k].x), fmaf(bs, gk.y, as * v[k].y));
                 } else {  // (c_hat - dt M |k|^2 g_hat) / (1 + dt M kappa |k|^4); Allen-Cahn: 1 and |k|^2
-                    const float f = a.invL / fmaf(a.dtMk, ac ? k2 : k2 * k2, 1.f);
+                    const float f = a.invL * inverse(fmaf(a.dtMk, ac ? k2 : k2 * k2, 1.f));
                     const float b = -a.dtM * (ac ? 1.f : k2);
                     v[k] = make_float2(f * fmaf(b, gk.x, v[k].x), f * fmaf(b, gk.y, v[k].y));
                 }
@@ -76,9 +83,9 @@ struct ColUpdate {
     }
 };
 
-// BIG1 / BIG2: radices above 16 for R1 / R2
-template <int MODE, bool BIG1, bool BIG2>
-__global__ void __launch_bounds__(BIG1 ? 256 : 128, BIG1 ? 2 : 5) mx_x_kernel(XUpdArgs a, int R1, int R2) {
+// M1, M2: largest radices of R1 and R2
+template <int MODE, int M1, int M2>
+__global__ void __launch_bounds__(8 * M1, M1 <= 16 ? 5 : M1 <= 20 ? 4 : 2) mx_x_kernel(XUpdArgs a, int R1, int R2) {
     extern __shared__ float4 smem4[];
     const int p = threadIdx.x & 7, it = threadIdx.x >> 3, T = blockDim.x >> 3;
     const int R2p = R2 | 1, pitch = R2p * CP;
@@ -91,7 +98,7 @@ __global__ void __launch_bounds__(BIG1 ? 256 : 128, BIG1 ? 2 : 5) mx_x_kernel(XU
         for (int i = it; i < (MODE == 2 ? R2 : 2 * R2); i += T) {
             const bool second = i >= R2;
             const int n2 = second ? i - R2 : i;
-            with_radix<BIG1>(R1, ColLoad<-1>{(second ? a.S : a.W) + base + n2 * a.rs, R2 * a.rs,
+            with_radix<M1>(R1, ColLoad<-1>{(second ? a.S : a.W) + base + n2 * a.rs, R2 * a.rs,
                                              (second ? xs : xw) + n2 * CP + p, pitch, a.tw, n2});
         }
     __syncthreads();
@@ -99,13 +106,13 @@ __global__ void __launch_bounds__(BIG1 ? 256 : 128, BIG1 ? 2 : 5) mx_x_kernel(XU
         const float k2yz = a.k2y[ky] + a.k2z[kz];
         const float gpb = MODE == 3 ? (float)(3.0 * (*a.cbar) * (*a.cbar) - 1.0) : 0.f;
         for (int k1 = it; k1 < R1; k1 += T)
-            with_radix<BIG2>(R2, ColUpdate<MODE, BIG2>{a, xw + k1 * pitch + p, xs + k1 * pitch + p, a.k2x + k1, R1, k1,
+            with_radix<M2>(R2, ColUpdate<MODE, (M2 > 16)>{a, xw + k1 * pitch + p, xs + k1 * pitch + p, a.k2x + k1, R1, k1,
                                                        k2yz, gpb, k1 == 0 && ky == 0 && kz == 0});
     }
     __syncthreads();
     if (valid)
         for (int n2 = it; n2 < R2; n2 += T)
-            with_radix<BIG1>(R1, ColStoreInv{a.S_out + base + n2 * a.rs, R2 * a.rs, xs + n2 * CP + p, pitch});
+            with_radix<M1>(R1, ColStoreInv{a.S_out + base + n2 * a.rs, R2 * a.rs, xs + n2 * CP + p, pitch});
 }
 
 // gradient energy: forward passes A and B of S, sum of w(kz) |k|^2 |c_hat|^2 on FP32 pairs
@@ -141,8 +148,8 @@ struct ColEnergy {
         acc += (edge ? 1.0 : 2.0) * ps.take();
     }
 };
-template <bool BIG>
-__global__ void __launch_bounds__(BIG ? 256 : 128, BIG ? 2 : 5) mx_energy_kernel(XEnergyArgs a, int R1, int R2) {
+template <int MAX>
+__global__ void __launch_bounds__(8 * MAX, MAX <= 16 ? 5 : 2) mx_energy_kernel(XEnergyArgs a, int R1, int R2) {
     extern __shared__ float4 smem4[];
     __shared__ double red[8];
     float2* xs = reinterpret_cast<float2*>(smem4);
@@ -153,13 +160,13 @@ __global__ void __launch_bounds__(BIG ? 256 : 128, BIG ? 2 : 5) mx_energy_kernel
     const long long base = split_off(ky, a.YB, a.os, a.os2) + kz;
     if (valid)
         for (int n2 = it; n2 < R2; n2 += T)
-            with_radix<BIG>(R1, ColLoad<-1>{a.S + base + n2 * a.rs, R2 * a.rs, xs + n2 * CP + p, pitch, a.tw, n2});
+            with_radix<MAX>(R1, ColLoad<-1>{a.S + base + n2 * a.rs, R2 * a.rs, xs + n2 * CP + p, pitch, a.tw, n2});
     __syncthreads();
     double acc = 0.0;
     if (valid) {
         const double k2yz = (double)a.k2y[ky] + (double)a.k2z[kz];
         for (int k1 = it; k1 < R1; k1 += T)
-            with_radix<BIG>(R2, ColEnergy{xs + k1 * pitch + p, a.k2x + k1, R1, k2yz, kz == 0 || kz == a.M, acc});
+            with_radix<MAX>(R2, ColEnergy{xs + k1 * pitch + p, a.k2x + k1, R1, k2yz, kz == 0 || kz == a.M, acc});
     }
     // fixed-order sum of the CTA (its last warp may be partial)
     const int lane = threadIdx.x & 31, live = min(32, (int)blockDim.x - (int)(threadIdx.x & ~31));
@@ -182,9 +189,10 @@ __global__ void __launch_bounds__(BIG ? 256 : 128, BIG ? 2 : 5) mx_energy_kernel
 
 template <int MODE>
 static auto mx_x_pick(int R1, int R2) {
-    return R2 > 16   ? mixed::mx_x_kernel<MODE, true, true>
-           : R1 > 16 ? mixed::mx_x_kernel<MODE, true, false>
-                     : mixed::mx_x_kernel<MODE, false, false>;
+    return R2 > 16   ? mixed::mx_x_kernel<MODE, 32, 32>
+           : R1 > 20 ? mixed::mx_x_kernel<MODE, 32, 16>
+           : R1 > 16 ? mixed::mx_x_kernel<MODE, 20, 16>
+                     : mixed::mx_x_kernel<MODE, 16, 16>;
 }
 
 bool mixed_xupdate(const XUpdArgs& a, cudaStream_t st, cudaError_t* err) {
@@ -204,7 +212,7 @@ bool mixed_xenergy(const XEnergyArgs& a, cudaStream_t st, cudaError_t* err) {
     int R1, R2;
     if (!mixed_split(a.L, &R1, &R2)) return false;
     const size_t smem = sizeof(float2) * R1 * (R2 | 1) * SP;
-    auto kern = R1 > 16 ? mixed::mx_energy_kernel<true> : mixed::mx_energy_kernel<false>;
+    auto kern = R1 > 16 ? mixed::mx_energy_kernel<32> : mixed::mx_energy_kernel<16>;
     if ((*err = mx_smem(kern, smem)) != cudaSuccess) return true;
     kern<<<dim3(a.nchunks, a.ny), R1 * SP, smem, st>>>(a, R1, R2);
     *err = cudaGetLastError();

@@ -4,8 +4,8 @@
 namespace evx {
 namespace mixed {
 
-template <int DIR, bool BIG>
-__global__ void __launch_bounds__(BIG ? 256 : 128, BIG ? 2 : 8) mx_y_kernel(SPassArgs a, int R1, int R2) {
+template <int DIR, int MAX>
+__global__ void __launch_bounds__(8 * MAX, MAX <= 16 ? 8 : MAX <= 20 ? 5 : 2) mx_y_kernel(SPassArgs a, int R1, int R2) {
     extern __shared__ float4 smem4[];
     float2* xb = reinterpret_cast<float2*>(smem4);
     const int p = threadIdx.x & 7, it = threadIdx.x >> 3, T = blockDim.x >> 3;
@@ -14,11 +14,11 @@ __global__ void __launch_bounds__(BIG ? 256 : 128, BIG ? 2 : 8) mx_y_kernel(SPas
     const long long base = (long long)blockIdx.y * a.os + (long long)blockIdx.x * CP + p;
     if (valid)
         for (int n2 = it; n2 < R2; n2 += T)
-            with_radix<BIG>(R1, ColLoad<DIR>{a.in + base + n2 * a.rs, R2 * a.rs, xb + n2 * CP + p, R2p * CP, a.tw, n2});
+            with_radix<MAX>(R1, ColLoad<DIR>{a.in + base + n2 * a.rs, R2 * a.rs, xb + n2 * CP + p, R2p * CP, a.tw, n2});
     __syncthreads();
     if (valid)
         for (int k1 = it; k1 < R1; k1 += T)
-            with_radix<BIG>(R2, ColStore<DIR>{a.out + base + k1 * a.rs, R1 * a.rs, xb + k1 * R2p * CP + p});
+            with_radix<MAX>(R2, ColStore<DIR>{a.out + base + k1 * a.rs, R1 * a.rs, xb + k1 * R2p * CP + p});
 }
 
 }  // namespace mixed
@@ -47,8 +47,9 @@ bool mixed_spass(const SPassArgs& a, int dir, cudaStream_t st, cudaError_t* err)
     int R1, R2;
     if (!plain_rows(a.YB, a.L) || !mixed_split(a.L, &R1, &R2)) return false;
     const size_t smem = sizeof(float2) * R1 * (R2 | 1) * SP;
-    auto kern = R1 > 16 ? (dir < 0 ? mixed::mx_y_kernel<-1, true> : mixed::mx_y_kernel<1, true>)
-                        : (dir < 0 ? mixed::mx_y_kernel<-1, false> : mixed::mx_y_kernel<1, false>);
+    auto kern = R1 > 20   ? (dir < 0 ? mixed::mx_y_kernel<-1, 32> : mixed::mx_y_kernel<1, 32>)
+                : R1 > 16 ? (dir < 0 ? mixed::mx_y_kernel<-1, 20> : mixed::mx_y_kernel<1, 20>)
+                          : (dir < 0 ? mixed::mx_y_kernel<-1, 16> : mixed::mx_y_kernel<1, 16>);
     if ((*err = mx_smem(kern, smem)) != cudaSuccess) return true;
     kern<<<dim3(a.nchunks, a.nouter), R1 * SP, smem, st>>>(a, R1, R2);
     *err = cudaGetLastError();

@@ -173,8 +173,8 @@ struct ZFwdA {
     }
 };
 
-template <int MODE, bool BIG>
-__global__ void __launch_bounds__(BIG ? 256 : 192, BIG ? 2 : 3) mx_z_kernel(ZPassArgs a, int R1, int R2, int RS) {
+template <int MODE, int MAX>
+__global__ void __launch_bounds__(MAX > 16 ? 256 : 192, MAX > 16 ? 2 : MAX > 12 ? 3 : 4) mx_z_kernel(ZPassArgs a, int R1, int R2, int RS) {
     extern __shared__ float4 smem4[];
     float2* buf = reinterpret_cast<float2*>(smem4);
     const int tx = threadIdx.x, ty = threadIdx.y, T = blockDim.x, RPC = blockDim.y, M = a.M;
@@ -201,13 +201,13 @@ __global__ void __launch_bounds__(BIG ? 256 : 192, BIG ? 2 : 3) mx_z_kernel(ZPas
     const bool actA = rowok && tx < R2, actB = rowok;  // T = R1
     float gs = 0.f, ge = 0.f;
     if (MODE == Z_R2C) {
-        with_radix<BIG>(R2, ZFwdB{z, cb, cbl, tx, actB});
+        with_radix<MAX>(R2, ZFwdB{z, cb, cbl, tx, actB});
         __syncthreads();
     } else {
-        with_radix<BIG>(R1, ZInvA{z, tx, actA});
+        with_radix<MAX>(R1, ZInvA{z, tx, actA});
         __syncthreads();
         if (MODE == Z_C2R) {
-            with_radix<BIG>(R2, ZInvB{z, a.scale, cb, cbl, tx, actB});
+            with_radix<MAX>(R2, ZInvB{z, a.scale, cb, cbl, tx, actB});
             __syncthreads();
             if (a.partials) {  // energy: nothing is written
                 double acc = 0.0;
@@ -232,15 +232,27 @@ __global__ void __launch_bounds__(BIG ? 256 : 192, BIG ? 2 : 3) mx_z_kernel(ZPas
             if (rowok) {
                 const long long ur = a.map_rows ? user_row(row, a.YB, a.nxr, a.nyr) : row;
                 float2* dst = reinterpret_cast<float2*>(a.rout + ur * a.rpitch);
-                for (int q = tx; q < M; q += T) dst[q] = a.accumulate ? cadd(dst[q], z.row[q]) : z.row[q];
+                if (a.accumulate) {  // eight reads in flight
+                    for (int q = tx; q < M; q += 8 * T) {
+                        float2 prev[8];
+#pragma unroll
+                        for (int u = 0; u < 8; ++u)
+                            if (q + u * T < M) prev[u] = dst[q + u * T];
+#pragma unroll
+                        for (int u = 0; u < 8; ++u)
+                            if (q + u * T < M) dst[q + u * T] = cadd(prev[u], z.row[q + u * T]);
+                    }
+                } else {
+                    for (int q = tx; q < M; q += T) dst[q] = z.row[q];
+                }
             }
             return;
         }
         const float gp = a.nl_only ? 0.f : (float)(3.0 * cbd * cbd - 1.0), c3 = (float)(3.0 * cbd);
-        if (actB) with_radix<BIG>(R2, ZMiddle<MODE == Z_ADJ>{z, a, tx, row, rowok, cb, cbl, gp, c3, gs, ge});
+        if (actB) with_radix<MAX>(R2, ZMiddle<MODE == Z_ADJ>{z, a, tx, row, rowok, cb, cbl, gp, c3, gs, ge});
         __syncthreads();
     }
-    with_radix<BIG>(R1, ZFwdA{z, tx, actA});
+    with_radix<MAX>(R1, ZFwdA{z, tx, actA});
     __syncthreads();
     // R2C post-processing, pairs (k, M - k)
     if (rowok) {
@@ -306,15 +318,18 @@ bool mixed_zpass(const ZPassArgs& a, int mode, cudaStream_t st, cudaError_t* err
     const int RS = mixed_zstride(a, R1, R2), rpc = mixed_zrows(a, R1, RS);
     const int grid = (int)((a.nrows + rpc - 1) / rpc);
     const size_t smem = sizeof(float2) * RS * rpc;
-    const bool big = R1 > 16;
+    auto pick = [&](auto small, auto mid, auto big) { return R1 > 16 ? big : R1 > 12 ? mid : small; };
     void (*kern)(ZPassArgs, int, int, int) = nullptr;
+#define EVX_MX_Z(MODE) \
+    case MODE: kern = pick(mixed::mx_z_kernel<MODE, 12>, mixed::mx_z_kernel<MODE, 16>, mixed::mx_z_kernel<MODE, 32>); break;
     switch (mode) {
-        case Z_STEP: kern = big ? mixed::mx_z_kernel<Z_STEP, true> : mixed::mx_z_kernel<Z_STEP, false>; break;
-        case Z_ADJ: kern = big ? mixed::mx_z_kernel<Z_ADJ, true> : mixed::mx_z_kernel<Z_ADJ, false>; break;
-        case Z_R2C: kern = big ? mixed::mx_z_kernel<Z_R2C, true> : mixed::mx_z_kernel<Z_R2C, false>; break;
-        case Z_C2R: kern = big ? mixed::mx_z_kernel<Z_C2R, true> : mixed::mx_z_kernel<Z_C2R, false>; break;
+        EVX_MX_Z(Z_STEP)
+        EVX_MX_Z(Z_ADJ)
+        EVX_MX_Z(Z_R2C)
+        EVX_MX_Z(Z_C2R)
         default: return false;
     }
+#undef EVX_MX_Z
     if ((*err = mx_smem(kern, smem)) != cudaSuccess) return true;
     if (grid_used) *grid_used = grid;
     kern<<<grid, dim3(R1, rpc), smem, st>>>(a, R1, R2, RS);
