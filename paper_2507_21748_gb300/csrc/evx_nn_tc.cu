@@ -157,11 +157,11 @@ __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::be
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 // bias + fused epilogue on NCH (a multiple of 8) channels c0 .. of voxel vox,
-// r = FP32 accumulator bits, bias = the NCH biases (registers); BF16 stores
-// of 16 bytes
+// r = FP32 accumulator bits, bias = the NCH biases (registers), pf = the voxel's
+// pre-activations (GELU_BWD), loaded ahead; BF16 stores of 16 bytes
 template <int EPI, int NCH>
 __device__ __forceinline__ void epilogue_store(const ConvArgs& a, long long vox, int c0, const uint32_t* r,
-                                               const float* bias) {
+                                               const float* bias, const uint4* pf) {
     const long long o = vox * 32 + c0;
 #pragma unroll
     for (int q = 0; q < NCH / 8; ++q) {
@@ -180,7 +180,7 @@ __device__ __forceinline__ void epilogue_store(const ConvArgs& a, long long vox,
             }
             if (a.pre) *reinterpret_cast<uint4*>(a.pre + o + q * 8) = pw;  // NULL: inference, not kept
         } else if (EPI == EVX_NN_EPI_GELU_BWD) {
-            const uint4 pw = *reinterpret_cast<const uint4*>(a.pre + o + q * 8);
+            const uint4 pw = pf[q];
             const __nv_bfloat162* pp = reinterpret_cast<const __nv_bfloat162*>(&pw);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -195,17 +195,6 @@ __device__ __forceinline__ void epilogue_store(const ConvArgs& a, long long vox,
                 const float2 rf = __bfloat1622float2(rp[j]);
                 ow[j] = __floats2bfloat162_rn(v[2 * j] + rf.x, v[2 * j + 1] + rf.y);
             }
-        } else if (EPI == EVX_NN_EPI_RESID32) {  // FP32 stream in a.pre, updated in place
-            float4* sp = reinterpret_cast<float4*>(reinterpret_cast<float*>(a.pre) + o + q * 8);
-            float4 s0 = sp[0], s1 = sp[1];
-            s0.x += v[0], s0.y += v[1], s0.z += v[2], s0.w += v[3];
-            s1.x += v[4], s1.y += v[5], s1.z += v[6], s1.w += v[7];
-            sp[0] = s0;
-            sp[1] = s1;
-            ow[0] = __floats2bfloat162_rn(s0.x, s0.y);
-            ow[1] = __floats2bfloat162_rn(s0.z, s0.w);
-            ow[2] = __floats2bfloat162_rn(s1.x, s1.y);
-            ow[3] = __floats2bfloat162_rn(s1.z, s1.w);
         } else {
 #pragma unroll
             for (int j = 0; j < 4; ++j) ow[j] = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
@@ -219,9 +208,15 @@ __device__ __forceinline__ void epilogue_store(const ConvArgs& a, long long vox,
 // 16-byte chunk c of row v at chunk c ^ ((v >> 1) & 3): conflict-free both ways) and
 // the stream is read and written with lane l on voxel l / 4 + 8 i, channels
 // c0 + 4 (l % 4) ..: every instruction covers 8 whole 64-byte row pieces instead of
-// one 16-byte piece of 32 rows.
+// one 16-byte piece of 32 rows. s: the stream's values, loaded ahead by resid32_load.
+__device__ __forceinline__ void resid32_load(const ConvArgs& a, long long vox0, int c0, int lane, float4 (&s)[4]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        s[i] = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(a.pre) +
+                                                (vox0 + (lane >> 2) + 8 * i) * 32 + c0 + 4 * (lane & 3));
+}
 __device__ __forceinline__ void resid32_staged(const ConvArgs& a, long long vox0, int c0, const uint32_t* acc,
-                                               const float* bias, float* stg, int lane) {
+                                               const float* bias, float* stg, int lane, float4 (&s)[4]) {
 #pragma unroll
     for (int q = 0; q < 4; ++q)
         *reinterpret_cast<float4*>(stg + lane * 16 + 4 * (q ^ ((lane >> 1) & 3))) =
@@ -230,12 +225,6 @@ __device__ __forceinline__ void resid32_staged(const ConvArgs& a, long long vox0
                         __uint_as_float(acc[4 * q + 3]) + bias[4 * q + 3]);
     __syncwarp();
     const int c = lane & 3;
-    float4 s[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int v = (lane >> 2) + 8 * i;
-        s[i] = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(a.pre) + (vox0 + v) * 32 + c0 + 4 * c);
-    }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int v = (lane >> 2) + 8 * i;
@@ -261,8 +250,12 @@ constexpr int NS = 5;                      // ring slots (one input row each)
 constexpr int SLOT = 3 * RUN;              // bytes per slot: runs for x-1, x, x+1
 constexpr int WB = 9 * 12 * 4 * 128;       // staged weights: [dx][dz][n/8 (12)][ci/8][8 n][8 ci]
 constexpr int NBLK = 16;                   // accumulator blocks of 32 columns (a ring over output rows)
-constexpr int NEPI = 8;                    // epilogue warps
-constexpr int NTH = (2 + NEPI) * 32;
+constexpr int NEPI = 8;                    // epilogue warps of a group
+// groups of epilogue warps, which take alternate output rows: two for the GELU-backward
+// epilogue, whose arithmetic and loads set the pace (8 x 256^3: 12.3 ms with one group, 8.2
+// with two and its pre-activations loaded ahead). GELU is slower with two (8.3 -> 8.7).
+__host__ __device__ constexpr int groups(int epi) { return epi == EVX_NN_EPI_GELU_BWD ? 2 : 1; }
+__host__ __device__ constexpr int threads(int epi) { return (2 + NEPI * groups(epi)) * 32; }
 constexpr int BAR = WB + NS * SLOT;        // barriers: full[NS], tfull[NBLK], tempty[NBLK]
 constexpr int STG = (BAR + 8 * (NS + 2 * NBLK) + 16 + 15) & ~15;  // after the tensor-memory slot and abort flag
 constexpr int STG_WARP = 32 * 16 * 4;      // per epilogue warp: [32 voxels][16 channels] FP32 staging
@@ -354,7 +347,7 @@ __device__ __forceinline__ void tmem_st16_zero(uint32_t taddr) {
 // WX: columns are walked along x and may end in a 64-voxel chunk (a template parameter: as
 // run-time values the two forms cost the Z % 128 = 0 convolutions 4 to 9%)
 template <int EPI, bool WX>
-__global__ void __launch_bounds__(ring::NTH, 1)
+__global__ void __launch_bounds__(ring::threads(EPI), 1)
     conv_ring_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap hmap, RingArgs r) {
     using namespace ring;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -371,7 +364,7 @@ __global__ void __launch_bounds__(ring::NTH, 1)
     // weights [t][co][ci] -> [dx][dz][n = 32 (dy+1) + co][ci]: one input row feeds the output rows
     // y' + 1 (dy = -1), y' (dy = 0), y' - 1 (dy = +1) through N = 96 stacked columns (walking x:
     // x and y change places)
-    for (int e = threadIdx.x; e < 9 * 96 * 4; e += NTH) {
+    for (int e = threadIdx.x; e < 9 * 96 * 4; e += threads(EPI)) {
         const int kg = e & 3, n = (e >> 2) % 96, dd = e / (96 * 4), dxi = dd / 3, dzi = dd % 3;
         const int t = WX ? 9 * (n >> 5) + 3 * dxi + dzi : 9 * dxi + 3 * (n >> 5) + dzi, co = n & 31;
         const uint4 v = *reinterpret_cast<const uint4*>(a.w + (t * 32 + co) * 32 + kg * 8);
@@ -397,7 +390,7 @@ __global__ void __launch_bounds__(ring::NTH, 1)
     __syncthreads();
     fence_after();
     const uint32_t tmem = *tslot;
-    if (warp >= 2) {  // every accumulator block starts at zero; the MMAs only accumulate
+    if (warp >= 2 && warp < 2 + NEPI) {  // every accumulator block starts at zero; the MMAs only accumulate
         const uint32_t tq = tmem + ((uint32_t)((warp & 3) * 32) << 16) + ((warp - 2) >> 2) * 16;
         for (int c = 0; c < NBLK; ++c) tmem_st16_zero(tq + c * 32);
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
@@ -473,14 +466,17 @@ __global__ void __launch_bounds__(ring::NTH, 1)
                 // blocks are claimed 8 rows at a time (rows up to V+i+9, freed by the epilogue
                 // once it has read rows up to V+i-7), so the tensor-memory fence that orders
                 // the epilogue's reads before these MMAs runs once per 8 input rows. Every
-                // epilogue warp frees rows in order, so the phase of the last claimed block
-                // (row V+i-7 freed by all warps) implies the earlier ones: one probe, not 8,
-                // of a barrier the tensor core's operand reads make slow to reach.
+                // epilogue warp frees its rows in order, so the phase of the last claimed block
+                // (row V+i-7 freed by all warps of its group) implies the group's earlier ones:
+                // one probe per group, not 8, of a barrier the tensor core's operand reads make
+                // slow to reach.
                 const bool claim = V + i + 2 > vready;
                 uint32_t w_ok = 1;
                 if (lane == 0) {
                     const uint32_t vc = V + i + 9;
                     if (claim) w_ok = ring_wait(tempty + 8 * ring_blk(vc), ((vc / NBLK) & 1) ^ 1, abort_flag);
+                    if (groups(EPI) == 2 && claim && w_ok)  // the other group's last claimed row
+                        w_ok = ring_wait(tempty + 8 * ring_blk(vc - 1), (((vc - 1) / NBLK) & 1) ^ 1, abort_flag);
                     if (w_ok) w_ok = ring_wait(full + 8 * (k % NS), (k / NS) & 1, abort_flag);
                 }
                 if (!__shfl_sync(0xffffffffu, w_ok, 0)) {
@@ -534,12 +530,18 @@ __global__ void __launch_bounds__(ring::NTH, 1)
         __syncwarp();
     } else {
         // --------------------------------------------------------- epilogue
-        const int q4 = warp & 3, h = (warp - 2) >> 2;  // accumulator lanes 32 q4 .., columns 16 h ..
+        // Virtual row v belongs to group v mod G. The FP32 stream and the pre-activations of
+        // GELU' are loaded one row of the group ahead (RESID32 9.9 -> 9.25 ms at 8 x 256^3; the
+        // BF16 residuals of RESID gain nothing: 6.6 -> 7.2).
+        constexpr int G = groups(EPI);
+        constexpr bool STREAM = EPI == EVX_NN_EPI_RESID32, AHEAD = EPI == EVX_NN_EPI_GELU_BWD;
+        const int q4 = warp & 3, h = ((warp - 2) & 7) >> 2;  // accumulator lanes 32 q4 .., columns 16 h ..
+        const uint32_t grp = G == 2 ? (warp - 2) >> 3 : 0;
         float* stg = reinterpret_cast<float*>(sm + STG + (warp - 2) * STG_WARP);
         float bias[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) bias[i] = a.bias ? a.bias[h * 16 + i] : 0.f;
-        uint32_t v = 0;
+        uint32_t V = 0;
         bool ok = true;
         for (int u = blockIdx.x; u < r.nunits && ok; u += gridDim.x) {
             int bx, z0, ys, ye;
@@ -548,9 +550,28 @@ __global__ void __launch_bounds__(ring::NTH, 1)
             // voxel of the row's lane 0 and the distance to the next row's
             const long long row0 = WX ? ((long long)(bx / Y) * X + ys) * Y + bx % Y : (long long)bx * Y + ys;
             const long long step = WX ? (long long)Y * Z : Z;
-            long long vox0 = row0 * Z + z0 + q4 * 32 - 2 * step;  // of virtual row jv = 0
-            for (int jv = 0; jv < L + 4; ++jv, ++v, vox0 += step) {
-                const uint32_t blk = ring_blk(v);
+            const int j0 = G == 2 ? (int)((grp - V) & 1) : 0;
+            long long vox0 = row0 * Z + z0 + q4 * 32 + (j0 - 2) * step;  // of virtual row jv
+            // rows that are stored; a half chunk's lanes 64 .. are not voxels
+            auto stored = [&](int j) { return j >= 2 && j < L + 2 && (!WX || z0 + q4 * 32 < Z); };
+            uint4 pf[2], pfn[2];
+            float4 sf[4], sfn[4];
+            for (int jv = j0; jv < L + 4; jv += G, vox0 += G * step) {
+                const uint32_t v = V + jv, blk = ring_blk(v);
+                if (AHEAD || STREAM) {  // (the first stored row of a group is never its first row)
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) pf[i] = pfn[i];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) sf[i] = sfn[i];
+                    if (stored(jv + G)) {
+                        const long long vn = vox0 + G * step;
+                        if (STREAM) resid32_load(a, vn, h * 16, lane, sfn);
+                        if (AHEAD)
+#pragma unroll
+                            for (int i = 0; i < 2; ++i)
+                                pfn[i] = *reinterpret_cast<const uint4*>(a.pre + (vn + lane) * 32 + h * 16 + 8 * i);
+                    }
+                }
                 uint32_t w_ok = 1;
                 if (lane == 0) w_ok = ring_wait(tfull + 8 * blk, (v / NBLK) & 1, abort_flag);
                 if (!__shfl_sync(0xffffffffu, w_ok, 0)) {
@@ -567,13 +588,14 @@ __global__ void __launch_bounds__(ring::NTH, 1)
                 fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(tempty + 8 * blk);
-                if (jv >= 2 && jv < L + 2 && (!WX || z0 + q4 * 32 < Z)) {  // a half chunk's lanes 64 .. are not voxels
-                    if (EPI == EVX_NN_EPI_RESID32)
-                        resid32_staged(a, vox0, h * 16, acc, bias, stg, lane);
+                if (stored(jv)) {
+                    if constexpr (STREAM)
+                        resid32_staged(a, vox0, h * 16, acc, bias, stg, lane, sf);
                     else
-                        epilogue_store<EPI, 16>(a, vox0 + lane, h * 16, acc, bias);
+                        epilogue_store<EPI, 16>(a, vox0 + lane, h * 16, acc, bias, pf);
                 }
             }
+            V += (uint32_t)L + 4;
         }
     }
     fence_before();
@@ -865,7 +887,7 @@ cudaError_t launch_walk(const ConvArgs& a, cudaStream_t st, int sms) {
     cudaError_t e =
         cudaFuncSetAttribute(conv_ring_kernel<EPI, WX>, cudaFuncAttributeMaxDynamicSharedMemorySize, ring::SMEM);
     if (e != cudaSuccess) return e;
-    conv_ring_kernel<EPI, WX><<<std::min(r.nunits, sms), ring::NTH, ring::SMEM, st>>>(map, hmap, r);
+    conv_ring_kernel<EPI, WX><<<std::min(r.nunits, sms), ring::threads(EPI), ring::SMEM, st>>>(map, hmap, r);
     return cudaGetLastError();
 }
 
