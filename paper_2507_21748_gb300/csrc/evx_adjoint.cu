@@ -144,6 +144,7 @@ __global__ void __launch_bounds__(NT, 1) xadj_kernel(XAdjArgs a) {
 // out[0] += scale * sum(partials[0..n)), deterministic order
 __global__ void __launch_bounds__(1024) accum_partials_kernel(const double* partials, int n,
                                                                double* out, double scale) {
+    chain_wait();
     __shared__ double ws[32];
     double acc = 0.0;
     for (int i = threadIdx.x; i < n; i += 1024) acc += partials[i];
@@ -361,9 +362,8 @@ extern "C" evx_status evx_ch_adjoint(evx_grid* g, const float* d_c0, int n_steps
                 fe = cudaGetLastError();
             }
             CKA(fe);
-            accum_partials_kernel<<<1, 1024, 0, sst>>>(A->part, xg, A->d_acc + 0, 1.0 / V);
-            accum_partials_kernel<<<1, 1024, 0, sst>>>(A->part + xg, xg, A->d_acc + 1, 1.0 / V);
-            CKA(cudaGetLastError());
+            CKA(launch_chained(accum_partials_kernel, 1, 1024, 0, sst, A->part, xg, A->d_acc + 0, 1.0 / V));
+            CKA(launch_chained(accum_partials_kernel, 1, 1024, 0, sst, A->part + xg, xg, A->d_acc + 1, 1.0 / V));
             CKA(launch_spass(y_args(g, g->W, g->W), +1, sst));
             ZPassArgs z = z_args(g);
             z.in = g->W;

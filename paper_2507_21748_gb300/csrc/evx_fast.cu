@@ -49,6 +49,7 @@ __global__ void __launch_bounds__(NTZ, 512 / NTZ) fzstep_kernel(ZPassArgs a, int
     if (tile >= ntiles) return;
     fill_twiddles<R1, TP>(tA, tB, a.tw, NTZ);
     for (int i = threadIdx.x; i <= M; i += NTZ) rtws[i] = a.rtw[i];
+    chain_wait();
     // rows to warps, 16-byte pieces of a row to lanes (no division by the runtime pitch)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     auto issue = [&](int tl) {
@@ -180,6 +181,7 @@ __global__ void __launch_bounds__(NTZ, 512 / NTZ) fr2c_kernel(ZPassArgs a, int n
     if (tile >= ntiles) return;
     fill_twiddles<R1, TP>(tA, tB, a.tw, NTZ);
     for (int i = threadIdx.x; i <= M; i += NTZ) rtws[i] = a.rtw[i];
+    chain_wait();
     // rows to warps (the caller's row once per row), 16-byte chunks of 4 floats to lanes
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     auto issue = [&](int tl) {
@@ -256,6 +258,7 @@ __global__ void __launch_bounds__(NTZ, 512 / NTZ) fc2r_kernel(ZPassArgs a, int n
         fill_twiddles<R1, TP>(tA, tB, a.tw, NTZ);
         for (int i = threadIdx.x; i <= M; i += NTZ) rtws[i] = a.rtw[i];
     }
+    chain_wait();
     // rows to warps, 16-byte pieces of a row to lanes (no division by the runtime pitch)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     auto issue = [&](int tl) {
@@ -466,6 +469,7 @@ __global__ void __launch_bounds__(8 * TP) fspass_tma_kernel(SPassArgs a, int nti
         for (int b = 0; b < NBUF; ++b) mbar_init(bar + b, 1);
         s_abort = 0;
     }
+    chain_wait();
     __syncthreads();
     auto issue = [&](int tl, int b) {
         const int outer = tl / nchunks, chunk = tl - outer * nchunks;
@@ -555,6 +559,7 @@ __global__ void __launch_bounds__(8 * TP, SEP ? 1 : (8 * TP >= 128 ? 3 : 1))
         mbar_init(bars + 1, 1);
         s_abort = 0;
     }
+    chain_wait();
     __syncthreads();
     const int YB = a.YB;
     auto issue = [&](const CUtensorMap* m, float2* buf, uint64_t* bar, int tl) {
@@ -710,6 +715,7 @@ __global__ void __launch_bounds__(8 * TP) fxadj_kernel(XAdjArgs a) {
     float2* tA = xb + (L + TP) * P;
     float2* tB = NB == 1 ? tA : tA + L;
     fill_twiddles<R1, TP>(tA, tB, a.tw, NT);
+    chain_wait();
     __shared__ double red[2][NT / 32 + 1];
     const int p = threadIdx.x % P, n2 = threadIdx.x / P;
     const int chunk = blockIdx.x, ky = blockIdx.y;
@@ -917,8 +923,7 @@ static bool run_fspass_tma(const SPassArgs& a, cudaStream_t st, cudaError_t* err
     }
     const int ntiles = a.nchunks * a.nouter;
     const int grid = std::min(ntiles, per * num_sms());
-    fast::fspass_tma_kernel<R1, TP, DIR, NBUF><<<grid, 8 * TP, smem, st>>>(a, ntiles, mi, mo);
-    *err = cudaGetLastError();
+    *err = launch_chained(fast::fspass_tma_kernel<R1, TP, DIR, NBUF>, grid, 8 * TP, smem, st, a, ntiles, mi, mo);
     return true;
 }
 
@@ -949,8 +954,7 @@ static bool run_fxupd_tma(const XUpdArgs& a, cudaStream_t st, cudaError_t* err) 
     }
     const int ntiles = a.nchunks * a.ny;
     const int grid = std::min(ntiles, per * num_sms());
-    kern<<<grid, 8 * TP, smem, st>>>(a, ntiles, mw, ms, mo);
-    *err = cudaGetLastError();
+    *err = launch_chained(kern, grid, 8 * TP, smem, st, a, ntiles, mw, ms, mo);
     return true;
 }
 
@@ -1005,8 +1009,7 @@ static cudaError_t run_fzstep(const ZPassArgs& a, cudaStream_t st, int* grid_use
     const int ntiles = (int)((a.nrows + RPC - 1) / RPC);
     const int grid = std::min(ntiles, per * num_sms());
     if (grid_used) *grid_used = grid;
-    kern<<<grid, NTZ, smem, st>>>(a, ntiles);
-    return cudaGetLastError();
+    return launch_chained(kern, grid, NTZ, smem, st, a, ntiles);
 }
 
 template <int R1, int TP>
@@ -1026,8 +1029,7 @@ static cudaError_t run_fzconv(const ZPassArgs& a, int dir, cudaStream_t st, int*
     if (e != cudaSuccess) return e;
     const int grid = std::min(ntiles, per * num_sms());
     if (grid_used) *grid_used = grid;
-    kern<<<grid, NTZ, smem, st>>>(a, ntiles);
-    return cudaGetLastError();
+    return launch_chained(kern, grid, NTZ, smem, st, a, ntiles);
 }
 
 // z R2C (dir < 0) or C2R (dir > 0) alone; false when the fast kernels do not apply
@@ -1051,8 +1053,7 @@ static cudaError_t run_fxadj(const XAdjArgs& a, cudaStream_t st) {
     int per = 0;
     cudaError_t e = prep(fast::fxadj_kernel<R1, TP>, smem, 8 * TP, &per);
     if (e != cudaSuccess) return e;
-    fast::fxadj_kernel<R1, TP><<<dim3(a.nchunks, a.ny), 8 * TP, smem, st>>>(a);
-    return cudaGetLastError();
+    return launch_chained(fast::fxadj_kernel<R1, TP>, dim3(a.nchunks, a.ny), 8 * TP, smem, st, a);
 }
 
 bool fast_xadj(const XAdjArgs& a, cudaStream_t st, cudaError_t* err) {

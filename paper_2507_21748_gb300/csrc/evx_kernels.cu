@@ -371,6 +371,7 @@ __global__ void __launch_bounds__(NT, 2) zpass_kernel(ZPassArgs a) {
 // partials[b] = sum over rows b, b + nblocks, ... of sum_z c[row * pitch + z]
 __global__ void __launch_bounds__(NT) sum_rows_kernel(const float* c, long long nrows, int rowlen,
                                                       long long pitch, double* partials) {
+    chain_wait();
     __shared__ double ws[NT / 32];
     double acc = 0.0;
     for (long long r = blockIdx.x; r < nrows; r += gridDim.x) {
@@ -395,6 +396,7 @@ __device__ __forceinline__ void two_sum_acc(float& s, float& e, float x) {
 }
 __global__ void __launch_bounds__(NT) sum_rows_vec_kernel(const float* c, long long nrows, int rowlen,
                                                           long long pitch, double* partials) {
+    chain_wait();
     __shared__ double ws[NT / 32];
     const int lane = threadIdx.x & 31;
     const long long nw = ((long long)gridDim.x * NT) >> 5;
@@ -425,6 +427,7 @@ __global__ void __launch_bounds__(NT) sum_rows_vec_kernel(const float* c, long l
 // x-sum of its (ky = 0, kz = 0) line: removing it subtracts the line's mean
 // from each of its n elements (stride apart). One block, FP64 sum.
 __global__ void __launch_bounds__(1024) remove_k0_kernel(float2* line, int n, long long stride) {
+    chain_wait();
     __shared__ double ws[32];
     __shared__ double mre, mim;
     double sr = 0.0, si = 0.0;
@@ -452,6 +455,7 @@ __global__ void __launch_bounds__(1024) remove_k0_kernel(float2* line, int n, lo
 
 __global__ void __launch_bounds__(1024) reduce_partials_kernel(const double* partials, int n,
                                                                 double* out, double scale) {
+    chain_wait();
     __shared__ double ws[32];
     double acc = 0.0;
     for (int i = threadIdx.x; i < n; i += 1024) acc += partials[i];
@@ -554,6 +558,7 @@ __device__ __forceinline__ void vm_cp_async(float* dst, const float* src) {
 }
 __global__ void __launch_bounds__(VM_NT, 2) vm_fd_kernel(const float* __restrict__ c, float* __restrict__ rhs, int nx,
                                                          int ny, int nz, int xc, float kh2, float M0, float ih2) {
+    chain_wait();
     extern __shared__ __align__(16) float vm_smem[];
     float* cs = vm_smem;               // [4][VM_CY][VM_CZ]
     float* ms = cs + 4 * VM_CP;        // [2][VM_MY][VM_MZ] mu
@@ -730,6 +735,7 @@ __global__ void __launch_bounds__(256) vm_energy_kernel(const float* __restrict_
 // cbar' = cbar - dt L mean(g(c)), mean(g(c)) = g(cbar) + sum(g(c) - g(cbar)) / V
 __global__ void __launch_bounds__(1024) ac_mean_kernel(const double* gsum, int n, double* cbar, double dtL,
                                                         double invV) {
+    chain_wait();
     __shared__ double ws[32];
     double acc = 0.0;
     for (int i = threadIdx.x; i < n; i += 1024) acc += gsum[i];
@@ -741,6 +747,7 @@ __global__ void __launch_bounds__(1024) ac_mean_kernel(const double* gsum, int n
 }
 
 __global__ void cadd_kernel(const float2* a, const float2* b, float2* out, long long n) {
+    chain_wait();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)
         out[i] = cadd(a[i], b[i]);
@@ -870,10 +877,8 @@ cudaError_t launch_zpass(const ZPassArgs& a, int mode, cudaStream_t st, int* gri
 cudaError_t launch_sum_field(const float* c, long long nrows, int rowlen, long long pitch,
                              double* partials, int nblocks, cudaStream_t st) {
     if (rowlen % 4 == 0 && pitch % 4 == 0 && ((uintptr_t)c & 15) == 0)
-        sum_rows_vec_kernel<<<nblocks, NT, 0, st>>>(c, nrows, rowlen, pitch, partials);
-    else
-        sum_rows_kernel<<<nblocks, NT, 0, st>>>(c, nrows, rowlen, pitch, partials);
-    return cudaGetLastError();
+        return launch_chained(sum_rows_vec_kernel, nblocks, NT, 0, st, c, nrows, rowlen, pitch, partials);
+    return launch_chained(sum_rows_kernel, nblocks, NT, 0, st, c, nrows, rowlen, pitch, partials);
 }
 
 static int vm_grid(int nx, int ny) {
@@ -903,8 +908,8 @@ cudaError_t launch_vm_fd(const float* c, float* rhs, int nx, int ny, int nz, flo
     // x chunks of 64 planes (each loads 4 more), shorter while the launch would leave SMs idle
     int xc = 64;
     while (xc > 8 && (long long)ty * tz * ((nx + xc - 1) / xc) < 2 * 152) xc /= 2;
-    vm_fd_kernel<<<dim3(ty, tz, (nx + xc - 1) / xc), VM_NT, VM_SMEM, st>>>(c, rhs, nx, ny, nz, xc, kappa_h2, M0, inv_h2);
-    return cudaGetLastError();
+    return launch_chained(vm_fd_kernel, dim3(ty, tz, (nx + xc - 1) / xc), VM_NT, VM_SMEM, st, c, rhs, nx, ny, nz, xc, kappa_h2,
+                          M0, inv_h2);
 }
 
 cudaError_t launch_vm_rhs(const float* c, const float* mu, float* rhs, int nx, int ny, int nz, float M0,
@@ -925,25 +930,21 @@ cudaError_t launch_vm_energy(const float* c, int nx, int ny, int nz, double kapp
 int vm_energy_grid(int nx, int ny, int nparts) { return std::min(vm_grid(nx, ny), nparts); }
 
 cudaError_t launch_ac_mean(const double* gsum, int n, double* cbar, double dtL, double invV, cudaStream_t st) {
-    ac_mean_kernel<<<1, 1024, 0, st>>>(gsum, n, cbar, dtL, invV);
-    return cudaGetLastError();
+    return launch_chained(ac_mean_kernel, 1, 1024, 0, st, gsum, n, cbar, dtL, invV);
 }
 
 cudaError_t launch_remove_k0(float2* line, int n, long long stride, cudaStream_t st) {
-    remove_k0_kernel<<<1, 1024, 0, st>>>(line, n, stride);
-    return cudaGetLastError();
+    return launch_chained(remove_k0_kernel, 1, 1024, 0, st, line, n, stride);
 }
 
 cudaError_t launch_reduce_partials(const double* partials, int n, double* out, double scale,
                                    cudaStream_t st) {
-    reduce_partials_kernel<<<1, 1024, 0, st>>>(partials, n, out, scale);
-    return cudaGetLastError();
+    return launch_chained(reduce_partials_kernel, 1, 1024, 0, st, partials, n, out, scale);
 }
 
 cudaError_t launch_cadd(const float2* a, const float2* b, float2* out, long long n,
                         cudaStream_t st) {
-    cadd_kernel<<<SUM_BLOCKS, NT, 0, st>>>(a, b, out, n);
-    return cudaGetLastError();
+    return launch_chained(cadd_kernel, SUM_BLOCKS, NT, 0, st, a, b, out, n);
 }
 
 }  // namespace evx

@@ -86,6 +86,7 @@ struct ColUpdate {
 // M1, M2: largest radices of R1 and R2
 template <int MODE, int M1, int M2>
 __global__ void __launch_bounds__(8 * M1, M1 <= 16 ? 5 : M1 <= 20 ? 4 : 2) mx_x_kernel(XUpdArgs a, int R1, int R2) {
+    chain_wait();
     extern __shared__ float4 smem4[];
     const int p = threadIdx.x & 7, it = threadIdx.x >> 3, T = blockDim.x >> 3;
     const int R2p = R2 | 1, pitch = R2p * CP;
@@ -150,6 +151,7 @@ struct ColEnergy {
 };
 template <int MAX>
 __global__ void __launch_bounds__(8 * MAX, MAX <= 16 ? 5 : 2) mx_energy_kernel(XEnergyArgs a, int R1, int R2) {
+    chain_wait();
     extern __shared__ float4 smem4[];
     __shared__ double red[8];
     float2* xs = reinterpret_cast<float2*>(smem4);
@@ -201,8 +203,7 @@ bool mixed_xupdate(const XUpdArgs& a, cudaStream_t st, cudaError_t* err) {
     const size_t smem = sizeof(float2) * R1 * (R2 | 1) * SP * (a.model == 2 ? 1 : 2);
     auto kern = a.model == 3 ? mx_x_pick<3>(R1, R2) : a.model == 2 ? mx_x_pick<2>(R1, R2) : mx_x_pick<0>(R1, R2);
     if ((*err = mx_smem(kern, smem)) != cudaSuccess) return true;
-    kern<<<dim3(a.nchunks, a.ny), R1 * SP, smem, st>>>(a, R1, R2);
-    *err = cudaGetLastError();
+    *err = launch_chained(kern, dim3(a.nchunks, a.ny), R1 * SP, smem, st, a, R1, R2);
     return true;
 }
 
@@ -214,8 +215,7 @@ bool mixed_xenergy(const XEnergyArgs& a, cudaStream_t st, cudaError_t* err) {
     const size_t smem = sizeof(float2) * R1 * (R2 | 1) * SP;
     auto kern = R1 > 16 ? mixed::mx_energy_kernel<32> : mixed::mx_energy_kernel<16>;
     if ((*err = mx_smem(kern, smem)) != cudaSuccess) return true;
-    kern<<<dim3(a.nchunks, a.ny), R1 * SP, smem, st>>>(a, R1, R2);
-    *err = cudaGetLastError();
+    *err = launch_chained(kern, dim3(a.nchunks, a.ny), R1 * SP, smem, st, a, R1, R2);
     return true;
 }
 

@@ -6,6 +6,7 @@ namespace mixed {
 
 template <int DIR, int MAX>
 __global__ void __launch_bounds__(8 * MAX, MAX <= 16 ? 8 : MAX <= 20 ? 5 : 2) mx_y_kernel(SPassArgs a, int R1, int R2) {
+    chain_wait();
     extern __shared__ float4 smem4[];
     float2* xb = reinterpret_cast<float2*>(smem4);
     const int p = threadIdx.x & 7, it = threadIdx.x >> 3, T = blockDim.x >> 3;
@@ -51,8 +52,7 @@ bool mixed_spass(const SPassArgs& a, int dir, cudaStream_t st, cudaError_t* err)
                 : R1 > 16 ? (dir < 0 ? mixed::mx_y_kernel<-1, 20> : mixed::mx_y_kernel<1, 20>)
                           : (dir < 0 ? mixed::mx_y_kernel<-1, 16> : mixed::mx_y_kernel<1, 16>);
     if ((*err = mx_smem(kern, smem)) != cudaSuccess) return true;
-    kern<<<dim3(a.nchunks, a.nouter), R1 * SP, smem, st>>>(a, R1, R2);
-    *err = cudaGetLastError();
+    *err = launch_chained(kern, dim3(a.nchunks, a.nouter), R1 * SP, smem, st, a, R1, R2);
     return true;
 }
 

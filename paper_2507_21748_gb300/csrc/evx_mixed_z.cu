@@ -175,6 +175,7 @@ struct ZFwdA {
 
 template <int MODE, int MAX>
 __global__ void __launch_bounds__(MAX > 16 ? 256 : 192, MAX > 16 ? 2 : MAX > 12 ? 3 : 4) mx_z_kernel(ZPassArgs a, int R1, int R2, int RS) {
+    chain_wait();
     extern __shared__ float4 smem4[];
     float2* buf = reinterpret_cast<float2*>(smem4);
     const int tx = threadIdx.x, ty = threadIdx.y, T = blockDim.x, RPC = blockDim.y, M = a.M;
@@ -332,8 +333,7 @@ bool mixed_zpass(const ZPassArgs& a, int mode, cudaStream_t st, cudaError_t* err
 #undef EVX_MX_Z
     if ((*err = mx_smem(kern, smem)) != cudaSuccess) return true;
     if (grid_used) *grid_used = grid;
-    kern<<<grid, dim3(R1, rpc), smem, st>>>(a, R1, R2, RS);
-    *err = cudaGetLastError();
+    *err = launch_chained(kern, grid, dim3(R1, rpc), smem, st, a, R1, R2, RS);
     return true;
 }
 

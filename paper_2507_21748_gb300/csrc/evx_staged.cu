@@ -129,6 +129,7 @@ struct TrailToGlobal {
 
 template <int DIR>
 __global__ void __launch_bounds__(256, 3) stg_y_kernel(SPassArgs a, Cut c) {
+    chain_wait();
     extern __shared__ float4 smem4[];
     float2* xb = reinterpret_cast<float2*>(smem4);
     const int p = threadIdx.x & 7, it = threadIdx.x >> 3;
@@ -233,6 +234,7 @@ struct LeadFromRows {
 };
 
 __global__ void __launch_bounds__(256, 2) stg_x_kernel(XUpdArgs a, Cut c) {
+    chain_wait();
     extern __shared__ float4 smem4[];
     const int p = threadIdx.x & 7, it = threadIdx.x >> 3;
     const int ky = blockIdx.y, kz = (int)blockIdx.x * CP + p;
@@ -393,6 +395,7 @@ struct LeadNatural {
 
 template <int MODE>
 __global__ void __launch_bounds__(256, 2) stg_z_kernel(ZPassArgs a, Cut c, int RS) {
+    chain_wait();
     extern __shared__ float4 smem4[];
     float2* buf = reinterpret_cast<float2*>(smem4);
     __shared__ double red[256];
@@ -519,8 +522,7 @@ bool staged_spass(const SPassArgs& a, int dir, cudaStream_t st, cudaError_t* err
     if (!a.small || a.YB != a.L || !staged_cut(a.plan, a.L, &c)) return false;
     const size_t smem = sizeof(float2) * c.R1 * c.R2p * SP;  // at most 128 x 33 / 32 rows of 64 B: 9 KB
     auto kern = dir < 0 ? staged::stg_y_kernel<-1> : staged::stg_y_kernel<1>;
-    kern<<<dim3(a.nchunks, a.nouter), std::max(c.R1, c.R2) * SP, smem, st>>>(a, c);
-    *err = cudaGetLastError();
+    *err = launch_chained(kern, dim3(a.nchunks, a.nouter), std::max(c.R1, c.R2) * SP, smem, st, a, c);
     return true;
 }
 
@@ -528,8 +530,7 @@ bool staged_xupdate(const XUpdArgs& a, cudaStream_t st, cudaError_t* err) {
     staged::Cut c;
     if (!a.small || !a.W || !staged_cut(a.plan, a.L, &c)) return false;
     const size_t smem = 2 * sizeof(float2) * c.R1 * c.R2p * SP;
-    staged::stg_x_kernel<<<dim3(a.nchunks, a.ny), std::max(c.R1, c.R2) * SP, smem, st>>>(a, c);
-    *err = cudaGetLastError();
+    *err = launch_chained(staged::stg_x_kernel, dim3(a.nchunks, a.ny), std::max(c.R1, c.R2) * SP, smem, st, a, c);
     return true;
 }
 
@@ -564,8 +565,7 @@ bool staged_zpass(const ZPassArgs& a, int mode, cudaStream_t st, cudaError_t* er
                 : mode == Z_R2C ? staged::stg_z_kernel<Z_R2C>
                                 : staged::stg_z_kernel<Z_C2R>;
     if (grid_used) *grid_used = grid;
-    kern<<<grid, dim3(T, rpc), sizeof(float2) * RS * rpc, st>>>(a, c, RS);
-    *err = cudaGetLastError();
+    *err = launch_chained(kern, grid, dim3(T, rpc), sizeof(float2) * RS * rpc, st, a, c, RS);
     return true;
 }
 
