@@ -141,12 +141,13 @@ __global__ void __launch_bounds__(NT, 1) xadj_kernel(XAdjArgs a) {
     if (threadIdx.x == 0) a.partials[nblk + blk] = acc_m;
 }
 
-// out[0] += scale * sum(partials[0..n)), deterministic order
+// CTA b: out[b] += scale * sum(partials[b n .. (b + 1) n)), deterministic order
 __global__ void __launch_bounds__(1024) accum_partials_kernel(const double* partials, int n,
                                                                double* out, double scale) {
     chain_wait();
     __shared__ double ws[32];
     double acc = 0.0;
+    partials += (long long)blockIdx.x * n;
     for (int i = threadIdx.x; i < n; i += 1024) acc += partials[i];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
@@ -156,7 +157,7 @@ __global__ void __launch_bounds__(1024) accum_partials_kernel(const double* part
         acc = ws[threadIdx.x];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-        if (threadIdx.x == 0) *out += acc * scale;
+        if (threadIdx.x == 0) out[blockIdx.x] += acc * scale;
     }
 }
 
@@ -350,8 +351,13 @@ extern "C" evx_status evx_ch_adjoint(evx_grid* g, const float* d_c0, int n_steps
             if (r != EVX_OK) return r;
         }
         for (int j = n - 1; j >= 0; --j) {
+            // the fast x pass reads Lambda as the two parts the step before left, P and W
+            // (nothing else of a segment's adjoint steps uses them), so the sum is formed
+            // once per segment instead of in a pass of its own per step
+            const bool parts = fast_xadj_length(g->nx) && j != n - 1;
             XAdjArgs x = xa;
-            x.Lam = A->Lam;
+            x.Lam = parts ? A->P : A->Lam;
+            x.Lam2 = parts ? g->W : nullptr;
             x.Sn1 = A->Sn[j];
             x.Gn = A->G[j];
             x.P = A->P;
@@ -362,8 +368,7 @@ extern "C" evx_status evx_ch_adjoint(evx_grid* g, const float* d_c0, int n_steps
                 fe = cudaGetLastError();
             }
             CKA(fe);
-            CKA(launch_chained(accum_partials_kernel, 1, 1024, 0, sst, A->part, xg, A->d_acc + 0, 1.0 / V));
-            CKA(launch_chained(accum_partials_kernel, 1, 1024, 0, sst, A->part + xg, xg, A->d_acc + 1, 1.0 / V));
+            CKA(launch_chained(accum_partials_kernel, 2, 1024, 0, sst, A->part, xg, A->d_acc, 1.0 / V));
             CKA(launch_spass(y_args(g, g->W, g->W), +1, sst));
             ZPassArgs z = z_args(g);
             z.in = g->W;
@@ -372,7 +377,7 @@ extern "C" evx_status evx_ch_adjoint(evx_grid* g, const float* d_c0, int n_steps
             z.cnpitch = g->nz;
             CKA(launch_zpass(z, Z_ADJ, sst));
             CKA(launch_spass(y_args(g, g->W, g->W), -1, sst));
-            CKA(launch_cadd(A->P, g->W, A->Lam, nspec, sst));
+            if (j == 0 || !fast_xadj_length(g->nx)) CKA(launch_cadd(A->P, g->W, A->Lam, nspec, sst));
         }
         return EVX_OK;
     };

@@ -725,10 +725,13 @@ __global__ void __launch_bounds__(8 * TP) fxadj_kernel(XAdjArgs a) {
     const float k2yz = a.k2y[ky] + (valid ? a.k2z[kz] : 0.f);
     const float w = (kz == 0 || kz == a.M) ? 1.f : 2.f;
     __syncthreads();
-    auto forward = [&](const float2* f, float2 (&v)[R1]) {
+    auto forward = [&](const float2* f, const float2* f2, float2 (&v)[R1]) {
 #pragma unroll
         for (int n1 = 0; n1 < R1; ++n1)
             v[n1] = valid ? f[base + (long long)(n2 + TP * n1) * a.rs] : make_float2(0.f, 0.f);
+        if (f2 && valid)
+#pragma unroll
+            for (int n1 = 0; n1 < R1; ++n1) v[n1] = cadd(v[n1], f2[base + (long long)(n2 + TP * n1) * a.rs]);
         Dft<R1, -1>::run(v);
         twiddle_a<R1, TP, -1>(v, n2, tA);
         __syncthreads();  // earlier reads of xb done
@@ -746,9 +749,9 @@ __global__ void __launch_bounds__(8 * TP) fxadj_kernel(XAdjArgs a) {
             for (int n1 = 0; n1 < R1; ++n1) out[base + (long long)(n2 + TP * n1) * a.rs] = v[n1];
     };
     float2 lam[R1], v[R1];
-    forward(a.Lam, lam);
+    forward(a.Lam, a.Lam2, lam);
     float acck = 0.f, accm = 0.f;
-    forward(a.Sn1, v);
+    forward(a.Sn1, nullptr, v);
 #pragma unroll
     for (int i = 0; i < NB; ++i)
 #pragma unroll
@@ -760,7 +763,7 @@ __global__ void __launch_bounds__(8 * TP) fxadj_kernel(XAdjArgs a) {
             acck = fmaf(re, -a.dtM * k4 * Dinv, acck);
             accm = fmaf(re, -a.dtk * k4 * Dinv, accm);
         }
-    forward(a.Gn, v);
+    forward(a.Gn, nullptr, v);
 #pragma unroll
     for (int i = 0; i < NB; ++i)
 #pragma unroll
@@ -1056,6 +1059,9 @@ static cudaError_t run_fxadj(const XAdjArgs& a, cudaStream_t st) {
     return launch_chained(fast::fxadj_kernel<R1, TP>, dim3(a.nchunks, a.ny), 8 * TP, smem, st, a);
 }
 
+bool fast_xadj_length(int L) {
+    return fast_paths_enabled() && (L == 64 || L == 128 || L == 256 || L == 512 || L == 1024 || L == 400);
+}
 bool fast_xadj(const XAdjArgs& a, cudaStream_t st, cudaError_t* err) {
     if (!fast_paths_enabled() || a.os * a.YB != a.rs) return false;
     switch (a.L) {

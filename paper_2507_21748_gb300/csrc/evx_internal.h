@@ -122,7 +122,8 @@ struct XUpdArgs {
 // Lambda_{n+1}, S_{n+1} and G_n, P = F_x^-1(a lambda_hat)/nx, T = F_x^-1(b lambda_hat)/nx
 // and per-CTA FP64 partials of the two parameter gradients.
 struct XAdjArgs {
-    const float2* Lam;   // Lambda_{n+1}
+    const float2* Lam;   // Lambda_{n+1}, or with Lam2 its first part: Lambda_{n+1} = Lam + Lam2
+    const float2* Lam2;  // or null; Lam may be P and Lam2 may be T (a CTA reads its columns before it writes them)
     const float2* Sn1;   // S_{n+1}
     const float2* Gn;    // G_n
     float2* P;
@@ -259,6 +260,7 @@ bool fast_xupdate(const XUpdArgs& a, cudaStream_t st, cudaError_t* err);
 bool fast_zstep(const ZPassArgs& a, cudaStream_t st, cudaError_t* err, int* grid_used, bool adj = false);
 // adjoint x pass with the four-step transforms; false if the length has no fast kernel
 bool fast_xadj(const XAdjArgs& a, cudaStream_t st, cudaError_t* err);
+bool fast_xadj_length(int L);
 bool fast_zconv(const ZPassArgs& a, int dir, cudaStream_t st, cudaError_t* err, int* grid_used);
 bool fast_paths_enabled();  // false when the environment sets EVX_GENERIC=1
 // grids whose mixed-radix passes run with grouped stages (evx_staged.cu), bit for bit
