@@ -41,6 +41,8 @@ __device__ __forceinline__ void ldsm_x2_trans(uint32_t& r0, uint32_t& r1, const 
 }
 
 
+__device__ __forceinline__ int wrapi(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
+
 // load the halo rows (x+dx, y0-1 .. y0+TY) x (z0-1 .. z0+TZ), periodic, into
 // s[HR][TZ+2][C+8] (pitch C+8 halves: conflict-free fragment loads); halo
 // row index (dx+1) * (TY+2) + (y - y0 + 1)
@@ -52,7 +54,9 @@ __device__ __forceinline__ void load_halo(__nv_bfloat16* s, const __nv_bfloat16*
     for (int e = threadIdx.x; e < n; e += nthreads) {
         const int q = e % V16, rem = e / V16, zi = rem % (TZ + 2), nb = rem / (TZ + 2);
         const int dx = nb / (TY + 2) - 1, yi = nb % (TY + 2) - 1;
-        const int xx = (x + dx + X) % X, yy = (y0 + yi + Y) % Y, zz = (z0 + zi - 1 + Z) % Z;
+        // one step beyond an edge at most: a comparison each (three divisions by run-time sizes per
+        // 16-byte piece made the copy dearer than the tile's MMAs)
+        const int xx = wrapi(x + dx, X), yy = wrapi(y0 + yi, Y), zz = wrapi(z0 + zi - 1, Z);
         const long long vox = (((long long)b * X + xx) * Y + yy) * Z + zz;
         const uint4 val = *reinterpret_cast<const uint4*>(g + vox * C + q * 8);
         *reinterpret_cast<uint4*>(s + (nb * (TZ + 2) + zi) * P + q * 8) = val;
@@ -786,7 +790,6 @@ __global__ void __launch_bounds__(256) project_direct_kernel(const __nv_bfloat16
 // of a voxel is one coalesced row of its 32 channels, and each input row segment
 // is read once per warp for all the outputs it feeds (3 dz taps along z, up to
 // 3 dy taps across the RY rows). Needs Z % 32 = 0 and Y % RY = 0.
-__device__ __forceinline__ int wrapi(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
 
 // lane l ends with the lane sum of v[l] (a butterfly that halves the values per step)
 __device__ __forceinline__ float lane_sum_transpose(float (&v)[32], int lane) {
