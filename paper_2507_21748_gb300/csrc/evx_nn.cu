@@ -12,6 +12,7 @@
 #include <cuda_bf16.h>
 
 #include <atomic>
+#include <climits>
 #include <cstdlib>
 #include <cstdint>
 
@@ -785,12 +786,12 @@ __global__ void __launch_bounds__(256) project_direct_kernel(const __nv_bfloat16
 }
 
 // ---------------------------------------------------------------------------
-// Lift and projection with one warp per RY x 32 outputs of a (b, x) plane
+// Projection of BF16 activations with one warp per RY x 32 outputs of a (b, x) plane
 // (rows y0 .. y0 + RY - 1, z0 .. z0 + 31) and lane = channel: every global access
 // of a voxel is one coalesced row of its 32 channels, and each input row segment
 // is read once per warp for all the outputs it feeds (3 dz taps along z, up to
-// 3 dy taps across the RY rows). Needs Z % 32 = 0 and Y % RY = 0.
-
+// 3 dy taps across the RY rows). Needs Z % 32 = 0 and Y % RY = 0. (The FP32 stream's
+// projection walks x: evx_nn_tc.cu.)
 // lane l ends with the lane sum of v[l] (a butterfly that halves the values per step)
 __device__ __forceinline__ float lane_sum_transpose(float (&v)[32], int lane) {
 #pragma unroll
@@ -819,9 +820,8 @@ __device__ __forceinline__ bool lane_unit(long long u, int X, int Y, int Z, int&
 }
 
 // out(v) = bias(0) + sum_t sum_ci w[t][0][ci] h(v + off_t, ci); lane = ci
-template <bool F32, int RY, int MINB>
+template <int RY, int MINB>
 __global__ void __launch_bounds__(256, MINB) project_lane_kernel(const __nv_bfloat16* __restrict__ h,
-                                                            const float* __restrict__ h32,
                                                             const __nv_bfloat16* __restrict__ w, int wcout,
                                                             const float* __restrict__ bias, float* out, int B,
                                                             int X, int Y, int Z) {
@@ -849,19 +849,11 @@ __global__ void __launch_bounds__(256, MINB) project_lane_kernel(const __nv_bflo
             for (int yy = 0; yy < RY + 2; ++yy) {
                 const long long row = (((long long)b * X + xx) * Y + wrapi(y0 + yy - 1, Y)) * Z;
                 float hv[34];
-                if (F32) {
-                    const float* rp = h32 + (row + z0) * 32 + lane;  // z0 + j - 1 at rp[(j - 1) 32]
-                    hv[0] = __ldg(h32 + (row + zl) * 32 + lane);
+                const __nv_bfloat16* rp = h + (row + z0) * 32 + lane;
+                hv[0] = __bfloat162float(h[(row + zl) * 32 + lane]);
 #pragma unroll
-                    for (int j = 1; j < 33; ++j) hv[j] = __ldg(rp + (j - 1) * 32);
-                    hv[33] = __ldg(h32 + (row + zh) * 32 + lane);
-                } else {
-                    const __nv_bfloat16* rp = h + (row + z0) * 32 + lane;
-                    hv[0] = __bfloat162float(h[(row + zl) * 32 + lane]);
-#pragma unroll
-                    for (int j = 1; j < 33; ++j) hv[j] = __bfloat162float(rp[(j - 1) * 32]);
-                    hv[33] = __bfloat162float(h[(row + zh) * 32 + lane]);
-                }
+                for (int j = 1; j < 33; ++j) hv[j] = __bfloat162float(rp[(j - 1) * 32]);
+                hv[33] = __bfloat162float(h[(row + zh) * 32 + lane]);
 #pragma unroll
                 for (int r = 0; r < RY; ++r) {
                     const int dy = yy - r;  // tap 9 dx + 3 dy + dz  // input row y0 + yy - 1 = output row y0 + r + dy - 1
@@ -884,46 +876,80 @@ __global__ void __launch_bounds__(256, MINB) project_lane_kernel(const __nv_bflo
 }
 
 // out(v, co) = bias(co) + sum_t w[t][co][0] val(f(v + off_t)), val = scale f (F32) or its
-// BF16 rounding; lane = co. F32 also writes the FP32 copy out32.
-template <bool F32, int RY, int MINB>
-__global__ void __launch_bounds__(256, MINB) lift_lane_kernel(const float* __restrict__ f, float scale,
-                                                         const __nv_bfloat16* __restrict__ w, int wcin,
-                                                         const float* __restrict__ bias, __nv_bfloat16* out,
-                                                         float* __restrict__ out32, int B, int X, int Y, int Z) {
+// BF16 rounding; lane = co. F32 also writes the FP32 copy out32. A CTA's 8 warps cover a
+// tile of 16 / ZW rows x 32 ZW columns of one (b, x) plane, whose 3 x (rows + 2) x
+// (columns + 2) inputs are copied to shared memory one tile ahead: a lane reads its 34
+// neighbours as 16-byte broadcasts. (Distributing them by 34 shuffles per input row bound the kernel by
+// the shuffle pipe: 10.4 ms at 8 x 256^3, 7.7 now; its stores alone take 3.8 ms.)
+constexpr int LIFT_PLANE = 816;  // floats per staged plane: at least (rows + 2) x pitch for ZW = 1, 2, 4
+template <bool F32>
+__global__ void __launch_bounds__(256, 2) lift_tile_kernel(const float* __restrict__ f, float scale,
+                                                           const __nv_bfloat16* __restrict__ w, int wcin,
+                                                           const float* __restrict__ bias, __nv_bfloat16* out,
+                                                           float* __restrict__ out32, int B, int X, int Y, int Z, int ZW,
+                                                           int ntiles) {
     __shared__ float ws[27][32];  // w[t][co][0]
+    __shared__ __align__(16) float st[2][3 * LIFT_PLANE];  // two tiles; row pitch 32 ZW + 8: z0 - 1 at 3, z0 at 4
     for (int i = threadIdx.x; i < 27 * 32; i += blockDim.x) ws[i >> 5][i & 31] = __bfloat162float(w[i * wcin]);
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int rows = 16 / ZW, cols = 32 * ZW, pitch = cols + 8;
+    const int wy = 2 * (warp / ZW), wz = 32 * (warp % ZW);
     const float bl = bias ? bias[lane] : 0.f;
-    const long long units = (long long)B * X * (Y / RY) * (Z >> 5);
-    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
-    for (long long u = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < units; u += nw) {
+    const int nzt = Z / cols, nyt = (Y + rows - 1) / rows;
+    auto place = [&](int tile, int& b, int& x, int& y0, int& z0) {
+        z0 = (tile % nzt) * cols;
+        int c = tile / nzt;
+        y0 = (c % nyt) * rows;
+        c /= nyt;
+        x = c % X, b = c / X;
+    };
+    auto load = [&](int tile, float* buf) {  // an input row to a warp, four bytes to a lane
         int b, x, y0, z0;
-        lane_unit<RY>(u, X, Y, Z, b, x, y0, z0);
-        float acc[RY][32];
+        place(tile, b, x, y0, z0);
+        for (int rr = warp; rr < 3 * (rows + 2); rr += 8) {
+            const int dx = rr / (rows + 2), yy = rr - dx * (rows + 2);
+            const float* src = f + (((long long)b * X + wrapi(x + dx - 1, X)) * Y + (y0 + yy - 1 + Y) % Y) * Z;
+            const unsigned dst = (unsigned)__cvta_generic_to_shared(buf + dx * LIFT_PLANE + yy * pitch + 3);
+            for (int i = lane; i < cols + 2; i += 32)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + 4 * i), "l"(src + wrapi(z0 - 1 + i, Z))
+                             : "memory");
+        }
+    };
+    if ((int)blockIdx.x < ntiles) load(blockIdx.x, st[0]);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    int cur = 0;
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, cur ^= 1) {
+        int b, x, y0, z0;
+        place(tile, b, x, y0, z0);
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();  // the tile has arrived; the other buffer's has been read (and the weights are staged)
+        if (tile + (int)gridDim.x < ntiles) load(tile + gridDim.x, st[cur ^ 1]);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        if (y0 + wy >= Y) continue;  // Y is even: both rows or none
+        float acc[2][32];
 #pragma unroll
-        for (int r = 0; r < RY; ++r)
-#pragma unroll
-            for (int j = 0; j < 32; ++j) acc[r][j] = bl;
+        for (int j = 0; j < 32; ++j) acc[0][j] = acc[1][j] = bl;
 #pragma unroll 1
         for (int dx = 0; dx < 3; ++dx) {
-            const int xx = wrapi(x + dx - 1, X);
-#pragma unroll 1
-            for (int yy = 0; yy < RY + 2; ++yy) {
-                const long long row = (((long long)b * X + xx) * Y + wrapi(y0 + yy - 1, Y)) * Z;
-                // lane l holds z0 - 1 + l; lanes 0, 1 also z0 + 31, z0 + 32
-                float f0 = scale * f[row + wrapi(z0 - 1 + lane, Z)];
-                float f1 = lane < 2 ? scale * f[row + wrapi(z0 + 31 + lane, Z)] : 0.f;
-                if (!F32) {
-                    f0 = __bfloat162float(__float2bfloat16_rn(f0));
-                    f1 = __bfloat162float(__float2bfloat16_rn(f1));
-                }
+#pragma unroll
+            for (int yy = 0; yy < 4; ++yy) {
+                const float* row = st[cur] + dx * LIFT_PLANE + (wy + yy) * pitch + wz;
                 float hv[34];
+                hv[0] = row[3];
 #pragma unroll
-                for (int j = 0; j < 34; ++j)
-                    hv[j] = j < 32 ? __shfl_sync(0xffffffffu, f0, j) : __shfl_sync(0xffffffffu, f1, j - 32);
+                for (int q = 0; q < 8; ++q) {
+                    const float4 v = *reinterpret_cast<const float4*>(row + 4 + 4 * q);
+                    hv[1 + 4 * q] = v.x, hv[2 + 4 * q] = v.y, hv[3 + 4 * q] = v.z, hv[4 + 4 * q] = v.w;
+                }
+                hv[33] = row[36];
+                if (!F32 || scale != 1.f)
 #pragma unroll
-                for (int r = 0; r < RY; ++r) {
+                    for (int j = 0; j < 34; ++j) {
+                        hv[j] *= scale;
+                        if (!F32) hv[j] = __bfloat162float(__float2bfloat16_rn(hv[j]));
+                    }
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
                     const int dy = yy - r;  // tap 9 dx + 3 dy + dz
                     if (dy < 0 || dy > 2) continue;
 #pragma unroll
@@ -936,8 +962,8 @@ __global__ void __launch_bounds__(256, MINB) lift_lane_kernel(const float* __res
             }
         }
 #pragma unroll
-        for (int r = 0; r < RY; ++r) {
-            const long long v0 = (((long long)b * X + x) * Y + y0 + r) * Z + z0;
+        for (int r = 0; r < 2; ++r) {
+            const long long v0 = (((long long)b * X + x) * Y + y0 + wy + r) * Z + z0 + wz;
 #pragma unroll
             for (int j = 0; j < 32; ++j) {
                 out[(v0 + j) * 32 + lane] = __float2bfloat16_rn(acc[r][j]);
@@ -1038,6 +1064,19 @@ evx_status launch_wgrad(const WgradArgs& a0, float* dw, float* partials, size_t 
     return nn_cuda(cudaGetLastError());
 }
 
+int lift_zw(int Z) { return Z % 128 == 0 ? 4 : Z % 64 == 0 ? 2 : 1; }
+long long lift_tiles(int B, int X, int Y, int Z) {
+    const int zw = lift_zw(Z), rows = 16 / zw;
+    return (long long)B * X * ((Y + rows - 1) / rows) * (Z / (32 * zw));
+}
+template <bool F32>
+void launch_lift(const float* f, float scale, const void* w, int cin, const float* bias, void* out, float* out32, int B,
+                        int X, int Y, int Z, cudaStream_t st) {
+    const int ntiles = (int)lift_tiles(B, X, Y, Z);
+    lift_tile_kernel<F32><<<std::min(ntiles, 2 * nn_sms()), 256, 0, st>>>(
+        f, scale, (const __nv_bfloat16*)w, cin, bias, (__nv_bfloat16*)out, out32, B, X, Y, Z, lift_zw(Z), ntiles);
+}
+
 }  // namespace
 
 extern "C" {
@@ -1090,9 +1129,9 @@ evx_status evx_nn_conv3d(const void* in, const void* w, const float* bias, void*
     return nn_fail(EVX_ERR_ARG, "supported channel pairs: 16/32 -> 16/32");
 }
 
-// the lane-per-channel lift and projection: RY = 2 rows x 32 z per warp, two
-// 256-thread CTAs per SM (measured at 8 x 256^3: projection 10.6 ms against 13.2 for
-// one row per warp and 16.1 with one CTA per SM; lift 10.4 against 12.6 for one row)
+// the lane-per-channel projection of BF16 activations: RY = 2 rows x 32 z per warp, two
+// 256-thread CTAs per SM (measured at 8 x 256^3: 10.6 ms against 13.2 for one row per warp
+// and 16.1 with one CTA per SM)
 constexpr int LANE_RY = 2;
 static bool lane_path(int Y, int Z) { return Z % 32 == 0 && Y % LANE_RY == 0; }
 static int lane_grid(int B, int X, int Y, int Z) {
@@ -1105,9 +1144,8 @@ evx_status evx_nn_lift(const float* f, float scale, const void* w, int cin, int 
     if (!f || !w || !out) return nn_fail(EVX_ERR_ARG, "NULL pointer");
     if (B <= 0 || X <= 0 || Y <= 0 || Z <= 0) return nn_fail(EVX_ERR_SIZE, "empty grid");
     if (cout != 32 || cin < 1) return nn_fail(EVX_ERR_ARG, "lift: cout must be 32, cin >= 1");
-    if (lane_path(Y, Z))
-        lift_lane_kernel<false, LANE_RY, 2><<<lane_grid(B, X, Y, Z), 256, 0, (cudaStream_t)stream>>>(
-            f, scale, (const __nv_bfloat16*)w, cin, bias, (__nv_bfloat16*)out, nullptr, B, X, Y, Z);
+    if (lane_path(Y, Z) && lift_tiles(B, X, Y, Z) <= INT_MAX)
+        launch_lift<false>(f, scale, w, cin, bias, out, nullptr, B, X, Y, Z, (cudaStream_t)stream);
     else
         lift_direct_kernel<false><<<8 * nn_sms(), 256, 0, (cudaStream_t)stream>>>(
             f, scale, (const __nv_bfloat16*)w, cin, bias, (__nv_bfloat16*)out, nullptr, B, X, Y, Z);
@@ -1119,9 +1157,8 @@ evx_status evx_nn_lift32(const float* f, float scale, const void* w, int cin, in
     if (!f || !w || !out || !out32) return nn_fail(EVX_ERR_ARG, "NULL pointer");
     if (B <= 0 || X <= 0 || Y <= 0 || Z <= 0) return nn_fail(EVX_ERR_SIZE, "empty grid");
     if (cout != 32 || cin < 1) return nn_fail(EVX_ERR_ARG, "lift: cout must be 32, cin >= 1");
-    if (lane_path(Y, Z))
-        lift_lane_kernel<true, LANE_RY, 2><<<lane_grid(B, X, Y, Z), 256, 0, (cudaStream_t)stream>>>(
-            f, scale, (const __nv_bfloat16*)w, cin, bias, (__nv_bfloat16*)out, out32, B, X, Y, Z);
+    if (lane_path(Y, Z) && lift_tiles(B, X, Y, Z) <= INT_MAX)
+        launch_lift<true>(f, scale, w, cin, bias, out, out32, B, X, Y, Z, (cudaStream_t)stream);
     else
         lift_direct_kernel<true><<<8 * nn_sms(), 256, 0, (cudaStream_t)stream>>>(
             f, scale, (const __nv_bfloat16*)w, cin, bias, (__nv_bfloat16*)out, out32, B, X, Y, Z);
@@ -1134,8 +1171,8 @@ evx_status evx_nn_project(const void* h, const void* w, int cin, int cout, const
     if (B <= 0 || X <= 0 || Y <= 0 || Z <= 0) return nn_fail(EVX_ERR_SIZE, "empty grid");
     if (cin != 32 || cout < 1) return nn_fail(EVX_ERR_ARG, "project: cin must be 32, cout >= 1");
     if (lane_path(Y, Z))
-        project_lane_kernel<false, LANE_RY, 2><<<lane_grid(B, X, Y, Z), 256, 0, (cudaStream_t)stream>>>(
-            (const __nv_bfloat16*)h, nullptr, (const __nv_bfloat16*)w, cout, bias, out, B, X, Y, Z);
+        project_lane_kernel<LANE_RY, 2><<<lane_grid(B, X, Y, Z), 256, 0, (cudaStream_t)stream>>>(
+            (const __nv_bfloat16*)h, (const __nv_bfloat16*)w, cout, bias, out, B, X, Y, Z);
     else
         project_direct_kernel<false><<<8 * nn_sms(), 256, 0, (cudaStream_t)stream>>>(
             (const __nv_bfloat16*)h, nullptr, (const __nv_bfloat16*)w, cout, bias, out, B, X, Y, Z);
@@ -1147,9 +1184,9 @@ evx_status evx_nn_project32(const float* h32, const void* w, int cin, int cout, 
     if (!h32 || !w || !out) return nn_fail(EVX_ERR_ARG, "NULL pointer");
     if (B <= 0 || X <= 0 || Y <= 0 || Z <= 0) return nn_fail(EVX_ERR_SIZE, "empty grid");
     if (cin != 32 || cout < 1) return nn_fail(EVX_ERR_ARG, "project: cin must be 32, cout >= 1");
-    if (lane_path(Y, Z))
-        project_lane_kernel<true, LANE_RY, 2><<<lane_grid(B, X, Y, Z), 256, 0, (cudaStream_t)stream>>>(
-            nullptr, h32, (const __nv_bfloat16*)w, cout, bias, out, B, X, Y, Z);
+    if (lane_path(Y, Z) && ((uintptr_t)h32 & 15) == 0)
+        return nn_cuda(project32_walk(h32, (const __nv_bfloat16*)w, cout, bias, out, B, X, Y, Z, (cudaStream_t)stream,
+                                      nn_sms()));
     else
         project_direct_kernel<true><<<8 * nn_sms(), 256, 0, (cudaStream_t)stream>>>(
             nullptr, h32, (const __nv_bfloat16*)w, cout, bias, out, B, X, Y, Z);
