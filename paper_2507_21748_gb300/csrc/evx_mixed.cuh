@@ -19,7 +19,7 @@
 // inverse walks back through the same slots with one barrier per exchange.
 //
 // Measured on a GB300 against the stage-by-stage kernels, 300 x 240 x 200: y pass
-// 137 -> 21 us (5.5 TB/s), z pass 237 -> 61 us, x pass 620 -> 74 us; 48 x 40 x 36:
+// 137 -> 21 us (5.5 TB/s), z pass 237 -> 55 us, x pass 620 -> 62 us; 48 x 40 x 36:
 // y 10.9 -> 3.6, z 56 -> 8, x 26 -> 8 us. The y pass is bound by memory, the z and
 // x passes by instruction issue and their barriers.
 #pragma once

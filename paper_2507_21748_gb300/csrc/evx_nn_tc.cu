@@ -43,7 +43,7 @@
 // producer loads 64-row boxes, the MMAs still run with M = 128 (the upper lanes
 // accumulate stale rows, and are zeroed and not stored). Half of such a chunk's
 // tensor work is idle, but an unpipelined kernel with 2 x 64 voxel tiles took
-// 740 us where this takes 180 us (4 x 64^3, GELU epilogue).
+// 740 us where this takes 170 us (4 x 64^3, GELU epilogue).
 //
 // Every mbarrier wait is bounded (about 1 s); a wait that runs out sets the
 // device flag g_tc_timeout, makes the other roles stop, waits (bounded) for
@@ -620,7 +620,7 @@ __global__ void __launch_bounds__(ring::threads(EPI), 1)
 // rows each count in full (the halo is on the dY rows: 8 of the 38 KB a row
 // loads). The mma.sync kernel it replaces for 32 -> 32 re-read its fragments from
 // shared memory for every tap: 382 us at 64 x 96 x 128 and 3.71 ms at 4 x 128^3 with the
-// sum of the partials, this kernel 102 us and 0.62 ms (error against 64 bits unchanged).
+// sum of the partials, this kernel 76 us and 0.61 ms (error against 64 bits unchanged).
 //   warp 0 producer, warp 1 MMA issuer, warps 2..5 write the CTA's partial sums.
 namespace wg {
 constexpr int NS = 4;                        // input-row slots (3 runs each, as in the ring)
