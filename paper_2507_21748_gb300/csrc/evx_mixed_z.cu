@@ -1,4 +1,5 @@
 // Two-radix z passes (see evx_mixed.cuh).
+#include "evx_cta_sum.cuh"
 #include "evx_mixed.cuh"
 
 namespace evx {
@@ -222,10 +223,7 @@ __global__ void __launch_bounds__(MAX > 16 ? 256 : 192, MAX > 16 ? 2 : MAX > 12 
                 red[tid] = acc + ps.take();
                 __syncthreads();
                 if (tid < 32) {
-                    double t = 0.0;
-                    for (int i = tid; i < nthr; i += 32) t += red[i];
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+                    const double t = first_warp_sum(red, nthr, tid);
                     if (tid == 0) a.partials[blockIdx.x] = t;
                 }
                 return;
@@ -279,10 +277,7 @@ __global__ void __launch_bounds__(MAX > 16 ? 256 : 192, MAX > 16 ? 2 : MAX > 12 
         red[tid] = (double)gs + (double)ge;
         __syncthreads();
         if (tid < 32) {
-            double t = 0.0;
-            for (int i = tid; i < nthr; i += 32) t += red[i];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+            const double t = first_warp_sum(red, nthr, tid);
             if (tid == 0) a.gsum[blockIdx.x] = t;
         }
     }

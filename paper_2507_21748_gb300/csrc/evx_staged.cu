@@ -20,6 +20,7 @@
 #include <algorithm>
 #include <cstdint>
 
+#include "evx_cta_sum.cuh"
 #include "evx_internal.h"
 
 namespace evx {
@@ -450,10 +451,7 @@ __global__ void __launch_bounds__(256, 2) stg_z_kernel(ZPassArgs a, Cut c, int R
                 red[tid] = acc + ps.take();
                 __syncthreads();
                 if (tid < 32) {
-                    double t = 0.0;
-                    for (int i = tid; i < nthr; i += 32) t += red[i];
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+                    const double t = first_warp_sum(red, nthr, tid);
                     if (tid == 0) a.partials[blockIdx.x] = t;
                 }
             }
@@ -482,10 +480,7 @@ __global__ void __launch_bounds__(256, 2) stg_z_kernel(ZPassArgs a, Cut c, int R
         red[tid] = (double)gs + (double)ge;
         __syncthreads();
         if (tid < 32) {
-            double t = 0.0;
-            for (int i = tid; i < nthr; i += 32) t += red[i];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+            const double t = first_warp_sum(red, nthr, tid);
             if (tid == 0) a.gsum[blockIdx.x] = t;
         }
     }
