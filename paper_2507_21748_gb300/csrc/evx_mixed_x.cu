@@ -1,14 +1,18 @@
 // Two-radix x pass with the k-space update (see evx_mixed.cuh).
+#include <cfloat>
+
 #include "evx_mixed.cuh"
 
 namespace evx {
 namespace mixed {
 
-// 1 / D for D >= 1: the hardware's approximation and one Newton step r + r (1 - D r)
+// 1 / D for D >= 1: the hardware's approximation and one Newton step r + r (1 - D r).
+// D = inf (|k|^4 beyond FP32) gives 0, as a division: its residual is taken at the largest
+// finite number, inf * 0 would make the mode NaN and with it the field.
 __device__ __forceinline__ float inverse(float D) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(D));
-    return fmaf(r, fmaf(-D, r, 1.f), r);
+    return fmaf(r, fmaf(-fminf(D, FLT_MAX), r, 1.f), r);
 }
 
 // middle of the x pass: forward pass B of W and S, the update, inverse pass B;
