@@ -292,6 +292,13 @@ __global__ void __launch_bounds__(256) reduce_partials_f32(const float* partials
             float v[16];
 #pragma unroll
             for (int u = 0; u < 16; ++u) v[u] = b + 8 * u < nparts ? partials[(long long)(b + 8 * u) * n + i] : 0.f;
+            bool huge = false;
+#pragma unroll
+            for (int u = 0; u < 16; ++u) huge |= fabsf(v[u]) > HUGE_VALUE;
+            if (huge) {  // infinities, and sums beyond FP32
+                for (float x : v) acc += (double)x;
+                continue;
+            }
             Sum2 t;
 #pragma unroll
             for (int u = 0; u < 16; ++u) t.add(v[u]);
