@@ -139,12 +139,15 @@ struct ColEnergy {
 #pragma unroll
         for (int k = 0; k < R; ++k) {
             const float kx = __ldg(k2x + R1 * k);
-            if (fabsf(v[k].x) > 0x1p50f || fabsf(v[k].y) > 0x1p50f) {
+            float2 k2 = two_sum(yh, kx);
+            k2.y += yl;
+            // pairs hold |c_hat|^2 and its product with |k|^2 while neither overflows and their low
+            // parts (2^-48) stay normal numbers; anything else, NaN too, is added in FP64
+            const float big = fmaxf(fabsf(v[k].x), fabsf(v[k].y)), e = big * big * k2.x;
+            if (big != 0.f && !(big >= 0x1p-39f && big <= 0x1p50f && e >= 0x1p-78f && e <= 0x1p100f)) {
                 acc += (edge ? 1.0 : 2.0) * ((double)kx + k2yz) * ((double)v[k].x * v[k].x + (double)v[k].y * v[k].y);
                 continue;
             }
-            float2 k2 = two_sum(yh, kx);
-            k2.y += yl;
             const float px = v[k].x * v[k].x, py = v[k].y * v[k].y;
             float2 m = two_sum(px, py);
             m.y += fmaf(v[k].x, v[k].x, -px) + fmaf(v[k].y, v[k].y, -py);
