@@ -60,6 +60,17 @@ __device__ __forceinline__ void load_cols(float2* tile, int c0, const float2* g,
     }
 }
 
+// adds to the elements that load_cols has read for the same thread
+__device__ __forceinline__ void add_cols(float2* tile, int c0, const float2* g, long long base, long long rs, int L,
+                                         int col0, int ncols, long long nbuf) {
+    for (int e = threadIdx.x; e < L * SP; e += NT) {
+        const int i = e / SP, p = e % SP;
+        const long long idx = base + i * rs + p;
+        float2* t = tile + i * (2 * SP) + c0 + p;
+        if (col0 + p < ncols && EVX_IN(idx, nbuf)) *t = cadd(*t, g[idx]);
+    }
+}
+
 __device__ __forceinline__ void store_cols(float2* g, const float2* tile, int c0, long long base,
                                            long long rs, int L, int col0, int ncols, long long nbuf) {
     for (int e = threadIdx.x; e < L * SP; e += NT) {
@@ -88,6 +99,7 @@ __global__ void __launch_bounds__(NT, 1) xadj_kernel(XAdjArgs a) {
     const long long base = split_off(ky, a.YB, a.os, a.os2) + col0;
     const long long nbuf = (long long)(a.ny / a.YB) * a.os2;  // complex elements of each field
     load_cols(tile, 0, a.Lam, base, a.rs, L, col0, a.ncols, nbuf);
+    if (a.Lam2) add_cols(tile, 0, a.Lam2, base, a.rs, L, col0, a.ncols, nbuf);
     load_cols(tile, SP, a.Sn1, base, a.rs, L, col0, a.ncols, nbuf);
     __syncthreads();
     fft_cols2<-1>(tile, L, a.plan, tws);
@@ -351,10 +363,10 @@ extern "C" evx_status evx_ch_adjoint(evx_grid* g, const float* d_c0, int n_steps
             if (r != EVX_OK) return r;
         }
         for (int j = n - 1; j >= 0; --j) {
-            // the fast x pass reads Lambda as the two parts the step before left, P and W
+            // the x pass reads Lambda as the two parts the step before left, P and W
             // (nothing else of a segment's adjoint steps uses them), so the sum is formed
             // once per segment instead of in a pass of its own per step
-            const bool parts = fast_xadj_length(g->nx) && j != n - 1;
+            const bool parts = j != n - 1;
             XAdjArgs x = xa;
             x.Lam = parts ? A->P : A->Lam;
             x.Lam2 = parts ? g->W : nullptr;
@@ -377,11 +389,11 @@ extern "C" evx_status evx_ch_adjoint(evx_grid* g, const float* d_c0, int n_steps
             z.cnpitch = g->nz;
             CKA(launch_zpass(z, Z_ADJ, sst));
             CKA(launch_spass(y_args(g, g->W, g->W), -1, sst));
-            if (j == 0 || !fast_xadj_length(g->nx)) CKA(launch_cadd(A->P, g->W, A->Lam, nspec, sst));
+            if (j == 0) CKA(launch_cadd(A->P, g->W, A->Lam, nspec, sst));
         }
         return EVX_OK;
     };
-    // full segments replay one captured graph (about 11 launches per step) whose
+    // full segments replay one captured graph (9 launches per step and one sum) whose
     // input is the seg0 buffer; a shorter last segment runs eagerly
     cudaGraphExec_t gexec = nullptr;
     if (n_steps >= K && nseg > (n_steps % K ? 1 : 0)) {

@@ -1059,9 +1059,6 @@ static cudaError_t run_fxadj(const XAdjArgs& a, cudaStream_t st) {
     return launch_chained(fast::fxadj_kernel<R1, TP>, dim3(a.nchunks, a.ny), 8 * TP, smem, st, a);
 }
 
-bool fast_xadj_length(int L) {
-    return fast_paths_enabled() && (L == 64 || L == 128 || L == 256 || L == 512 || L == 1024 || L == 400);
-}
 bool fast_xadj(const XAdjArgs& a, cudaStream_t st, cudaError_t* err) {
     if (!fast_paths_enabled() || a.os * a.YB != a.rs) return false;
     switch (a.L) {

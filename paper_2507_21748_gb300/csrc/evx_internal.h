@@ -260,7 +260,6 @@ bool fast_xupdate(const XUpdArgs& a, cudaStream_t st, cudaError_t* err);
 bool fast_zstep(const ZPassArgs& a, cudaStream_t st, cudaError_t* err, int* grid_used, bool adj = false);
 // adjoint x pass with the four-step transforms; false if the length has no fast kernel
 bool fast_xadj(const XAdjArgs& a, cudaStream_t st, cudaError_t* err);
-bool fast_xadj_length(int L);
 bool fast_zconv(const ZPassArgs& a, int dir, cudaStream_t st, cudaError_t* err, int* grid_used);
 bool fast_paths_enabled();  // false when the environment sets EVX_GENERIC=1
 // grids whose mixed-radix passes run with grouped stages (evx_staged.cu), bit for bit
