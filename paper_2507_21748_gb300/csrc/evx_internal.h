@@ -26,6 +26,32 @@ __device__ __forceinline__ bool evx_in_bounds(long long i, long long n, int line
 #endif
 int bounds_line_kernels(bool clear);   // evx_kernels.cu (0 in the normal build)
 int bounds_line_adjoint(bool clear);   // evx_adjoint.cu
+int bounds_line_mixed_x(bool clear);   // evx_mixed_x.cu
+int bounds_line_mixed_y(bool clear);   // evx_mixed_y.cu
+int bounds_line_mixed_z(bool clear);   // evx_mixed_z.cu
+int bounds_line_staged(bool clear);    // evx_staged.cu
+// a translation unit's function of these: its line, -1 if it cannot be read
+inline int bounds_take(const int& line, bool clear) {
+    int h = 0;
+    if (cudaMemcpyFromSymbol(&h, line, sizeof(int)) != cudaSuccess) return -1;
+    if (clear && h) {
+        const int z = 0;
+        cudaMemcpyToSymbol(line, &z, sizeof(int));
+    }
+    return h;
+}
+#ifdef EVX_BOUNDS_CHECK
+#define EVX_BOUNDS_TAKE(clear) ::evx::bounds_take(g_bounds_line, clear)
+#else
+#define EVX_BOUNDS_TAKE(clear) ((void)(clear), 0)
+#endif
+// a buffer of n elements, for kernels that walk it by pointer: EVX_AT(p, b) is EVX_IN of p's index
+template <typename T>
+struct Extent {
+    const T* org;
+    long long n;
+};
+#define EVX_AT(p, b) EVX_IN((p) - (b).org, (b).n)
 
 // Programmatic dependent launch. A solver step is a chain of short kernels, each
 // reading what the one before wrote. launch_chained lets a kernel be set up while

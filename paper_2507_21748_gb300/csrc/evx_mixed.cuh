@@ -70,11 +70,12 @@ struct ColLoad {
     int pitch;  // R2p * 8
     const float2* tw;
     int n2;
+    Extent<float2> ext;
     template <int R>
     __device__ __forceinline__ void run() const {
         float2 v[R];
 #pragma unroll
-        for (int i = 0; i < R; ++i) v[i] = src[i * stride];
+        for (int i = 0; i < R; ++i) v[i] = EVX_AT(src + i * stride, ext) ? src[i * stride] : make_float2(0.f, 0.f);
         Dft<R, DIR>::run(v);
         x[0] = v[0];
 #pragma unroll
@@ -87,6 +88,7 @@ struct ColStore {
     float2* dst;
     long long stride;
     const float2* x;  // exchange, at column p and row k1
+    Extent<float2> ext;
     template <int R>
     __device__ __forceinline__ void run() const {
         float2 v[R];
@@ -94,7 +96,8 @@ struct ColStore {
         for (int i = 0; i < R; ++i) v[i] = x[i * CP];
         Dft<R, DIR>::run(v);
 #pragma unroll
-        for (int k = 0; k < R; ++k) dst[k * stride] = v[k];
+        for (int k = 0; k < R; ++k)
+            if (EVX_AT(dst + k * stride, ext)) dst[k * stride] = v[k];
     }
 };
 // last pass of an inverse, to global: v[k1] from column n2, DFT-R1, dst[n1 stride]
@@ -103,6 +106,7 @@ struct ColStoreInv {
     long long stride;
     const float2* x;  // exchange, at column p and n2
     int pitch;
+    Extent<float2> ext;
     template <int R>
     __device__ __forceinline__ void run() const {
         float2 v[R];
@@ -110,7 +114,8 @@ struct ColStoreInv {
         for (int k = 0; k < R; ++k) v[k] = x[k * pitch];
         Dft<R, 1>::run(v);
 #pragma unroll
-        for (int i = 0; i < R; ++i) dst[i * stride] = v[i];
+        for (int i = 0; i < R; ++i)
+            if (EVX_AT(dst + i * stride, ext)) dst[i * stride] = v[i];
     }
 };
 

@@ -99,12 +99,14 @@ __global__ void __launch_bounds__(8 * M1, M1 <= 16 ? 5 : M1 <= 20 ? 4 : 2) mx_x_
     const int ky = blockIdx.y, kz = (int)blockIdx.x * CP + p;
     const bool valid = kz < a.ncols;
     const long long base = split_off(ky, a.YB, a.os, a.os2) + kz;
+    const long long nbuf = (long long)(a.ny / a.YB) * a.os2;  // complex elements of W, S and S_out
     if (valid)
         for (int i = it; i < (MODE == 2 ? R2 : 2 * R2); i += T) {
             const bool second = i >= R2;
             const int n2 = second ? i - R2 : i;
             with_radix<M1>(R1, ColLoad<-1>{(second ? a.S : a.W) + base + n2 * a.rs, R2 * a.rs,
-                                             (second ? xs : xw) + n2 * CP + p, pitch, a.tw, n2});
+                                             (second ? xs : xw) + n2 * CP + p, pitch, a.tw, n2,
+                                             {second ? a.S : a.W, nbuf}});
         }
     __syncthreads();
     if (valid) {
@@ -117,7 +119,7 @@ __global__ void __launch_bounds__(8 * M1, M1 <= 16 ? 5 : M1 <= 20 ? 4 : 2) mx_x_
     __syncthreads();
     if (valid)
         for (int n2 = it; n2 < R2; n2 += T)
-            with_radix<M1>(R1, ColStoreInv{a.S_out + base + n2 * a.rs, R2 * a.rs, xs + n2 * CP + p, pitch});
+            with_radix<M1>(R1, ColStoreInv{a.S_out + base + n2 * a.rs, R2 * a.rs, xs + n2 * CP + p, pitch, {a.S_out, nbuf}});
 }
 
 // gradient energy: forward passes A and B of S, sum of w(kz) |k|^2 |c_hat|^2 on FP32 pairs
@@ -167,9 +169,10 @@ __global__ void __launch_bounds__(8 * MAX, MAX <= 16 ? 5 : 2) mx_energy_kernel(X
     const int ky = blockIdx.y, kz = (int)blockIdx.x * CP + p;
     const bool valid = kz < a.ncols;
     const long long base = split_off(ky, a.YB, a.os, a.os2) + kz;
+    const long long nbuf = (long long)(a.ny / a.YB) * a.os2;
     if (valid)
         for (int n2 = it; n2 < R2; n2 += T)
-            with_radix<MAX>(R1, ColLoad<-1>{a.S + base + n2 * a.rs, R2 * a.rs, xs + n2 * CP + p, pitch, a.tw, n2});
+            with_radix<MAX>(R1, ColLoad<-1>{a.S + base + n2 * a.rs, R2 * a.rs, xs + n2 * CP + p, pitch, a.tw, n2, {a.S, nbuf}});
     __syncthreads();
     double acc = 0.0;
     if (valid) {
@@ -195,6 +198,8 @@ __global__ void __launch_bounds__(8 * MAX, MAX <= 16 ? 5 : 2) mx_energy_kernel(X
 }
 
 }  // namespace mixed
+
+int bounds_line_mixed_x(bool clear) { return EVX_BOUNDS_TAKE(clear); }
 
 template <int MODE>
 static auto mx_x_pick(int R1, int R2) {

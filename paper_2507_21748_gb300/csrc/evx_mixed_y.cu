@@ -13,16 +13,19 @@ __global__ void __launch_bounds__(8 * MAX, MAX <= 16 ? 8 : MAX <= 20 ? 5 : 2) mx
     const int R2p = R2 | 1;
     const bool valid = (int)blockIdx.x * CP + p < a.ncols;
     const long long base = (long long)blockIdx.y * a.os + (long long)blockIdx.x * CP + p;
+    const long long nbuf = (long long)(a.L / a.YB) * a.os2;  // complex elements of in / out
     if (valid)
         for (int n2 = it; n2 < R2; n2 += T)
-            with_radix<MAX>(R1, ColLoad<DIR>{a.in + base + n2 * a.rs, R2 * a.rs, xb + n2 * CP + p, R2p * CP, a.tw, n2});
+            with_radix<MAX>(R1, ColLoad<DIR>{a.in + base + n2 * a.rs, R2 * a.rs, xb + n2 * CP + p, R2p * CP, a.tw, n2, {a.in, nbuf}});
     __syncthreads();
     if (valid)
         for (int k1 = it; k1 < R1; k1 += T)
-            with_radix<MAX>(R2, ColStore<DIR>{a.out + base + k1 * a.rs, R1 * a.rs, xb + k1 * R2p * CP + p});
+            with_radix<MAX>(R2, ColStore<DIR>{a.out + base + k1 * a.rs, R1 * a.rs, xb + k1 * R2p * CP + p, {a.out, nbuf}});
 }
 
 }  // namespace mixed
+
+int bounds_line_mixed_y(bool clear) { return EVX_BOUNDS_TAKE(clear); }
 
 // The radices of a length: the smallest R1 >= R2 whose product is L (0 if none).
 bool mixed_split(int L, int* R1, int* R2) {

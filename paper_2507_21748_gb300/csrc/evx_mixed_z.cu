@@ -80,10 +80,12 @@ struct ZMiddle {
             const int m = k1 + z.R1 * k;
             const float d0 = v[k].x * s, d1 = v[k].y * s;
             if (ADJ) {
-                const float2 c = rowok ? reinterpret_cast<const float2*>(a.cn + row * a.cnpitch)[m] : make_float2(0.f, 0.f);
+                const float2 c = rowok && EVX_IN(row * a.cnpitch + 2 * m + 1, a.nrows * a.cnpitch)
+                                     ? reinterpret_cast<const float2*>(a.cn + row * a.cnpitch)[m]
+                                     : make_float2(0.f, 0.f);
                 v[k] = make_float2(d0 * fmaf(3.f * c.x, c.x, -1.f), d1 * fmaf(3.f * c.y, c.y, -1.f));
             } else {
-                if (a.rout && rowok)
+                if (a.rout && rowok && EVX_IN(row * a.rpitch + 2 * m + 1, a.nrows * a.rpitch))
                     reinterpret_cast<float2*>(a.rout + row * a.rpitch)[m] =
                         make_float2(fmaf(v[k].x, s, cbl) + cb, fmaf(v[k].y, s, cbl) + cb);
                 // g(c) - g(cbar) about the mean, as in the fast z pass
@@ -192,11 +194,13 @@ __global__ void __launch_bounds__(MAX > 16 ? 256 : 192, MAX > 16 ? 2 : MAX > 12 
         if (rowok) {
             const long long ur = a.map_rows ? user_row(row, a.YB, a.nxr, a.nyr) : row;
             const float2* src = reinterpret_cast<const float2*>(a.rin + ur * a.rpitch);
-            for (int q = tx; q < M; q += T) cp8(z.row + q, src + q);
+            for (int q = tx; q < M; q += T)
+                if (EVX_IN(ur * a.rpitch + 2 * q + 1, a.nrows * a.rpitch)) cp8(z.row + q, src + q);
         }
     } else if (rowok) {
         const float2* src = a.in + row * a.Zp;
-        for (int q = tx; q < a.Zp / 2; q += T) cp16(z.row + 2 * q, src + 2 * q);
+        for (int q = tx; q < a.Zp / 2; q += T)
+            if (EVX_IN(row * a.Zp + 2 * q + 1, a.nrows * a.Zp)) cp16(z.row + 2 * q, src + 2 * q);
     }
     cp_wait_all();
     __syncthreads();
@@ -231,18 +235,20 @@ __global__ void __launch_bounds__(MAX > 16 ? 256 : 192, MAX > 16 ? 2 : MAX > 12 
             if (rowok) {
                 const long long ur = a.map_rows ? user_row(row, a.YB, a.nxr, a.nyr) : row;
                 float2* dst = reinterpret_cast<float2*>(a.rout + ur * a.rpitch);
+                auto ok = [&](int q) { return EVX_IN(ur * a.rpitch + 2 * q + 1, a.nrows * a.rpitch); };
                 if (a.accumulate) {  // eight reads in flight
                     for (int q = tx; q < M; q += 8 * T) {
                         float2 prev[8];
 #pragma unroll
                         for (int u = 0; u < 8; ++u)
-                            if (q + u * T < M) prev[u] = dst[q + u * T];
+                            if (q + u * T < M) prev[u] = ok(q + u * T) ? dst[q + u * T] : make_float2(0.f, 0.f);
 #pragma unroll
                         for (int u = 0; u < 8; ++u)
-                            if (q + u * T < M) dst[q + u * T] = cadd(prev[u], z.row[q + u * T]);
+                            if (q + u * T < M && ok(q + u * T)) dst[q + u * T] = cadd(prev[u], z.row[q + u * T]);
                     }
                 } else {
-                    for (int q = tx; q < M; q += T) dst[q] = z.row[q];
+                    for (int q = tx; q < M; q += T)
+                        if (ok(q)) dst[q] = z.row[q];
                 }
             }
             return;
@@ -256,11 +262,14 @@ __global__ void __launch_bounds__(MAX > 16 ? 256 : 192, MAX > 16 ? 2 : MAX > 12 
     // R2C post-processing, pairs (k, M - k)
     if (rowok) {
         float2* out = a.out + row * a.Zp;
+        auto put = [&](int k, float2 v) {
+            if (EVX_IN(row * a.Zp + k, a.nrows * a.Zp)) out[k] = v;
+        };
         for (int k = tx; k <= M / 2; k += T) {
             if (k == 0) {
                 const float2 z0 = z.row[0];
-                out[0] = make_float2(z0.x + z0.y, 0.f);
-                out[M] = make_float2(z0.x - z0.y, 0.f);
+                put(0, make_float2(z0.x + z0.y, 0.f));
+                put(M, make_float2(z0.x - z0.y, 0.f));
                 continue;
             }
             // X_k = (P - i w Q) / 2, P = Z_k + conj Z_{M-k}, Q = Z_k - conj Z_{M-k}; X_{M-k} = conj(P + i w Q) / 2
@@ -268,8 +277,8 @@ __global__ void __launch_bounds__(MAX > 16 ? 256 : 192, MAX > 16 ? 2 : MAX > 12 
             const float px = 0.5f * (zk.x + zm.x), py = 0.5f * (zk.y - zm.y);
             const float qx = 0.5f * (zk.x - zm.x), qy = 0.5f * (zk.y + zm.y);
             const float ux = fmaf(w.x, qy, w.y * qx), uy = fmaf(-w.x, qx, w.y * qy);  // -i w Q
-            out[k] = make_float2(px + ux, py + uy);
-            if (M - k != k) out[M - k] = make_float2(px - ux, uy - py);
+            put(k, make_float2(px + ux, py + uy));
+            if (M - k != k) put(M - k, make_float2(px - ux, uy - py));
         }
     }
     if (MODE == Z_STEP && a.gsum) {  // FP64 partial of the CTA, fixed order
@@ -284,6 +293,8 @@ __global__ void __launch_bounds__(MAX > 16 ? 256 : 192, MAX > 16 ? 2 : MAX > 12 
 }
 
 }  // namespace mixed
+
+int bounds_line_mixed_z(bool clear) { return EVX_BOUNDS_TAKE(clear); }
 
 // rows per CTA: up to 192 threads (256 with radices above 16) and 48 KB, fewer while the grid would leave SMs idle
 static int mixed_zrows(const ZPassArgs& a, int R1, int RS) {

@@ -869,8 +869,12 @@ evx_status evx_debug_bounds(int* enabled, int* line) {
     if (line) {
         cudaError_t e = cudaDeviceSynchronize();
         if (e != cudaSuccess) return fail(nullptr, EVX_ERR_CUDA, "synchronise: %s", cudaGetErrorString(e));
-        const int a = bounds_line_kernels(true), b = bounds_line_adjoint(true);
-        *line = a ? a : b;
+        *line = 0;
+        for (auto take : {bounds_line_kernels, bounds_line_adjoint, bounds_line_mixed_x, bounds_line_mixed_y,
+                          bounds_line_mixed_z, bounds_line_staged}) {
+            const int at = take(true);
+            if (!*line) *line = at;
+        }
     }
     return EVX_OK;
 }

@@ -98,11 +98,12 @@ struct LeadFromGlobal {
     float2* x;          // exchange at (0, n2)
     Cut c;
     const float2* tw;
+    Extent<float2> ext;
     template <int R>
     __device__ __forceinline__ void run() const {
         float2 v[R];
 #pragma unroll
-        for (int t = 0; t < R; ++t) v[t] = src[t * stride];
+        for (int t = 0; t < R; ++t) v[t] = EVX_AT(src + t * stride, ext) ? src[t * stride] : make_float2(0.f, 0.f);
         group<R, DIR>(v, 1, 0, c.L, tw);
 #pragma unroll
         for (int u = 0; u < R; ++u) x[u * c.R2p * CP] = v[u];
@@ -117,6 +118,7 @@ struct TrailToGlobal {
     Cut c;
     const float2* tw;
     int k1;
+    Extent<float2> ext;
     template <int R>
     __device__ __forceinline__ void run() const {
         float2 v[R];
@@ -124,7 +126,8 @@ struct TrailToGlobal {
         for (int t = 0; t < R; ++t) v[t] = x[t * CP];
         group<R, DIR>(v, c.R1, k1, c.L, tw);
 #pragma unroll
-        for (int u = 0; u < R; ++u) dst[u * stride] = v[u];
+        for (int u = 0; u < R; ++u)
+            if (EVX_AT(dst + u * stride, ext)) dst[u * stride] = v[u];
     }
 };
 
@@ -136,11 +139,13 @@ __global__ void __launch_bounds__(256, 3) stg_y_kernel(SPassArgs a, Cut c) {
     const int p = threadIdx.x & 7, it = threadIdx.x >> 3;
     const bool valid = (int)blockIdx.x * CP + p < a.ncols;
     const long long base = (long long)blockIdx.y * a.os + (long long)blockIdx.x * CP + p;
+    const long long nbuf = (long long)(c.L / a.YB) * a.os2;  // complex elements of in / out
     if (valid && it < c.R2)
-        with_group(c.R1, LeadFromGlobal<DIR>{a.in + base + it * a.rs, c.R2 * a.rs, xb + it * CP + p, c, a.tw});
+        with_group(c.R1, LeadFromGlobal<DIR>{a.in + base + it * a.rs, c.R2 * a.rs, xb + it * CP + p, c, a.tw, {a.in, nbuf}});
     __syncthreads();
     if (valid && it < c.R1)
-        with_group(c.R2, TrailToGlobal<DIR>{xb + it * c.R2p * CP + p, a.out + base + it * a.rs, c.R1 * a.rs, c, a.tw, it});
+        with_group(c.R2, TrailToGlobal<DIR>{xb + it * c.R2p * CP + p, a.out + base + it * a.rs, c.R1 * a.rs, c, a.tw, it,
+                                            {a.out, nbuf}});
 }
 
 // trailing groups of W and S, the update (the operations of xupdate_kernel), the
@@ -243,10 +248,11 @@ __global__ void __launch_bounds__(256, 2) stg_x_kernel(XUpdArgs a, Cut c) {
     float2* xw = reinterpret_cast<float2*>(smem4);
     float2* xs = xw + c.R1 * c.R2p * CP;
     const long long base = split_off(ky, a.YB, a.os, a.os2) + kz;
+    const long long nbuf = (long long)(a.ny / a.YB) * a.os2;  // complex elements of W, S and S_out
     if (valid && it < c.R2) {
-        with_group(c.R1, LeadFromGlobal<-1>{a.W + base + it * a.rs, c.R2 * a.rs, xw + it * CP + p, c, a.tw});
+        with_group(c.R1, LeadFromGlobal<-1>{a.W + base + it * a.rs, c.R2 * a.rs, xw + it * CP + p, c, a.tw, {a.W, nbuf}});
         if (a.model != 2)
-            with_group(c.R1, LeadFromGlobal<-1>{a.S + base + it * a.rs, c.R2 * a.rs, xs + it * CP + p, c, a.tw});
+            with_group(c.R1, LeadFromGlobal<-1>{a.S + base + it * a.rs, c.R2 * a.rs, xs + it * CP + p, c, a.tw, {a.S, nbuf}});
     }
     __syncthreads();
     if (valid && it < c.R1) {
@@ -259,7 +265,8 @@ __global__ void __launch_bounds__(256, 2) stg_x_kernel(XUpdArgs a, Cut c) {
         with_group(c.R1, LeadFromRows<1, CP, false>{xs + p, xw + it * CP + p, c, a.tw, it, true});
     __syncthreads();
     if (valid && it < c.R1)
-        with_group(c.R2, TrailToGlobal<1>{xw + it * c.R2p * CP + p, a.S_out + base + it * a.rs, c.R1 * a.rs, c, a.tw, it});
+        with_group(c.R2, TrailToGlobal<1>{xw + it * c.R2p * CP + p, a.S_out + base + it * a.rs, c.R1 * a.rs, c, a.tw, it,
+                                          {a.S_out, nbuf}});
 }
 
 // ---------------------------------------------------------------- z passes
@@ -320,7 +327,9 @@ struct TrailPoint {
             const int n = k1 + c.R1 * u;
             const float2 z = v[u];
             if (MODE == Z_ADJ) {
-                const float2 cn = reinterpret_cast<const float2*>(a.cn + row * a.cnpitch)[n];
+                const float2 cn = EVX_IN(row * a.cnpitch + 2 * n + 1, a.nrows * a.cnpitch)
+                                      ? reinterpret_cast<const float2*>(a.cn + row * a.cnpitch)[n]
+                                      : make_float2(0.f, 0.f);
                 const float d0 = fmaf(3.f * cn.x, cn.x, -1.f), d1 = fmaf(3.f * cn.y, cn.y, -1.f);
                 x[u] = make_float2(z.x * s * d0, z.y * s * d1);
                 continue;
@@ -330,7 +339,8 @@ struct TrailPoint {
                 x[u] = make_float2(c0, c1);
                 continue;
             }
-            if (a.rout) reinterpret_cast<float2*>(a.rout + row * a.rpitch)[n] = make_float2(c0, c1);
+            if (a.rout && EVX_IN(row * a.rpitch + 2 * n + 1, a.nrows * a.rpitch))
+                reinterpret_cast<float2*>(a.rout + row * a.rpitch)[n] = make_float2(c0, c1);
             const float d0 = z.x * s, d1 = z.y * s;
             const float2 gv = make_float2(d0 * fmaf(d0, c3 + d0, gp), d1 * fmaf(d1, c3 + d1, gp));
             x[u] = gv;
@@ -411,10 +421,11 @@ __global__ void __launch_bounds__(256, 2) stg_z_kernel(ZPassArgs a, Cut c, int R
     if (rowok) {
         if (MODE == Z_R2C) {
             const float2* src = reinterpret_cast<const float2*>(a.rin + ur * a.rpitch);
-            for (int n = tx; n < M; n += T) z[n] = src[n];
+            for (int n = tx; n < M; n += T)
+                z[n] = EVX_IN(ur * a.rpitch + 2 * n + 1, a.nrows * a.rpitch) ? src[n] : make_float2(0.f, 0.f);
         } else {
             const float2* src = a.in + row * a.Zp;
-            for (int n = tx; n <= M; n += T) z[n] = src[n];
+            for (int n = tx; n <= M; n += T) z[n] = EVX_IN(row * a.Zp + n, a.nrows * a.Zp) ? src[n] : make_float2(0.f, 0.f);
         }
     }
     __syncthreads();
@@ -439,6 +450,7 @@ __global__ void __launch_bounds__(256, 2) stg_z_kernel(ZPassArgs a, Cut c, int R
                     if (a.partials) {  // energy: nothing is written
                         add_well(ps, acc, v.x);
                         add_well(ps, acc, v.y);
+                    } else if (!EVX_IN(ur * a.rpitch + 2 * n + 1, a.nrows * a.rpitch)) {
                     } else if (a.accumulate) {
                         const float2 prev = o[n];
                         o[n] = make_float2(prev.x + v.x, prev.y + v.y);
@@ -465,6 +477,7 @@ __global__ void __launch_bounds__(256, 2) stg_z_kernel(ZPassArgs a, Cut c, int R
     if (rowok) {  // R2C post-processing
         float2* out = a.out + row * a.Zp;
         for (int k = tx; k <= M; k += T) {
+            if (!EVX_IN(row * a.Zp + k, a.nrows * a.Zp)) continue;
             if (k == 0 || k == M) {
                 const float2 z0 = z[0];
                 out[k] = make_float2(k == 0 ? z0.x + z0.y : z0.x - z0.y, 0.f);
@@ -489,6 +502,8 @@ __global__ void __launch_bounds__(256, 2) stg_z_kernel(ZPassArgs a, Cut c, int R
 }  // namespace staged
 
 // ----------------------------------------------------------------- dispatch
+int bounds_line_staged(bool clear) { return EVX_BOUNDS_TAKE(clear); }
+
 // The cut of a plan with both groups compiled in and the fewest threads per
 // pencil; lengths up to 128 (longer ones have none or run better on two radices).
 static bool staged_cut(const Plan& pl, int L, staged::Cut* c) {
