@@ -878,7 +878,8 @@ __global__ void __launch_bounds__(pj::NT, 1)
     const float b0 = r.bias ? r.bias[0] : 0.f;
     __syncthreads();
     uint32_t k = 0;  // planes consumed
-    for (int u = blockIdx.x; u < r.nunits; u += gridDim.x) {
+    bool failed = false;  // the same in every thread
+    for (int u = blockIdx.x; u < r.nunits && !failed; u += gridDim.x) {
         const int seg = u % r.nseg;
         int c = u / r.nseg;
         const int z0 = (c % (Z / ZT)) * ZT;
@@ -908,7 +909,7 @@ __global__ void __launch_bounds__(pj::NT, 1)
 #pragma unroll
             for (int j = 0; j < 32; ++j) acc[d][0][j] = acc[d][1][j] = 0.f;
         for (int q = 0; q < np; ++q, ++k) {
-            ring_wait(full + 8 * (k & 1), (k >> 1) & 1, abort_flag);  // on failure: stale data, flag set
+            const bool arrived = ring_wait(full + 8 * (k & 1), (k >> 1) & 1, abort_flag);
             const float* pl = reinterpret_cast<const float*>(smem_raw + (k & 1) * PLANE) + (2 * warp) * PROW + lane;
 #pragma unroll
             for (int yy = 0; yy < 4; ++yy) {
@@ -929,7 +930,13 @@ __global__ void __launch_bounds__(pj::NT, 1)
                         }
                 }
             }
-            __syncthreads();  // the plane has been read
+            // the plane has been read; a wait that ran out in any thread ends the CTA: nothing is
+            // stored or loaded after it, and the copies in flight land first (bounded)
+            if ((failed = __syncthreads_or(!arrived))) {
+                if (threadIdx.x == 0)
+                    for (int m = 0; m < 2 && q + m < np; ++m) tc_wait(full + 8 * ((k + m) & 1), ((k + m) >> 1) & 1);
+                break;
+            }
             if (q + 2 < np) load(q + 2, k + 2);
             if (q >= 2) {
                 const int x = xs + q - 2, y = y0 + 2 * warp;
