@@ -50,6 +50,14 @@ __device__ __forceinline__ void with_radix(int r, Fn&& f) {
     }
 }
 
+// The register DFTs of these passes. 10 and 20 from coprime factors, without twiddles: the
+// rounded twiddles of the forms the four-step kernels use scale a transform and its inverse
+// by a fixed amount, and the state goes through both along x in every step (a length of 300:
+// 1 + 4.0e-8 against 1 + 2.4e-8 this way; the radices 5 5 4 3 one by one 1 + 2.2e-8).
+template <int R, int DIR> struct MxDft : Dft<R, DIR> {};
+template <int DIR> struct MxDft<10, DIR> : DftCoprime<2, 5, DIR> {};
+template <int DIR> struct MxDft<20, DIR> : DftCoprime<4, 5, DIR> {};
+
 template <int DIR>
 __device__ __forceinline__ float2 twmul(float2 v, float2 w) {
     if (DIR > 0) w.y = -w.y;
@@ -76,7 +84,7 @@ struct ColLoad {
         float2 v[R];
 #pragma unroll
         for (int i = 0; i < R; ++i) v[i] = EVX_AT(src + i * stride, ext) ? src[i * stride] : make_float2(0.f, 0.f);
-        Dft<R, DIR>::run(v);
+        MxDft<R, DIR>::run(v);
         x[0] = v[0];
 #pragma unroll
         for (int k = 1; k < R; ++k) x[k * pitch] = twmul<DIR>(v[k], __ldg(tw + n2 * k));
@@ -94,7 +102,7 @@ struct ColStore {
         float2 v[R];
 #pragma unroll
         for (int i = 0; i < R; ++i) v[i] = x[i * CP];
-        Dft<R, DIR>::run(v);
+        MxDft<R, DIR>::run(v);
 #pragma unroll
         for (int k = 0; k < R; ++k)
             if (EVX_AT(dst + k * stride, ext)) dst[k * stride] = v[k];
@@ -112,7 +120,7 @@ struct ColStoreInv {
         float2 v[R];
 #pragma unroll
         for (int k = 0; k < R; ++k) v[k] = x[k * pitch];
-        Dft<R, 1>::run(v);
+        MxDft<R, 1>::run(v);
 #pragma unroll
         for (int i = 0; i < R; ++i)
             if (EVX_AT(dst + i * stride, ext)) dst[i * stride] = v[i];

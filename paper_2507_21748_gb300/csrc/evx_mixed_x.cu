@@ -6,13 +6,16 @@
 namespace evx {
 namespace mixed {
 
-// 1 / D for D >= 1: the hardware's approximation and one Newton step r + r (1 - D r).
-// D = inf (|k|^4 beyond FP32) gives 0, as a division: its residual is taken at the largest
+// a / D for D >= 1: the hardware's reciprocal and one Newton step on the quotient,
+// q + r (a - D q), which rounds a result that is exact to about 2^-44 (a step on the
+// reciprocal and a product by a round twice, the same way for a mode in every step).
+// D = inf (|k|^4 beyond FP32) gives 0, as a division: the residual is taken at the largest
 // finite number, inf * 0 would make the mode NaN and with it the field.
-__device__ __forceinline__ float inverse(float D) {
+__device__ __forceinline__ float quotient(float a, float D) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(D));
-    return fmaf(r, fmaf(-fminf(D, FLT_MAX), r, 1.f), r);
+    const float q = a * r;
+    return fmaf(r, fmaf(-fminf(D, FLT_MAX), q, a), q);
 }
 
 // middle of the x pass: forward pass B of W and S, the update, inverse pass B;
@@ -46,13 +49,13 @@ struct ColUpdate {
         float2 g[R];
 #pragma unroll
         for (int i = 0; i < R; ++i) g[i] = w[i * CP];
-        Dft<R, -1>::run(g);
+        MxDft<R, -1>::run(g);
         float2 v[R];
         if (MODE == 2) {  // preconditioner: dt / (1 + dt M kappa |k|^4) F_x W / L (dtM holds dt)
 #pragma unroll
             for (int k = 0; k < R; ++k) {
                 const float k2 = __ldg(k2x + R1 * k) + k2yz;
-                v[k] = cscale(g[k], a.dtM * (a.invL * inverse(fmaf(a.dtMk, k2 * k2, 1.f))));
+                v[k] = cscale(g[k], a.dtM * quotient(a.invL, fmaf(a.dtMk, k2 * k2, 1.f)));
             }
         } else {
             if (SPILL) {
@@ -61,26 +64,26 @@ struct ColUpdate {
             }
 #pragma unroll
             for (int i = 0; i < R; ++i) v[i] = s[i * CP];
-            Dft<R, -1>::run(v);
+            MxDft<R, -1>::run(v);
 #pragma unroll
             for (int k = 0; k < R; ++k) {
                 const float2 gk = SPILL ? w[k * CP] : g[k];
                 const float k2 = __ldg(k2x + R1 * k) + k2yz;
                 if (MODE == 3) {
-                    const float Dinv = inverse(fmaf(a.dtMk, k2 * k2, 1.f));
+                    const float Dinv = quotient(1.f, fmaf(a.dtMk, k2 * k2, 1.f));
                     float P, S;
                     blk(k2, Dinv, P, S);
                     const float bs = -a.dtM * k2 * Dinv * S * a.invL, as = P * a.invL;
                     v[k] = make_float2(fmaf(bs, gk.x, as * v[k].x), fmaf(bs, gk.y, as * v[k].y));
                 } else {  // (c_hat - dt M |k|^2 g_hat) / (1 + dt M kappa |k|^4); Allen-Cahn: 1 and |k|^2
-                    const float f = a.invL * inverse(fmaf(a.dtMk, ac ? k2 : k2 * k2, 1.f));
+                    const float f = quotient(a.invL, fmaf(a.dtMk, ac ? k2 : k2 * k2, 1.f));
                     const float b = -a.dtM * (ac ? 1.f : k2);
                     v[k] = make_float2(f * fmaf(b, gk.x, v[k].x), f * fmaf(b, gk.y, v[k].y));
                 }
             }
         }
         if (zero) v[0] = make_float2(0.f, 0.f);  // the mean is carried in FP64
-        Dft<R, 1>::run(v);
+        MxDft<R, 1>::run(v);
         s[0] = v[0];
 #pragma unroll
         for (int i = 1; i < R; ++i) s[i * CP] = twmul<1>(v[i], __ldg(a.tw + i * k1));
@@ -135,7 +138,7 @@ struct ColEnergy {
         float2 v[R];
 #pragma unroll
         for (int i = 0; i < R; ++i) v[i] = s[i * CP];
-        Dft<R, -1>::run(v);
+        MxDft<R, -1>::run(v);
         PairSum ps;
         const float yh = (float)k2yz, yl = (float)(k2yz - (double)yh);
 #pragma unroll

@@ -49,7 +49,7 @@ struct ZInvA {
         }
         __syncthreads();  // rows read: their slots become the exchange
         if (act) {
-            Dft<R, 1>::run(v);
+            MxDft<R, 1>::run(v);
             z.row[n2] = v[0];
 #pragma unroll
             for (int k = 1; k < R; ++k) z.row[k * z.R2p + n2] = twmul<1>(v[k], __ldg(z.tA + k * z.R2 + n2));
@@ -73,7 +73,7 @@ struct ZMiddle {
         float2 v[R];
 #pragma unroll
         for (int i = 0; i < R; ++i) v[i] = x[i];
-        Dft<R, 1>::run(v);
+        MxDft<R, 1>::run(v);
         const float s = a.scale;
 #pragma unroll
         for (int k = 0; k < R; ++k) {
@@ -100,7 +100,7 @@ struct ZMiddle {
                 }
             }
         }
-        Dft<R, -1>::run(v);
+        MxDft<R, -1>::run(v);
         x[0] = v[0];
 #pragma unroll
         for (int i = 1; i < R; ++i) x[i] = twmul<-1>(v[i], __ldg(z.tB + i * z.R1 + k1));
@@ -119,7 +119,7 @@ struct ZInvB {
             const float2* x = z.row + k1 * z.R2p;
 #pragma unroll
             for (int i = 0; i < R; ++i) v[i] = x[i];
-            Dft<R, 1>::run(v);
+            MxDft<R, 1>::run(v);
         }
         __syncthreads();
         if (act) {
@@ -147,7 +147,7 @@ struct ZFwdB {
         }
         __syncthreads();
         if (act) {
-            Dft<R, -1>::run(v);
+            MxDft<R, -1>::run(v);
             float2* x = z.row + k1 * z.R2p;
             x[0] = v[0];
 #pragma unroll
@@ -169,7 +169,7 @@ struct ZFwdA {
         }
         __syncthreads();
         if (act) {
-            Dft<R, -1>::run(v);
+            MxDft<R, -1>::run(v);
 #pragma unroll
             for (int i = 0; i < R; ++i) z.row[n2 + z.R2 * i] = v[i];
         }

@@ -1,0 +1,54 @@
+"""Twenty steps with the two-radix x pass are no further from the FP64 oracle than with the
+stage-by-stage kernel (EVX_GENERIC=1). A mode goes through the x transform, its inverse and
+the division in every step, so a fixed gain error adds up. Summed over lengths with the
+factors 10 and 20, two seeds each; 5% for the scatter of rounding errors between kernels
+(480,000 voxels a field: under 1% of a norm, and the y and z passes' share in it)."""
+import os
+import subprocess
+import sys
+
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2507_21748_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+SCRIPT = r'''
+import sys
+sys.path.insert(0, %r)
+import numpy as np, torch
+from paper_2507_21748_gb300 import evx
+d = dict(np.load(sys.argv[1]))
+for key, c0 in d.items():
+    with evx.Grid(c0.shape) as g:
+        g.set_field(torch.from_numpy(c0).cuda())
+        g.step(20)
+        d[key] = g.get_field().cpu().numpy()
+np.savez(sys.argv[2], **d)
+''' % ROOT
+
+
+def test_no_further_from_fp64_than_stage_by_stage(tmp_path):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    c0 = {"%d_%d" % (nx, seed): inputs.uniform_field((nx, 40, 60), seed=seed, offset=0.1, lo=-0.05, hi=0.05)
+          for nx in (200, 300, 320, 360, 480) for seed in (1, 2)}
+    np.savez(tmp_path / "in.npz", **c0)
+    err = []
+    for generic in ("0", "1"):
+        env = dict(os.environ, EVX_GENERIC=generic)
+        out = str(tmp_path / ("out%s.npz" % generic))
+        r = subprocess.run([sys.executable, "-c", SCRIPT, str(tmp_path / "in.npz"), out], env=env, capture_output=True,
+                           text=True, timeout=300)
+        assert r.returncode == 0, r.stderr[-2000:]
+        err.append(dict(np.load(out)))
+    total = [0.0, 0.0]
+    for key, c in c0.items():
+        ref = O.ch_step(c, 0.1, 1.0, 1.0, 1.0, 20, check_imag=False)
+        for i in (0, 1):
+            total[i] += float(np.linalg.norm(err[i][key] - ref) / np.linalg.norm(ref))
+    assert 0.0 < total[0] <= 1.05 * total[1], total
