@@ -614,8 +614,8 @@ __global__ void __launch_bounds__(ring::threads(EPI), 1)
 //   A (M = 128): four groups of 32 ci, one z row (64 bytes) apart: dz = -1, 0, +1
 //                and a fourth that is not used
 //   B (N = 96):  three groups of 32 co, one dY row slot apart: dy = +1, 0, -1
-//   K = 16 voxels per MMA: 3 dx x 8 = 24 MMAs per row into 3 x 96 columns of
-//   tensor memory, accumulated over every row of the CTA (27 taps at once)
+//   K = 16 voxels per MMA: 3 dx x 8 = 24 MMAs per row into 96 columns of tensor
+//   memory per dx (acc_col), accumulated over the CTA's rows (27 taps at once)
 // An input row costs about what a convolution's does (18 MMAs of N = 96); a unit's
 // rows each count in full (the halo is on the dY rows: 8 of the 38 KB a row
 // loads). The mma.sync kernel it replaces for 32 -> 32 re-read its fragments from
@@ -631,6 +631,11 @@ constexpr int BAR = XOFF + NS * ring::SLOT;  // full[NS], free[NS], done
 constexpr int SMEM = BAR + 8 * (2 * NS + 1) + 16 + 1024;
 constexpr int NTH = 6 * 32;
 constexpr uint32_t COLS = 512;
+// column of dx's accumulator for the CTA's input row k: dx = -1 and 0 have one for even and
+// one for odd rows (5 x 96 of the 512 columns). The tensor core truncates as it adds, so the
+// error grows with the length of a chain: with one accumulator each, dW was up to 1.8%
+// further from 64 bits than the mma.sync kernel's.
+__device__ __forceinline__ uint32_t acc_col(int dx, uint32_t k) { return dx * 96 + (dx < 2 && (k & 1) ? 288 : 0); }
 }  // namespace wg
 
 struct WgArgs {
@@ -768,16 +773,16 @@ __global__ void __launch_bounds__(wg::NTH, 1)
                     for (int ks = 0; ks < ksteps; ++ks)
 #pragma unroll
                         for (int dx = 0; dx < 3; ++dx)
-                            tc_mma_lane0_acc(tmem + dx * 96, a0 + (dx * RUN + ks * 1024) / 16, b0 + ks * 64, I96,
-                                             k > 0 || ks > 0);
-                } else {  // the three slots wrap (never at k = 0): N = 64 + 32 or 32 + 64
+                            tc_mma_lane0_acc(tmem + acc_col(dx, k), a0 + (dx * RUN + ks * 1024) / 16, b0 + ks * 64, I96,
+                                             k > (dx < 2) || ks > 0);
+                } else {  // the three slots wrap (never at k = 0 or 1): N = 64 + 32 or 32 + 64
                     const uint32_t n1 = (NR - s0) * 32, i1 = n1 == 64 ? I64 : I32, i2 = n1 == 64 ? I32 : I64;
                     for (int ks = 0; ks < ksteps; ++ks)
 #pragma unroll
                         for (int dx = 0; dx < 3; ++dx) {
                             const uint64_t ad = a0 + (dx * RUN + ks * 1024) / 16;
-                            tc_mma_lane0_acc(tmem + dx * 96, ad, b0 + ks * 64, i1, 1);
-                            tc_mma_lane0_acc(tmem + dx * 96 + n1, ad, bw + ks * 64, i2, 1);
+                            tc_mma_lane0_acc(tmem + acc_col(dx, k), ad, b0 + ks * 64, i1, 1);
+                            tc_mma_lane0_acc(tmem + acc_col(dx, k) + n1, ad, bw + ks * 64, i2, 1);
                         }
                 }
                 if (lane == 0) tc_commit(freeb + 8 * (k % NS));
@@ -799,12 +804,27 @@ __global__ void __launch_bounds__(wg::NTH, 1)
         fence_after();
         if (w_ok && dzi < 3) {
             float* P = r.partials + (long long)blockIdx.x * 27 * 32 * 32;
+            int rows = 0;  // the odd rows' accumulators hold sums if there is a second row
+            for (int u = blockIdx.x; u < r.nunits && rows < 2; u += gridDim.x) {
+                int bx, z0, ys, ye;
+                wg_unit(r, u, bx, z0, ys, ye);
+                rows += ye - ys;
+            }
 #pragma unroll 1
             for (int g = 0; g < 18; ++g) {  // 16 output channels of one (dx, dy)
                 const int dxi = g / 6, j = (g / 2) % 3, co = (g & 1) * 16;
                 uint32_t acc[16];
-                tmem_ld16(tmem + ((uint32_t)(dzi * 32) << 16) + dxi * 96 + j * 32 + co, acc);
+                const uint32_t at = tmem + ((uint32_t)(dzi * 32) << 16) + j * 32 + co;
+                tmem_ld16(at + acc_col(dxi, 0), acc);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                if (dxi < 2 && rows > 1) {
+                    uint32_t odd[16];
+                    tmem_ld16(at + acc_col(dxi, 1), odd);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                    for (int c = 0; c < 16; ++c)
+                        acc[c] = __float_as_uint(__uint_as_float(acc[c]) + __uint_as_float(odd[c]));
+                }
                 const int t = 9 * dxi + 3 * (2 - j) + dzi;
 #pragma unroll
                 for (int c = 0; c < 16; ++c) P[(t * 32 + co + c) * 32 + lane] = __uint_as_float(acc[c]);
