@@ -793,12 +793,13 @@ __global__ void __launch_bounds__(256) project_direct_kernel(const __nv_bfloat16
 }
 
 // ---------------------------------------------------------------------------
-// Projection of BF16 activations with one warp per RY x 32 outputs of a (b, x) plane
+// Projection with one warp per RY x 32 outputs of a (b, x) plane
 // (rows y0 .. y0 + RY - 1, z0 .. z0 + 31) and lane = channel: every global access
 // of a voxel is one coalesced row of its 32 channels, and each input row segment
 // is read once per warp for all the outputs it feeds (3 dz taps along z, up to
-// 3 dy taps across the RY rows). Needs Z % 32 = 0 and Y % RY = 0. (The FP32 stream's
-// projection walks x: evx_nn_tc.cu.)
+// 3 dy taps across the RY rows). Needs Z % 32 = 0 and Y % RY = 0. For BF16 activations
+// and, on grids where project32_walk (evx_nn_tc.cu) has too few CTAs, for the FP32 stream
+// (the same sums in the same order, so the same bits).
 // lane l ends with the lane sum of v[l] (a butterfly that halves the values per step)
 __device__ __forceinline__ float lane_sum_transpose(float (&v)[32], int lane) {
 #pragma unroll
@@ -827,8 +828,10 @@ __device__ __forceinline__ bool lane_unit(long long u, int X, int Y, int Z, int&
 }
 
 // out(v) = bias(0) + sum_t sum_ci w[t][0][ci] h(v + off_t, ci); lane = ci
-template <int RY, int MINB>
-__global__ void __launch_bounds__(256, MINB) project_lane_kernel(const __nv_bfloat16* __restrict__ h,
+__device__ __forceinline__ float as_float(__nv_bfloat16 v) { return __bfloat162float(v); }
+__device__ __forceinline__ float as_float(float v) { return v; }
+template <typename T, int RY, int MINB>
+__global__ void __launch_bounds__(256, MINB) project_lane_kernel(const T* __restrict__ h,
                                                             const __nv_bfloat16* __restrict__ w, int wcout,
                                                             const float* __restrict__ bias, float* out, int B,
                                                             int X, int Y, int Z) {
@@ -856,11 +859,11 @@ __global__ void __launch_bounds__(256, MINB) project_lane_kernel(const __nv_bflo
             for (int yy = 0; yy < RY + 2; ++yy) {
                 const long long row = (((long long)b * X + xx) * Y + wrapi(y0 + yy - 1, Y)) * Z;
                 float hv[34];
-                const __nv_bfloat16* rp = h + (row + z0) * 32 + lane;
-                hv[0] = __bfloat162float(h[(row + zl) * 32 + lane]);
+                const T* rp = h + (row + z0) * 32 + lane;
+                hv[0] = as_float(h[(row + zl) * 32 + lane]);
 #pragma unroll
-                for (int j = 1; j < 33; ++j) hv[j] = __bfloat162float(rp[(j - 1) * 32]);
-                hv[33] = __bfloat162float(h[(row + zh) * 32 + lane]);
+                for (int j = 1; j < 33; ++j) hv[j] = as_float(rp[(j - 1) * 32]);
+                hv[33] = as_float(h[(row + zh) * 32 + lane]);
 #pragma unroll
                 for (int r = 0; r < RY; ++r) {
                     const int dy = yy - r;  // tap 9 dx + 3 dy + dz  // input row y0 + yy - 1 = output row y0 + r + dy - 1
@@ -1136,7 +1139,7 @@ evx_status evx_nn_conv3d(const void* in, const void* w, const float* bias, void*
     return nn_fail(EVX_ERR_ARG, "supported channel pairs: 16/32 -> 16/32");
 }
 
-// the lane-per-channel projection of BF16 activations: RY = 2 rows x 32 z per warp, two
+// the lane-per-channel projection: RY = 2 rows x 32 z per warp, two
 // 256-thread CTAs per SM (measured at 8 x 256^3: 10.6 ms against 13.2 for one row per warp
 // and 16.1 with one CTA per SM)
 constexpr int LANE_RY = 2;
@@ -1178,7 +1181,7 @@ evx_status evx_nn_project(const void* h, const void* w, int cin, int cout, const
     if (B <= 0 || X <= 0 || Y <= 0 || Z <= 0) return nn_fail(EVX_ERR_SIZE, "empty grid");
     if (cin != 32 || cout < 1) return nn_fail(EVX_ERR_ARG, "project: cin must be 32, cout >= 1");
     if (lane_path(Y, Z))
-        project_lane_kernel<LANE_RY, 2><<<lane_grid(B, X, Y, Z), 256, 0, (cudaStream_t)stream>>>(
+        project_lane_kernel<__nv_bfloat16, LANE_RY, 2><<<lane_grid(B, X, Y, Z), 256, 0, (cudaStream_t)stream>>>(
             (const __nv_bfloat16*)h, (const __nv_bfloat16*)w, cout, bias, out, B, X, Y, Z);
     else
         project_direct_kernel<false><<<8 * nn_sms(), 256, 0, (cudaStream_t)stream>>>(
@@ -1191,9 +1194,18 @@ evx_status evx_nn_project32(const float* h32, const void* w, int cin, int cout, 
     if (!h32 || !w || !out) return nn_fail(EVX_ERR_ARG, "NULL pointer");
     if (B <= 0 || X <= 0 || Y <= 0 || Z <= 0) return nn_fail(EVX_ERR_SIZE, "empty grid");
     if (cin != 32 || cout < 1) return nn_fail(EVX_ERR_ARG, "project: cin must be 32, cout >= 1");
-    if (lane_path(Y, Z) && ((uintptr_t)h32 & 15) == 0)
+    // Either kernel takes as long as its busiest CTA: the walk about 4.1 us per input plane, the
+    // lane kernel 12 us per round of units (measured at 10 to 34 planes and 1 to 14 rounds). 4 x 64^3:
+    // 18 planes 74 us, 7 rounds 84; 64^3: 10 planes 41 us, 2 rounds 25; 32 x 32 x 64: 41 against 11.
+    const int grid = lane_path(Y, Z) ? lane_grid(B, X, Y, Z) : 0;
+    const long long units = (long long)B * X * (Y / LANE_RY) * (Z / 32), resident = 2 * 8 * nn_sms();  // warps
+    if (grid && ((uintptr_t)h32 & 15) == 0 &&
+        project32_planes(B, X, Y, Z, nn_sms()) < 3 * ((units + resident - 1) / resident))
         return nn_cuda(project32_walk(h32, (const __nv_bfloat16*)w, cout, bias, out, B, X, Y, Z, (cudaStream_t)stream,
                                       nn_sms()));
+    else if (grid)
+        project_lane_kernel<float, LANE_RY, 2><<<grid, 256, 0, (cudaStream_t)stream>>>(
+            h32, (const __nv_bfloat16*)w, cout, bias, out, B, X, Y, Z);
     else
         project_direct_kernel<true><<<8 * nn_sms(), 256, 0, (cudaStream_t)stream>>>(
             nullptr, h32, (const __nv_bfloat16*)w, cout, bias, out, B, X, Y, Z);

@@ -53,6 +53,8 @@ cudaError_t conv32_tc(const ConvArgs& a, int epilogue, cudaStream_t st, int sms)
 // projection of the FP32 stream (Z a multiple of 32, Y even, 16-byte aligned h32)
 cudaError_t project32_walk(const float* h32, const __nv_bfloat16* w, int wcout, const float* bias, float* out, int B, int X,
                            int Y, int Z, cudaStream_t st, int sms);
+// input planes that its busiest CTA walks through
+long long project32_planes(int B, int X, int Y, int Z, int sms);
 // weight gradient of a 32 -> 32 convolution: *ctas <= max_ctas partial sums of 27 x 32 x 32
 cudaError_t wgrad32_tc(const __nv_bfloat16* dy, const __nv_bfloat16* x, float* partials, int max_ctas, int B, int X, int Y,
                        int Z, cudaStream_t st, int sms, int* ctas);

@@ -1083,6 +1083,15 @@ cudaError_t conv32_tc(const ConvArgs& a, int epilogue, cudaStream_t st, int sms)
     return cudaErrorInvalidValue;
 }
 
+// (b, y tile, z tile) columns of the walking projection
+static long long project32_columns(int B, int Y, int Z) { return (long long)B * ((Y + pj::ROWS - 1) / pj::ROWS) * (Z / pj::ZT); }
+
+long long project32_planes(int B, int X, int Y, int Z, int sms) {
+    const long long ncol = project32_columns(B, Y, Z);
+    const int nseg = segments(ncol, X, sms, 2);
+    return (ncol * nseg + sms - 1) / sms * ((X + nseg - 1) / nseg + 2);
+}
+
 cudaError_t project32_walk(const float* h32, const __nv_bfloat16* w, int wcout, const float* bias, float* out, int B, int X,
                            int Y, int Z, cudaStream_t st, int sms) {
     PjArgs r{};
@@ -1091,7 +1100,7 @@ cudaError_t project32_walk(const float* h32, const __nv_bfloat16* w, int wcout, 
     r.nyt = (Y + pj::ROWS - 1) / pj::ROWS;
     CUtensorMap m, hm;
     if (!stream_map(&m, h32, B, X, Y, Z, pj::ZT) || !stream_map(&hm, h32, B, X, Y, Z, 1)) return cudaErrorInvalidValue;
-    const long long ncol = (long long)B * r.nyt * (Z / pj::ZT);
+    const long long ncol = project32_columns(B, Y, Z);
     r.nseg = segments(ncol, X, sms, 2);
     if (ncol * r.nseg > (1LL << 30)) return cudaErrorInvalidValue;  // unit index would overflow int
     r.nunits = (int)(ncol * r.nseg);

@@ -1,0 +1,41 @@
+"""Calls that a kernel for large grids must not make slower on small ones, against a kernel of
+the same arithmetic: the FP32-stream projection against the BF16 one (both 864 FMAs per voxel;
+the walking kernel alone took 3.9 times as long here). Best of ten, half as much again allowed."""
+import numpy as np
+import pytest
+
+from oracle import nn as N
+
+pytestmark = pytest.mark.gpu
+
+
+def best_us(call):
+    import torch
+    times = []
+    for _ in range(10):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        for _ in range(20):
+            call()
+        b.record()
+        torch.cuda.synchronize()
+        times.append(a.elapsed_time(b) * 50.0)
+    return min(times)
+
+
+@pytest.mark.parametrize("shape", [(1, 24, 24, 64), (1, 32, 32, 64), (1, 24, 24, 128), (1, 64, 64, 64)])
+def test_project32(shape):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2507_21748_gb300 import surrogate as S
+    rng = np.random.default_rng(3)
+    h32 = torch.from_numpy(rng.standard_normal(shape + (32,)).astype(np.float32)).cuda()
+    h, w = h32.to(torch.bfloat16), torch.from_numpy(rng.standard_normal((27, 16, 32)).astype(np.float32)).to(torch.bfloat16).cuda()
+    out = torch.empty(shape, device="cuda")
+    t16 = best_us(lambda: S._ck(S.lib.evx_nn_project(S._p(h), S._p(w), 32, 16, None, S._p(out), *shape, S._stream())))
+    t32 = best_us(lambda: S._ck(S.lib.evx_nn_project32(S._p(h32), S._p(w), 32, 16, None, S._p(out), *shape, S._stream())))
+    S.check()
+    ref = N.conv(h32.double().cpu().numpy(), w.double().cpu().numpy())[..., 0]
+    assert np.linalg.norm(out.double().cpu().numpy() - ref) < 1e-5 * np.linalg.norm(ref)
+    assert t32 <= 1.5 * t16, (t32, t16)
