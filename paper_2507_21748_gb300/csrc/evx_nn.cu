@@ -935,6 +935,20 @@ __global__ void __launch_bounds__(256, 2) lift_tile_kernel(const float* __restri
         __syncthreads();  // the tile has arrived; the other buffer's has been read (and the weights are staged)
         if (tile + (int)gridDim.x < ntiles) load(tile + gridDim.x, st[cur ^ 1]);
         asm volatile("cp.async.commit_group;" ::: "memory");
+        if (!F32 || scale != 1.f) {  // once per value (in the loop below each of the 32 lanes did it again: 86 us
+                                     // at 4 x 64^3); the padding is changed too and never read
+            float4* v4 = reinterpret_cast<float4*>(st[cur]);
+            for (int i = threadIdx.x; i < 3 * LIFT_PLANE / 4; i += blockDim.x) {
+                float4 v = v4[i];
+                v.x *= scale, v.y *= scale, v.z *= scale, v.w *= scale;
+                if (!F32) {
+                    v.x = __bfloat162float(__float2bfloat16_rn(v.x)), v.y = __bfloat162float(__float2bfloat16_rn(v.y));
+                    v.z = __bfloat162float(__float2bfloat16_rn(v.z)), v.w = __bfloat162float(__float2bfloat16_rn(v.w));
+                }
+                v4[i] = v;
+            }
+            __syncthreads();
+        }
         if (y0 + wy >= Y) continue;  // Y is even: both rows or none
         float acc[2][32];
 #pragma unroll
@@ -952,12 +966,6 @@ __global__ void __launch_bounds__(256, 2) lift_tile_kernel(const float* __restri
                     hv[1 + 4 * q] = v.x, hv[2 + 4 * q] = v.y, hv[3 + 4 * q] = v.z, hv[4 + 4 * q] = v.w;
                 }
                 hv[33] = row[36];
-                if (!F32 || scale != 1.f)
-#pragma unroll
-                    for (int j = 0; j < 34; ++j) {
-                        hv[j] *= scale;
-                        if (!F32) hv[j] = __bfloat162float(__float2bfloat16_rn(hv[j]));
-                    }
 #pragma unroll
                 for (int r = 0; r < 2; ++r) {
                     const int dy = yy - r;  // tap 9 dx + 3 dy + dz

@@ -1,6 +1,9 @@
-"""Calls that a kernel for large grids must not make slower on small ones, against a kernel of
-the same arithmetic: the FP32-stream projection against the BF16 one (both 864 FMAs per voxel;
-the walking kernel alone took 3.9 times as long here). Best of ten, half as much again allowed."""
+"""Calls that must not take longer than a kernel of the same arithmetic, best of ten. The
+FP32-stream projection against the BF16 one (both 864 FMAs per voxel; the walking kernel
+alone took 3.9 times as long here), half as much again allowed. The BF16 lift against the
+FP32-stream one, which stores three times the bytes (1.19 times as long when every lane
+rounded every input). A 32 -> 32 convolution of one short column per CTA against mma.sync
+(1.22 times as long with columns of eight rows). A tenth allowed in these two."""
 import numpy as np
 import pytest
 
@@ -39,3 +42,17 @@ def test_project32(shape):
     ref = N.conv(h32.double().cpu().numpy(), w.double().cpu().numpy())[..., 0]
     assert np.linalg.norm(out.double().cpu().numpy() - ref) < 1e-5 * np.linalg.norm(ref)
     assert t32 <= 1.5 * t16, (t32, t16)
+
+
+def test_lift():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2507_21748_gb300 import surrogate as S
+    shape = (4, 64, 64, 64)
+    f, w = torch.randn(shape, device="cuda"), torch.randn((27, 32, 16), device="cuda").to(torch.bfloat16)
+    h, h32 = torch.empty(shape + (32,), dtype=torch.bfloat16, device="cuda"), torch.empty(shape + (32,), device="cuda")
+    t16 = best_us(lambda: S._ck(S.lib.evx_nn_lift(S._p(f), 1.0, S._p(w), 16, 32, None, S._p(h), *shape, S._stream())))
+    t32 = best_us(lambda: S._ck(S.lib.evx_nn_lift32(S._p(f), 1.0, S._p(w), 16, 32, None, S._p(h), S._p(h32), *shape,
+                                                    S._stream())))
+    assert t16 <= 1.1 * t32, (t16, t32)
