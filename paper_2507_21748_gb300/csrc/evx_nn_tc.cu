@@ -1028,12 +1028,12 @@ bool stream_map(CUtensorMap* m, const float* h32, int B, int X, int Y, int Z, in
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// segments of at least 8 rows that columns are split into: the split with the least
+// segments of at least min_rows rows that columns are split into: the split with the least
 // work on the busiest CTA, a segment of n rows costing n + extra
-int segments(long long ncol, int len, int ctas, int extra) {
+int segments(long long ncol, int len, int ctas, int extra, int min_rows = 8) {
     int nseg = 1;
     long long best = 0;
-    for (int s = 1; s == 1 || s <= len / 8; ++s) {
+    for (int s = 1; s == 1 || s <= len / min_rows; ++s) {
         const long long rows = (ncol * s + ctas - 1) / ctas * ((len + s - 1) / s + extra);
         if (s == 1 || rows < best) {
             best = rows;
@@ -1053,7 +1053,7 @@ cudaError_t launch_walk(const ConvArgs& a, cudaStream_t st, int sms) {
         return cudaErrorInvalidValue;
     r.len = WX ? a.X : a.Y;
     const long long ncol = (long long)a.B * (WX ? a.Y : a.X) * r.nzc;
-    const int nseg = segments(ncol, r.len, sms, 2);
+    const int nseg = segments(ncol, r.len, sms, 2, 2);
     if (ncol * nseg > (1LL << 30)) return cudaErrorInvalidValue;  // unit index would overflow int
     r.nseg = nseg;
     r.nunits = (int)(ncol * nseg);

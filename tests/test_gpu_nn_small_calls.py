@@ -56,3 +56,24 @@ def test_lift():
     t32 = best_us(lambda: S._ck(S.lib.evx_nn_lift32(S._p(f), 1.0, S._p(w), 16, 32, None, S._p(h), S._p(h32), *shape,
                                                     S._stream())))
     assert t16 <= 1.1 * t32, (t16, t32)
+
+
+@pytest.mark.parametrize("epi", ["PLAIN", "GELU"])
+def test_conv_short_columns(epi):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2507_21748_gb300 import surrogate as S
+    shape = (1, 8, 8, 64)
+    x, pre, out = (torch.randn(shape + (32,), device="cuda").to(torch.bfloat16) for _ in range(3))
+    w = torch.randn((27, 32, 32), device="cuda").to(torch.bfloat16)
+    before, t = S.lib.evx_nn_conv_engine(), {}
+    for engine in (S.ENGINE_TCGEN05, S.ENGINE_MMA_SYNC):
+        S._ck(S.lib.evx_nn_set_conv_engine(engine))
+        try:
+            t[engine] = best_us(lambda: S._ck(S.lib.evx_nn_conv3d(
+                S._p(x), S._p(w), None, S._p(out), S._p(pre), None, *shape, 32, 32, getattr(S, "EPI_" + epi), S._stream())))
+        finally:
+            S._ck(S.lib.evx_nn_set_conv_engine(before))
+    S.check()
+    assert t[S.ENGINE_TCGEN05] <= 1.1 * t[S.ENGINE_MMA_SYNC], t
