@@ -284,15 +284,15 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
 }
 
 // bounded wait that also gives up once another role has aborted; a phase that has
-// already completed is seen by the non-blocking probe first
-__device__ __forceinline__ bool ring_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+// already completed is seen by the non-blocking probe first. mark: the flag's value
+__device__ __forceinline__ bool ring_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int mark = 1) {
     if (mbar_test(bar, parity)) return true;
     const long long t0 = clock64();
     while (true) {
         if (mbar_try(bar, parity)) return true;
         if (*abort_flag) return false;
         if (clock64() - t0 > ring::WAIT_BUDGET) {
-            *abort_flag = 1;
+            *abort_flag = mark;
             atomicExch(&g_tc_timeout, 1);
             return false;
         }
@@ -898,8 +898,8 @@ __global__ void __launch_bounds__(pj::NT, 1)
     const float b0 = r.bias ? r.bias[0] : 0.f;
     __syncthreads();
     uint32_t k = 0;  // planes consumed
-    bool failed = false;  // the same in every thread
-    for (int u = blockIdx.x; u < r.nunits && !failed; u += gridDim.x) {
+    bool go = true;
+    for (int u = blockIdx.x; u < r.nunits && go; u += gridDim.x) {
         const int seg = u % r.nseg;
         int c = u / r.nseg;
         const int z0 = (c % (Z / ZT)) * ZT;
@@ -929,7 +929,7 @@ __global__ void __launch_bounds__(pj::NT, 1)
 #pragma unroll
             for (int j = 0; j < 32; ++j) acc[d][0][j] = acc[d][1][j] = 0.f;
         for (int q = 0; q < np; ++q, ++k) {
-            const bool arrived = ring_wait(full + 8 * (k & 1), (k >> 1) & 1, abort_flag);
+            (void)ring_wait(full + 8 * (k & 1), (k >> 1) & 1, abort_flag, (int)k + 1);  // seen in the flag below
             const float* pl = reinterpret_cast<const float*>(smem_raw + (k & 1) * PLANE) + (2 * warp) * PROW + lane;
 #pragma unroll
             for (int yy = 0; yy < 4; ++yy) {
@@ -950,15 +950,13 @@ __global__ void __launch_bounds__(pj::NT, 1)
                         }
                 }
             }
-            // the plane has been read; a wait that ran out in any thread ends the CTA: nothing is
-            // stored or loaded after it, and the copies in flight land first (bounded)
-            if ((failed = __syncthreads_or(!arrived))) {
-                if (threadIdx.x == 0)
-                    for (int m = 0; m < 2 && q + m < np; ++m) tc_wait(full + 8 * ((k + m) & 1), ((k + m) >> 1) & 1);
-                break;
-            }
-            if (q + 2 < np) load(q + 2, k + 2);
-            if (q >= 2) {
+            __syncthreads();  // the plane has been read
+            // a wait that ran out in any thread: nothing is loaded or stored from here on. Every thread
+            // finds the same: a plane's mark is set before its barrier or not at all
+            const uint32_t mark = *abort_flag;
+            go = mark == 0 || mark > k + 1;
+            if (go && q + 2 < np) load(q + 2, k + 2);
+            if (go && q >= 2) {
                 const int x = xs + q - 2, y = y0 + 2 * warp;
 #pragma unroll
                 for (int o = 0; o < 2; ++o) {
@@ -976,6 +974,8 @@ __global__ void __launch_bounds__(pj::NT, 1)
                 }
         }
     }
+    if (!go && threadIdx.x == 0)  // the copies in flight, of the late plane and the next of its unit, land first (bounded)
+        for (uint32_t m = (uint32_t)*abort_flag - 1, end = min(m + 2, k); m < end; ++m) tc_wait(full + 8 * (m & 1), (m >> 1) & 1);
 }
 
 }  // namespace evxnn

@@ -41,11 +41,27 @@ def test_every_late_plane_is_drained(units):
 
 
 def test_no_bounded_wait_is_ignored():
-    """A bounded pipeline wait that is a statement of its own drops its result; after a failed
-    one the projection drains before it could load or store again."""
+    """The result of a bounded pipeline wait is used, or its mark is: the projection reads the
+    flag after the plane's barrier, guards the loads and stores after it, and drains at its end."""
     with open(os.path.join(CSRC, "evx_nn_tc.cu")) as f:
         text = f.read()
-    assert not re.findall(r"(?m)^\s*(?:ring_wait|ring_wait_long)\(.*\);", text)
-    body = text[text.index("project_walk_kernel(const"):text.index("// =", text.index("project_walk_kernel(const"))]
-    stop = body.index("__syncthreads_or(!arrived)")
-    assert stop < body.index("tc_wait(") < body.index("load(q + 2") < body.index("r.out[")
+    dropped = re.findall(r"(?m)^\s*(?:\(void\))?ring_wait(?:_long)?\((.*)\);", text)
+    assert all(args.endswith("(int)k + 1") for args in dropped), dropped
+    i = text.index("project_walk_kernel(const")
+    body = text[i:text.index("// =", i)]
+    order = ["(int)k + 1", "__syncthreads();  // the plane", "mark = *abort_flag", "if (go && q + 2 < np) load(", "if (go && q >= 2)",
+             "r.out[", "if (!go && threadIdx.x == 0)", "tc_wait("]
+    at = [body.index(o) for o in order]
+    assert at == sorted(at) and body.count("r.out[") == 1 and "nunits && go;" in body
+
+
+def test_every_thread_takes_the_same_way():
+    """A thread reads the flag some time after plane k's barrier; by then threads ahead of it may
+    have marked plane k + 1 (not k + 2: they wait for it at the barrier between)."""
+    for k in range(6):
+        for first in [None] + list(range(8)):  # plane whose wait ran out first
+            seen = set()
+            for ahead in (0, 1):
+                flag = first + 1 if first is not None and first <= k + ahead else 0
+                seen.add(flag == 0 or flag > k + 1)
+            assert seen == {first is None or first > k}
