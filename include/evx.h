@@ -32,11 +32,13 @@
  *     entry point says it synchronises.
  *   - Sizes: nx, ny, nz each even, 8 <= n <= 1024, with no prime factor other
  *     than 2, 3 and 5; otherwise EVX_ERR_SIZE. Every such size runs the same
- *     arithmetic. Each pass picks its kernel by its own length: nx, ny in
- *     {64, ..., 1024 powers of two, 400} and nz in {128, ..., 1024 powers of
- *     two, 400} take the tuned four-step kernels, other lengths the two-radix
- *     kernels, and nx, ny = 972 and 1000 the mixed-radix ones (same results to
- *     FP32 rounding, several times slower).
+ *     scheme; kernels differ by FP32 rounding. Each pass picks its kernel by its
+ *     own length and by the grid's voxel count: nx, ny in {64, ..., 1024 powers
+ *     of two, 400} and nz in {128, ..., 1024 powers of two, 400} take the tuned
+ *     four-step kernels; on grids of up to 2^22 voxels, nx, ny up to 128 and nz
+ *     up to 256 the grouped-stage kernels; the rest the two-radix kernels, but
+ *     nx, ny = 972 and 1000 the mixed-radix ones (several times slower). So one
+ *     length may round differently on a small and on a large grid.
  */
 #ifndef EVX_H
 #define EVX_H

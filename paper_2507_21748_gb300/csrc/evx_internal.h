@@ -254,7 +254,7 @@ cudaError_t launch_zpass(const ZPassArgs& a, int mode, cudaStream_t st, int* gri
 //   rhs = (1 / h^2) sum over the 6 neighbours j of (M_i + M_j)/2 (mu_j - mu_i), M = M0 max(1 - c^2, 0)
 //   partials[b] = sum over the CTA's voxels of (c^2 - 1)^2 / 4 + (kappa / 2h^2) sum_d (c_{i+e_d} - c_i)^2
 cudaError_t launch_vm_mu(const float* c, float* mu, int nx, int ny, int nz, float kappa_h2, cudaStream_t st);
-// both stencils in one pass (ny a multiple of 8, nz of 64; vm_fd_fused_ok): rhs from c, mu not stored
+// both stencils in one pass (nz a multiple of 4, nx >= 8; vm_fd_fused_ok): rhs from c, mu not stored
 bool vm_fd_fused_ok(int nx, int ny, int nz);
 cudaError_t launch_vm_fd(const float* c, float* rhs, int nx, int ny, int nz, float kappa_h2, float M0, float inv_h2,
                          cudaStream_t st);
@@ -288,13 +288,16 @@ bool fast_zstep(const ZPassArgs& a, cudaStream_t st, cudaError_t* err, int* grid
 bool fast_xadj(const XAdjArgs& a, cudaStream_t st, cudaError_t* err);
 bool fast_zconv(const ZPassArgs& a, int dir, cudaStream_t st, cudaError_t* err, int* grid_used);
 bool fast_paths_enabled();  // false when the environment sets EVX_GENERIC=1
-// grids whose mixed-radix passes run with grouped stages (evx_staged.cu), bit for bit
+// Largest grid whose mixed-radix passes run with grouped stages (evx_staged.cu), bit for bit
+// as stage by stage. Not the line where the two-radix kernels become faster: they are faster
+// at every size (table in evx_staged.cu). Small grids are the ones that data sets of solver
+// runs are made on; 4 M voxels holds them with a margin.
 constexpr long long STAGED_MAX_VOXELS = 1LL << 22;
 bool staged_spass(const SPassArgs& a, int dir, cudaStream_t st, cudaError_t* err);
 bool staged_xupdate(const XUpdArgs& a, cudaStream_t st, cudaError_t* err);
 bool staged_zpass(const ZPassArgs& a, int mode, cudaStream_t st, cudaError_t* err, int* grid_used);
 int staged_zgrid(const ZPassArgs& a);
-// two-radix passes for lengths R1 R2, R1, R2 <= 32 (evx_mixed.cu); false if not applicable
+// two-radix passes for lengths R1 R2, R1, R2 <= 32 (evx_mixed_{x,y,z}.cu); false if not applicable
 bool mixed_split(int L, int* R1, int* R2);
 bool mixed_spass(const SPassArgs& a, int dir, cudaStream_t st, cudaError_t* err);
 bool mixed_xupdate(const XUpdArgs& a, cudaStream_t st, cudaError_t* err);

@@ -1202,9 +1202,9 @@ evx_status evx_nn_project32(const float* h32, const void* w, int cin, int cout, 
     if (!h32 || !w || !out) return nn_fail(EVX_ERR_ARG, "NULL pointer");
     if (B <= 0 || X <= 0 || Y <= 0 || Z <= 0) return nn_fail(EVX_ERR_SIZE, "empty grid");
     if (cin != 32 || cout < 1) return nn_fail(EVX_ERR_ARG, "project: cin must be 32, cout >= 1");
-    // Either kernel takes as long as its busiest CTA: the walk about 4.1 us per input plane, the
+    // Either kernel takes as long as its busiest CTA: the walk about 3.9 us per input plane, the
     // lane kernel 12 us per round of units (measured at 10 to 34 planes and 1 to 14 rounds). 4 x 64^3:
-    // 18 planes 74 us, 7 rounds 84; 64^3: 10 planes 41 us, 2 rounds 25; 32 x 32 x 64: 41 against 11.
+    // 18 planes 70 us, 7 rounds 84; 64^3: 10 planes 39 us, 2 rounds 24; 32 x 32 x 64: 39 against 11.
     const int grid = lane_path(Y, Z) ? lane_grid(B, X, Y, Z) : 0;
     const long long units = (long long)B * X * (Y / LANE_RY) * (Z / 32), resident = 2 * 8 * nn_sms();  // warps
     if (grid && ((uintptr_t)h32 & 15) == 0 &&

@@ -11,12 +11,20 @@
 // with the twiddles exp(-2 pi i t kk / (Ns r)) of the whole transform.
 //
 // Why beside the two-radix kernels (evx_mixed.cuh), which need one exchange less
-// per inverse: these give the fields of the stage-by-stage kernels to the bit, so
-// data sets made with them (the surrogate trains on BF16 activations, where a
-// last-bit change of an input moves gradients by 1e-4) are reproduced, and grids
-// of up to STAGED_MAX_VOXELS are bound by launches and latency, where the extra
-// exchange costs little. Measured on a GB300 (48 x 40 x 36, ncu, cold caches): stage by stage y 10.9,
-// z 56, x 26 us; grouped y 4.7, z 13.3, x 23.4 us; two-radix y 3.6, z 8.0, x 8.3 us.
+// per inverse and are faster: these give the fields of the stage-by-stage kernels
+// to the bit, so data sets made with them (the surrogate trains on BF16
+// activations, where a last-bit change of an input moves gradients by 1e-4) are
+// reproduced. That is the only reason; it holds for the fields, not for the
+// energies, and only up to STAGED_MAX_VOXELS. Measured on a GB300, microseconds per
+// Cahn-Hilliard step (64 steps in a graph):
+//   grid            stage by stage   grouped   two radices
+//   24^3                  50.2         17.2        10.9
+//   48 x 40 x 36          62.1         21.9        11.9
+//   96^3                 158.8         78.7        17.4
+//   120 x 108 x 100      174.9         60.0        22.4
+//   300 x 120 x 108      382.2         69.0        49.1
+// Per kernel at 48 x 40 x 36 (ncu, cold caches): stage by stage y 10.9, z 56, x 26
+// us; grouped 4.7, 13.3, 23.4; two-radix 3.6, 8.0, 8.3.
 #include <algorithm>
 #include <cstdint>
 
