@@ -398,7 +398,8 @@ __host__ __device__ constexpr int crt_index(int k1, int N1, int k2, int N2) {
         if (k % N1 == k1 && k % N2 == k2) return k;
     return 0;
 }
-template <int N1, int N2, int DIR>
+// F: the family its factors are taken from
+template <int N1, int N2, int DIR, template <int, int> class F = Dft>
 struct DftCoprime {
     template <int K1, int K2>
     __device__ __forceinline__ static void put(float2* v, const float2 (&t)[N1][N2]) {
@@ -416,14 +417,14 @@ struct DftCoprime {
         for (int n1 = 0; n1 < N1; ++n1) {
 #pragma unroll
             for (int n2 = 0; n2 < N2; ++n2) t[n1][n2] = v[(N2 * n1 + N1 * n2) % N];
-            Dft<N2, DIR>::run(t[n1]);
+            F<N2, DIR>::run(t[n1]);
         }
 #pragma unroll
         for (int k2 = 0; k2 < N2; ++k2) {
             float2 u[N1];
 #pragma unroll
             for (int n1 = 0; n1 < N1; ++n1) u[n1] = t[n1][k2];
-            Dft<N1, DIR>::run(u);
+            F<N1, DIR>::run(u);
 #pragma unroll
             for (int k1 = 0; k1 < N1; ++k1) t[k1][k2] = u[k1];
         }
@@ -431,7 +432,7 @@ struct DftCoprime {
     }
 };
 // length N1 N2, decimation in time: n = N2 n1 + n2, k = k1 + N1 k2
-template <int N1, int N2, int DIR>
+template <int N1, int N2, int DIR, template <int, int> class F = Dft>
 struct DftTwiddled {
     template <int n2, int k1>
     __device__ __forceinline__ static void twiddle(float2 (&t)[N2][N1]) {
@@ -447,7 +448,7 @@ struct DftTwiddled {
         for (int n2 = 0; n2 < N2; ++n2) {
 #pragma unroll
             for (int n1 = 0; n1 < N1; ++n1) t[n2][n1] = v[N2 * n1 + n2];
-            Dft<N1, DIR>::run(t[n2]);
+            F<N1, DIR>::run(t[n2]);
         }
         twiddle<1, 1>(t);
 #pragma unroll
@@ -455,7 +456,7 @@ struct DftTwiddled {
             float2 u[N2];
 #pragma unroll
             for (int n2 = 0; n2 < N2; ++n2) u[n2] = t[n2][k1];
-            Dft<N2, DIR>::run(u);
+            F<N2, DIR>::run(u);
 #pragma unroll
             for (int k2 = 0; k2 < N2; ++k2) v[k1 + N1 * k2] = u[k2];
         }

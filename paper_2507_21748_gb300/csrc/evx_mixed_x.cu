@@ -49,7 +49,7 @@ struct ColUpdate {
         float2 g[R];
 #pragma unroll
         for (int i = 0; i < R; ++i) g[i] = w[i * CP];
-        MxDft<R, -1>::run(g);
+        XDft<R, -1>::run(g);
         float2 v[R];
         if (MODE == 2) {  // preconditioner: dt / (1 + dt M kappa |k|^4) F_x W / L (dtM holds dt)
 #pragma unroll
@@ -64,7 +64,7 @@ struct ColUpdate {
             }
 #pragma unroll
             for (int i = 0; i < R; ++i) v[i] = s[i * CP];
-            MxDft<R, -1>::run(v);
+            XDft<R, -1>::run(v);
 #pragma unroll
             for (int k = 0; k < R; ++k) {
                 const float2 gk = SPILL ? w[k * CP] : g[k];
@@ -83,7 +83,7 @@ struct ColUpdate {
             }
         }
         if (zero) v[0] = make_float2(0.f, 0.f);  // the mean is carried in FP64
-        MxDft<R, 1>::run(v);
+        XDft<R, 1>::run(v);
         s[0] = v[0];
 #pragma unroll
         for (int i = 1; i < R; ++i) s[i * CP] = twmul<1>(v[i], __ldg(a.tw + i * k1));
@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(8 * M1, M1 <= 16 ? 5 : M1 <= 20 ? 4 : 2) mx_x_
         for (int i = it; i < (MODE == 2 ? R2 : 2 * R2); i += T) {
             const bool second = i >= R2;
             const int n2 = second ? i - R2 : i;
-            with_radix<M1>(R1, ColLoad<-1>{(second ? a.S : a.W) + base + n2 * a.rs, R2 * a.rs,
+            with_radix<M1>(R1, ColLoad<-1, XDft>{(second ? a.S : a.W) + base + n2 * a.rs, R2 * a.rs,
                                              (second ? xs : xw) + n2 * CP + p, pitch, a.tw, n2,
                                              {second ? a.S : a.W, nbuf}});
         }
